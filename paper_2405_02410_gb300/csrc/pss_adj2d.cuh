@@ -173,8 +173,7 @@ __global__ void __launch_bounds__(Adj2Shape<N, E>::THREADS) k2_col_adj(const Col
             C xin[2] = {mk<float>(0.f, 0.f), mk<float>(0.f, 0.f)};
             if (fp.noisy)
                 noise_pair<float>(kx0 == 0 || 2 * kx0 == sp.nx, kx0, ky, 0,
-                                  noise_amp<float>(fp.sigma0, fp.noise_pow, q2c[0]),
-                                  noise_amp<float>(fp.sigma0, fp.noise_pow, q2c[1]), v1, sp, (uint32_t)fp.field_id,
+                                  fp.sigma0, fp.noise_pow, q2c[0], q2c[1], v1, sp, (uint32_t)fp.field_id,
                                   key, step, xin[0], xin[1]);
 #pragma unroll
             for (int c = 0; c < 2; ++c) {

@@ -105,15 +105,17 @@ __device__ __forceinline__ double fast_sqrt(double x) { return sqrt(x); }
 __device__ __forceinline__ float fast_rcp(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ double fast_rcp(double x) { return 1.0 / x; }
 
-// Box-Muller pair.  FP32 uses the hardware log2 / sin / cos approximations
-// (absolute error ~1e-6 on these arguments); FP64 uses the libdevice calls.
-__device__ __forceinline__ void box_muller(float u0, float u1, float &n1, float &n2) {
-    const float r = fast_sqrt(-2.0f * __logf(u0));
-    float s, c;
-    __sincosf(6.283185307179586f * u1, &s, &c);
-    n1 = r * c;
-    n2 = r * s;
+// sqrt as x rsqrt(x) by the hardware approximation (about 2 ulp; 0 stays 0,
+// subnormals count as 0), without a branch or a select
+__device__ __forceinline__ float root_approx(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fmaxf(x, 1.17549435e-38f)));
+    return fmul(x, r);
 }
+
+// Box-Muller pair in FP64 (the library calls).  FP32 draws its normals in
+// noise_mode, with the hardware log2 / sqrt / sin / cos approximations
+// (absolute error ~1e-6 on these arguments).
 __device__ __forceinline__ void box_muller(double u0, double u1, double &n1, double &n2) {
     const double r = sqrt(-2.0 * log(u0));
     double s, c;

@@ -616,8 +616,7 @@ __device__ __forceinline__ void noise_range(const SysP<float> &sp, const FieldP<
                 const float qy = fmul(float(signed_k(pos, sp.ny)), sp.gy);
                 const float qx0 = fmul(float(kx0), sp.gx), qx1 = fmul(float(kx0 + 1), sp.gx);
                 const float q2a = q2sum(qx0, qy), q2b = q2sum(qx1, qy);
-                noise_pair<float>(kx0 == 0 || 2 * kx0 == sp.nx, kx0, pos, 0, noise_amp<float>(1.f, fp.noise_pow, q2a),
-                                  noise_amp<float>(1.f, fp.noise_pow, q2b), kx0 + 1 < sp.hx, sp, (uint32_t)fp.field_id,
+                noise_pair<float>(kx0 == 0 || 2 * kx0 == sp.nx, kx0, pos, 0, 1.f, fp.noise_pow, q2a, q2b, kx0 + 1 < sp.hx, sp, (uint32_t)fp.field_id,
                                   key, step, xa[u], xb[u]);
             }
         }

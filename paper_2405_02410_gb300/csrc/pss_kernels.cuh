@@ -39,18 +39,52 @@ template <typename T> __device__ __forceinline__ T poly5(const T *c, T x) {
 
 __device__ __forceinline__ int signed_k(int k, int n) { return k < (n + 1) / 2 ? k : k - n; }
 
+// sigma0 |q|^p with |q| = sqrt(q2)
+template <typename T> __device__ __forceinline__ T noise_amp(T sigma0, int p, T q2) {
+    if (p == 0) return sigma0;
+    const T qa = fast_sqrt(q2);
+    T amp = sigma0;
+    for (int i = 0; i < p; ++i) amp *= qa;
+    return amp;
+}
+
+// A pair of independent normals of standard deviation sigma0 |q|^p (Box-Muller
+// of two generator words).  FP32: drawing noise is a large part of every
+// step's instructions (issue-bound kernels), so the odd power of |q| goes
+// under Box-Muller's own root, sqrt(-2 ln u0 q^2) |q|^(p-1), which leaves one
+// root per mode, and the uniforms take one fused multiply-add (the same bits
+// as uniform24).  Written with rounding intrinsics: the persistent and the
+// per-step kernels draw the same bits.
+__device__ __forceinline__ float2 noise_mode(uint32_t w0, uint32_t w1, float sigma0, int p, float q2) {
+    const float u0 = ffma(float(w0 >> 8), 5.9604644775390625e-08f, 2.98023223876953125e-08f);
+    const float u1 = ffma(float(w1 >> 8), 5.9604644775390625e-08f, 2.98023223876953125e-08f);
+    const float L = fmul(fmul(-2.0f, __logf(u0)), (p & 1) ? q2 : 1.0f);
+    float amp = sigma0;
+    if (p >= 2) amp = fmul(amp, p >= 4 ? fmul(q2, q2) : q2);   // p is 0 .. 4
+    const float r = fmul(root_approx(L), amp);
+    float s, c;
+    __sincosf(fmul(6.283185307179586f, u1), &s, &c);
+    return mk<float>(fmul(r, c), fmul(r, s));
+}
+__device__ __forceinline__ double2 noise_mode(uint32_t w0, uint32_t w1, double sigma0, int p, double q2) {
+    double n1, n2;
+    box_muller(uniform24<double>(w0), uniform24<double>(w1), n1, n2);
+    const double amp = noise_amp<double>(sigma0, p, q2);
+    return mk<double>(amp * n1, amp * n2);
+}
+
 // Noise increments xi_q of two neighbouring modes kx0 = 2j, kx1 = 2j + 1 of
 // one row (ky, kz) of the half spectrum (Eq. noise_eq over one step).  Each
 // Hermitian pair of modes is drawn once, by its canonical member (the smaller
 // index in the half spectrum [kz][ky][kx]); one Philox4x32-10 call, counter
 // (((kz Ny + ky) Hxe + kx) / 2, step, field, 0), serves the canonical modes
 // 2j and 2j + 1 of a row: words (x0, x1) the even one, (x2, x3) the odd one.
-// A mode that is its own partner is real.  amp0/amp1 are the per-component
-// standard deviations sqrt(N_sites D~(q) dt / dV) of the two modes.
-// on_plane: kx0 is 0 or Nx/2 (its partner is (kx0, -ky, -kz)).
+// A mode that is its own partner is real.  The per-component standard
+// deviations are sigma0 |q|^npow = sqrt(N_sites D~(q) dt / dV); q2a, q2b are
+// the two modes' q^2.  on_plane: kx0 is 0 or Nx/2 (its partner is (kx0, -ky, -kz)).
 template <typename T>
-__device__ __forceinline__ void noise_pair(bool on_plane, int kx0, int ky, int kz, T amp0, T amp1, bool has1,
-                                           const SysP<T> &sp, uint32_t fid, const PhiloxKey &key,
+__device__ __forceinline__ void noise_pair(bool on_plane, int kx0, int ky, int kz, T sigma0, int npow, T q2a, T q2b,
+                                           bool has1, const SysP<T> &sp, uint32_t fid, const PhiloxKey &key,
                                            uint32_t step, cplx<T> &xi0, cplx<T> &xi1) {
     const uint32_t row = (uint32_t)(kz * sp.ny + ky);
     uint32_t crow = row;
@@ -61,15 +95,16 @@ __device__ __forceinline__ void noise_pair(bool on_plane, int kx0, int ky, int k
         if (prow < row) { crow = prow; cj = true; }
     }
     u32x4 r = philox4x32_10(u32x4{(crow * (uint32_t)sp.hxe + (uint32_t)kx0) >> 1, step, fid, 0u}, key);
-    T n1, n2;
-    box_muller(uniform24<T>(r.x), uniform24<T>(r.y), n1, n2);
-    xi0 = selfc ? mk<T>(T(1.4142135623730951) * amp0 * n1, T(0)) : mk<T>(amp0 * n1, cj ? -amp0 * n2 : amp0 * n2);
+    xi0 = noise_mode(r.x, r.y, sigma0, npow, q2a);
+    if (on_plane) {
+        if (cj) xi0.y = -xi0.y;
+        if (selfc) xi0 = mk<T>(T(1.4142135623730951) * xi0.x, T(0));
+    }
     if (has1) {
         // kx1 is odd, so it is never 0 or Nx/2: it is its own canonical member
         if (crow != row)
             r = philox4x32_10(u32x4{(row * (uint32_t)sp.hxe + (uint32_t)kx0) >> 1, step, fid, 0u}, key);
-        box_muller(uniform24<T>(r.z), uniform24<T>(r.w), n1, n2);
-        xi1 = mk<T>(amp1 * n1, amp1 * n2);
+        xi1 = noise_mode(r.z, r.w, sigma0, npow, q2b);
     }
 }
 
@@ -92,15 +127,6 @@ template <typename T> __device__ __forceinline__ void st_pair(cplx<T> *p, cplx<T
         p[0] = a;
         p[1] = b;
     }
-}
-
-// sigma0 |q|^p with |q| = sqrt(q2)
-template <typename T> __device__ __forceinline__ T noise_amp(T sigma0, int p, T q2) {
-    if (p == 0) return sigma0;
-    const T qa = fast_sqrt(q2);
-    T amp = sigma0;
-    for (int i = 0; i < p; ++i) amp *= qa;
-    return amp;
 }
 
 // Eq. (timeupdate) with the mode's factors given: g (phi + xi + m P), where
@@ -250,8 +276,8 @@ __device__ __forceinline__ void col_adjoint(const ColArgs<T> &a, const FieldP<T>
             if (fp.noisy && tile < a.n_tiles && kx0 < sp.hx && chunk_writes(chq)) {
                 const T qe = T(kx0) * sp.gx, qo = T(kx0 + 1) * sp.gx;
                 const T q2e = qe * qe + qy * qy + qz * qz, q2o = qo * qo + qy * qy + qz * qz;
-                noise_pair<T>(kx0 == 0 || 2 * kx0 == sp.nx, kx0, ky, kz, noise_amp<T>(fp.sigma0, fp.noise_pow, q2e),
-                              noise_amp<T>(fp.sigma0, fp.noise_pow, q2o), kx0 + 1 < sp.hx, sp, (uint32_t)fp.field_id,
+                noise_pair<T>(kx0 == 0 || 2 * kx0 == sp.nx, kx0, ky, kz, fp.sigma0, fp.noise_pow, q2e, q2o,
+                              kx0 + 1 < sp.hx, sp, (uint32_t)fp.field_id,
                               key, step, xin[0], xin[1]);
             }
 #pragma unroll
@@ -507,8 +533,7 @@ __global__ void __launch_bounds__(512, (N >= 512 || ADJ) ? 1 : 2) k_col(const Co
                     const T q2a = qx0s + qyz2, q2b = qx1s + qyz2;
                     C xi0 = mk<T>(0, 0), xi1 = mk<T>(0, 0);
                     if (noisy)
-                        noise_pair<T>(on_plane, kx0, ky, kz, noise_amp<T>(sigma0, noise_pow, q2a),
-                                      noise_amp<T>(sigma0, noise_pow, q2b), has1, sp, (uint32_t)fid, key,
+                        noise_pair<T>(on_plane, kx0, ky, kz, sigma0, noise_pow, q2a, q2b, has1, sp, (uint32_t)fid, key,
                                       step, xi0, xi1);
                     v0 = update_mode<T>(f0, v0, xi0, q2a, dtO, dtM, has_product);
                     v1 = update_mode<T>(f1, v1, xi1, q2b, dtO, dtM, has_product);

@@ -246,8 +246,7 @@ __global__ void __launch_bounds__(P2Shape<N, E, NNW>::THREADS, 1) k2p_step(const
                     const float qy = fmul(float(signed_k(ky, N)), sp.gy);
                     const float qx0 = fmul(float(kx0), sp.gx), qx1 = fmul(float(kx0 + 1), sp.gx);
                     const float q2a = q2sum(qx0, qy), q2b = q2sum(qx1, qy);
-                    noise_pair<float>(kx0 == 0 || 2 * kx0 == sp.nx, kx0, ky, 0, noise_amp<float>(1.f, fp.noise_pow, q2a),
-                                      noise_amp<float>(1.f, fp.noise_pow, q2b), kx0 + 1 < sp.hx, sp,
+                    noise_pair<float>(kx0 == 0 || 2 * kx0 == sp.nx, kx0, ky, 0, 1.f, fp.noise_pow, q2a, q2b, kx0 + 1 < sp.hx, sp,
                                       (uint32_t)fp.field_id, key, step, xa, xb);
                     nz[(2 * uu) * N + ky] = xa;
                     nz[(2 * uu + 1) * N + ky] = xb;
