@@ -251,6 +251,15 @@ int pss_time_kernels(pss_system *s, int64_t n, double *avg_ms);
  *                 and row phases (1, default) or as two launches a step on
  *                 the "fast2d" kernels (0); the same bits at the same FFT
  *                 radix;
+ *   "resident"    FP32 2D systems with sides of 32..512 and power products, at
+ *                 least one side below 256 (or 256 x 256 batches that fill the
+ *                 GPU), take a run of steps as one launch in which a cluster
+ *                 of CTAs holds each slot on chip (1, default) or the kernels
+ *                 pss_step_path names (0); they agree to FP32 rounding, and
+ *                 the other launch-shape keys do not act on such a run;
+ *                 "fast2d" 0 also turns it off;
+ *   "res_ctas"    CTAs per cluster of that launch (a power of two <= 16; 0:
+ *                 automatic); the same bits whatever their number;
  *   "persist_blocks" CTAs of that launch (0: automatic, one per SM and at
  *                 most one per column pair or row pair; values below the
  *                 smallest count that keeps every column and row pair in
@@ -389,8 +398,12 @@ int64_t pss_launch_count(const pss_system *s);
  * FP32 2D systems with sides of 256, 512 or 1024 points, unless the tuning
  * key "fast2d" is 0); 2 = the generic 3D kernels with the x pass on FFT
  * groups (k_col, k_mid, k2_row: FP32 3D systems whose x side is 256, 512 or
- * 1024 points, unless "fast3d" is 0); 0 = the generic kernels (k_col,
- * k_mid, k_row).  Returns PSS_EINVAL for a NULL handle. */
+ * 1024 points, unless "fast3d" is 0); 3 = the persistent 2D step (k2p_step:
+ * tuning key "persist"); 0 = the generic kernels (k_col, k_mid, k_row).  Runs
+ * of pss_step and pss_step_many on the cluster-resident path (tuning key
+ * "resident") replace the kernels of paths 0 and 1 by one launch; their path
+ * is still named here, since the calls other than stepping use it.  Returns
+ * PSS_EINVAL for a NULL handle. */
 int pss_step_path(const pss_system *s);
 
 #ifdef __cplusplus

@@ -136,6 +136,11 @@ struct pss_system {
     int tune_adj_col2 = 1;
     int tune_adj_radix = 0;                  // FFT radix of that backward pass (8 or 16; 0: the forward's)
     int tune_persist_adj = 1;                // FP32 2D adjoint on the persistent path: a segment's backward pass in one launch                   // FP32 2D adjoint: column parts on FFT groups (0: generic kernel)
+    int tune_resident = 1;                   // FP32 2D sides of 32..512: a run of steps with every slot in one cluster
+    int tune_res_ctas = 0;                   // its CTAs per cluster (0 = automatic)
+    int res_ctas_auto = 0, res_ctas_slots = 0;   // the automatic choice, for that many slots
+    mutable int res256_slots = 0;            // whether a 256^2 batch of that many slots takes that path
+    mutable bool res256_on = false;
     int tune_persist_blocks = 0;             // its CTAs (0: every SM, at most one CTA per column pair or row pair)
     int coop = 0;                            // the device takes cooperative launches
     // captured persistent launches by run length (one kernel node each); p2_capture < 0: capture
@@ -436,6 +441,72 @@ int p2_blocks(const pss_system *s) {
     const int lo = std::max((uc + 1) / 2, n / 8);
     const int want = s->tune_persist_blocks > 0 ? s->tune_persist_blocks : std::min(s->num_sms, std::max(uc, n / 2));
     return std::min(s->num_sms, std::max(lo, want));
+}
+
+// A run of steps of FP32 2D systems with sides of 32..512 points and power
+// products is one launch of one cluster per slot (k_res2d).
+bool side_res(int n) { return n == 32 || n == 64 || n == 128 || n == 256 || n == 512; }
+cudaError_t launch_res2(const Res2Args &a, int nslots, cudaStream_t st, int *active = nullptr) {
+    switch (a.sp.nx) {
+        case 32: return launch_res2_nx<32>(a, nslots, st, active);
+        case 64: return launch_res2_nx<64>(a, nslots, st, active);
+        case 128: return launch_res2_nx<128>(a, nslots, st, active);
+        case 256: return launch_res2_nx<256>(a, nslots, st, active);
+        case 512: return launch_res2_nx<512>(a, nslots, st, active);
+        default: return cudaErrorInvalidValue;
+    }
+}
+int res_active(const pss_system *s, int C) {
+    Res2Args a{};
+    a.sp = sys_params<float>(s);
+    a.C = C;
+    int active = 0;
+    if (launch_res2(a, s->nslots(), nullptr, &active) != cudaSuccess) { cudaGetLastError(); active = 0; }
+    return active;
+}
+// Where it is the faster path, measured on GB300 (us per step, other path ->
+// cluster-resident; batch x shape): with a side below 256 always (generic
+// kernels: 32^2 9.6 -> 2.7, 64^2 10.4 -> 3.2, 128^2 11.6 -> 4.2, 64^2 x 128
+// 13.7 -> 4.7, 128^2 x 128 27.3 -> 13.1, 128 x 512 12.4 -> 7.3, two fields of
+// 512 x 128 12.6 -> 8.4).  With both sides of 256 or more the two-kernel step
+// spreads one slot over the whole chip: 256^2 x 8 8.8 -> 10.1, x 32 20.7 ->
+// 17.6, x 128 73 -> 68, 512 x 256 8.2 -> 12.2, 512^2 x 32 85 -> 100; only
+// 256^2 gains, when its clusters of four fill most of the chip (36 at a time).
+constexpr int kRes256Fill = 29;   // slots per wave of 256^2 clusters from which it gains
+bool resident2d(const pss_system *s) {
+    if (!(s->tune_resident && s->tune_fast2d && s->prec == PSS_F32 && s->dim == 2 && side_res(s->nx) &&
+          side_res(s->ny) && !any_general(s) && !round_trip(s) && !s->tune_test_timeout))
+        return false;
+    if (s->nx < 256 || s->ny < 256) return true;
+    if (s->nx != 256 || s->ny != 256 || s->nslots() < kRes256Fill) return false;
+    if (s->res256_slots != s->nslots()) {
+        const int active = res_active(s, 4);
+        s->res256_on = active > 0 && s->nslots() >= kRes256Fill * ((s->nslots() + active - 1) / active);
+        s->res256_slots = s->nslots();
+    }
+    return s->res256_on;
+}
+// CTAs per cluster: the most that still run every slot at once and leave a CTA
+// kResSitesPerCta sites (64^2 on 1 .. 16 CTAs: 4.3, 3.8, 3.1, 3.2, 3.7 us per
+// step; 128^2: 13.0, 8.3, 5.4, 4.3, 4.1), else the fewest that hold one slot
+constexpr long long kResSitesPerCta = 512;
+int res_ctas(pss_system *s) {
+    int lo = 1;
+    while (lo < 16 && res2_smem_bytes(s->nx, s->ny, lo) > 227 * 1024) lo *= 2;
+    const int hi = std::min(16, s->ny / 2);
+    int c = lo;
+    if (s->tune_res_ctas > 0) {
+        while (c * 2 <= s->tune_res_ctas && c * 2 <= hi) c *= 2;
+        return c;
+    }
+    if (s->res_ctas_slots == s->nslots()) return s->res_ctas_auto;
+    for (int C = 2 * lo; C <= hi && s->nsites >= kResSitesPerCta * C; C *= 2) {
+        if (res_active(s, C) < s->nslots()) break;
+        c = C;
+    }
+    s->res_ctas_auto = c;
+    s->res_ctas_slots = s->nslots();
+    return c;
 }
 
 // Defaults of the FP32 2D two-kernel path.  A batch of 8 or more instances is
@@ -1113,7 +1184,15 @@ template <typename T> int step_once(pss_system *s, cudaStream_t st) {
     return full_prologue<T>(s, st);
 }
 
+int launch_resident(pss_system *s, int nsteps, cudaStream_t st);
+
 int record_steps(pss_system *s, cudaStream_t st, int64_t n) {
+    if (resident2d(s)) {
+        // (in a graph: a list with a system twice, recorded step by step)
+        int rc = PSS_OK;
+        for (int64_t k = 0; k < n && rc == PSS_OK; ++k) rc = launch_resident(s, 1, st);
+        return rc;
+    }
     for (int64_t k = 0; k < n; ++k) {
         int rc = s->prec == PSS_F64 ? step_once<double>(s, st) : step_once<float>(s, st);
         if (rc) return rc;
@@ -1272,11 +1351,82 @@ int run_persist(pss_system *s, int64_t n, cudaStream_t st) {
     return PSS_OK;
 }
 
+// The cluster-resident path: one launch per run of at most kMaxPersistSteps
+// steps.  It reads and writes only the state and the step counter; the work
+// arrays then hold nothing of the new state (stale), for the paths that use
+// them.
+int launch_resident(pss_system *s, int nsteps, cudaStream_t st) {
+    Res2Args a{};
+    a.sp = sys_params<float>(s);
+    a.fps = (const FieldP<float> *)s->fps;
+    a.state = (float2 *)s->state;
+    a.slot_stride = s->field_elems;
+    a.roots = (const float2 *)s->tw + kRootsOffset;
+    a.d_step = s->d_step;
+    a.d_status = s->d_status;
+    a.gs = s->gs;
+    a.nsteps = nsteps;
+    a.C = res_ctas(s);
+    cudaError_t e = launch_res2(a, s->nslots(), st);
+    s->launches++;
+    if (e != cudaSuccess) return cuda_fail(s, e, "k_res2d launch");
+    return PSS_OK;
+}
+
+int run_resident(pss_system *s, int64_t n, cudaStream_t st) {
+    for (int64_t done = 0; done < n;) {
+        const int len = (int)std::min<int64_t>(kMaxPersistSteps, n - done);
+        if (int rc = launch_resident(s, len, st)) return rc;
+        done += len;
+    }
+    s->stale = true;
+    return PSS_OK;
+}
+
+// pss_step_many: the resident systems' runs, side by side on their capture
+// streams after everything issued on the list's stream (the most costly
+// first; a single one with no graph beside it stays on that stream); the
+// others' graph follows on the list's stream, and join_resident makes that
+// stream wait for them.
+int run_resident_beside(pss_system *s0, std::vector<pss_system *> &res, bool beside, int64_t steps) {
+    if (res.empty()) return PSS_OK;
+    std::stable_sort(res.begin(), res.end(), [](const pss_system *a, const pss_system *b) {
+        return a->nsites * a->nslots() > b->nsites * b->nslots();
+    });
+    cudaEvent_t ev = nullptr;
+    if (beside || res.size() > 1) {
+        if (cudaError_t ce = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) return cuda_fail(s0, ce, "cudaEventCreateWithFlags");
+        cudaError_t e = cudaEventRecord(ev, s0->stream);
+        for (pss_system *s : res)
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(s->cap_stream, ev, 0);
+        cudaEventDestroy(ev);
+        if (e != cudaSuccess) return cuda_fail(s0, e, "forking the resident runs");
+    }
+    for (pss_system *s : res)
+        if (int rc = run_resident(s, steps, ev ? s->cap_stream : s0->stream)) return fail(s0, rc, "%s", s->err.c_str());
+    return PSS_OK;
+}
+
+int join_resident(pss_system *s0, const std::vector<pss_system *> &res) {
+    if (res.empty()) return PSS_OK;
+    cudaEvent_t ev = nullptr;
+    if (cudaError_t ce = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) return cuda_fail(s0, ce, "cudaEventCreateWithFlags");
+    cudaError_t e = cudaSuccess;
+    for (pss_system *s : res) {
+        if (e == cudaSuccess) e = cudaEventRecord(ev, s->cap_stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s0->stream, ev, 0);
+    }
+    cudaEventDestroy(ev);
+    if (e != cudaSuccess) return cuda_fail(s0, e, "joining the resident runs");
+    return PSS_OK;
+}
+
 // Every run of steps replays captured graphs: whole graphs of `graph_steps`
 // steps, then one graph of the remaining length (captured on its first use
 // and kept), so that the launches per step do not depend on n.
 int run_steps(pss_system *s, int64_t n) {
     if (persist2d(s)) return run_persist(s, n, s->stream);
+    if (resident2d(s)) return run_resident(s, n, s->stream);
     const int chunk = s->tune_graph_steps > 0 ? s->tune_graph_steps : kDefaultGraphSteps;
     if (!s->graph_valid) {
         drop_graphs(s);
@@ -1458,6 +1608,10 @@ int do_create(pss_system **out, int batch, int dim, int nx, int ny, int nz, doub
                             h[twiddle_offset(n, emax) + (P - E) + (r - 1) * P + k] = make_double2(std::cos(a), -std::sin(a));
                         }
             }
+        for (int j = 0; j < kMaxFftN; ++j) {
+            const double a = 2 * kPi * (double)j / kMaxFftN;
+            h[kRootsOffset + j] = make_double2(std::cos(a), -std::sin(a));
+        }
         if (precision == PSS_F64) {
             e = cudaMalloc(&s->tw, sizeof(double2) * total);
             if (e == cudaSuccess) e = cudaMemcpy(s->tw, h.data(), sizeof(double2) * total, cudaMemcpyHostToDevice);
@@ -1933,7 +2087,7 @@ int pss_step(pss_system *s, int64_t n) {
     int rc = upload_params(s);
     if (rc) return rc;
     if (round_trip(s) && (rc = ensure_real(s))) return rc;
-    if ((rc = prologue(s, persist2d(s)))) return rc;
+    if (!resident2d(s) && (rc = prologue(s, persist2d(s)))) return rc;
     if ((rc = run_steps(s, n))) return rc;
     s->step += n;
     return PSS_OK;
@@ -1953,10 +2107,23 @@ int pss_step_many(pss_system **systems, int n, int64_t steps) {
         }
         int rc = upload_params(s);
         if (!rc && round_trip(s)) rc = ensure_real(s);
-        if (!rc) rc = prologue(s);
+        if (!rc && !resident2d(s)) rc = prologue(s);
         if (rc) return i == 0 ? rc : fail(s0, rc, "%s", s->err.c_str());
     }
     if (steps == 0) return PSS_OK;
+    // systems on the cluster-resident path take all their steps in one launch
+    // each, on their own streams beside the others' graph (a system listed
+    // twice keeps the list order: everything in the graph)
+    std::vector<pss_system *> res, rest;
+    bool twice = false;
+    for (int i = 0; i < n; ++i)
+        for (int j = 0; j < i; ++j) twice |= systems[i] == systems[j];
+    for (int i = 0; i < n; ++i) (!twice && resident2d(systems[i]) ? res : rest).push_back(systems[i]);
+    if (int rc = run_resident_beside(s0, res, !rest.empty(), steps)) return rc;
+    pss_system **all = systems;
+    const int n_all = n;
+    systems = rest.data();
+    n = (int)rest.size();
     const int chunk = s0->tune_graph_steps > 0 ? s0->tune_graph_steps : kDefaultGraphSteps;
     // graphs of whole chunks and of the remainder, kept on systems[0] for this
     // list of systems as long as none of them changed its launches
@@ -1991,7 +2158,7 @@ int pss_step_many(pss_system **systems, int n, int64_t steps) {
         return PSS_OK;
     };
     int64_t done = 0;
-    while (done < steps) {
+    while (n > 0 && done < steps) {
         const int len = (int)std::min<int64_t>(chunk, steps - done);
         cudaGraphExec_t ge = nullptr;
         if (int rc = graph_of(len, &ge)) return rc;
@@ -2000,7 +2167,11 @@ int pss_step_many(pss_system **systems, int n, int64_t steps) {
         for (int i = 0; i < n; ++i) systems[i]->launches += (int64_t)len * systems[i]->graph_launches;
         done += len;
     }
-    for (int i = 0; i < n; ++i) systems[i]->step += steps;
+    if (int rc = join_resident(s0, res)) return rc;
+    for (int i = 0; i < n_all; ++i) {
+        all[i]->step += steps;
+        if (resident2d(all[i])) all[i]->stale = true;
+    }
     return PSS_OK;
 }
 
@@ -2134,6 +2305,11 @@ int pss_set_tuning(pss_system *s, const char *key, int value) {
     else if (k == "real_state") s->tune_real_state = value ? 1 : 0;
     else if (k == "test_timeout") s->tune_test_timeout = value ? 1 : 0;
     else if (k == "persist") s->tune_persist = value ? 1 : 0;
+    else if (k == "resident") s->tune_resident = value ? 1 : 0;
+    else if (k == "res_ctas") {
+        if (value > 16) return fail(s, PSS_EINVAL, "res_ctas is at most 16 (0 = automatic)");
+        s->tune_res_ctas = value;
+    }
     else if (k == "adj_col2") s->tune_adj_col2 = value ? 1 : 0;
     else if (k == "persist_adj") s->tune_persist_adj = value ? 1 : 0;
     else if (k == "adj_radix") {

@@ -25,7 +25,9 @@ constexpr int kMaxFftN = 1024;
 __host__ __device__ constexpr int twiddle_offset(int n, int emax) {
     return (emax == 32 ? 4 * kMaxFftN : emax == 16 ? 2 * kMaxFftN : 0) + n;
 }
-constexpr int kTwiddleEntries = 6 * kMaxFftN;
+// behind the tables: the kMaxFftN-th roots of unity, exp(-2 pi i j / kMaxFftN)
+constexpr int kRootsOffset = 6 * kMaxFftN;
+constexpr int kTwiddleEntries = 7 * kMaxFftN;
 
 constexpr int kTileW = 4;       // kx columns per tile of every spectral array
 constexpr int kMaxFields = 4;
@@ -257,6 +259,34 @@ struct P2AdjArgs {
     int len;                    // steps of the segment (>= 1)
 };
 cudaError_t launch_p2_adj(const P2AdjArgs &a, int n, int E, int nblocks, cudaStream_t st);
+// The cluster-resident FP32 2D step (k_res2d: sides of 32..512 points): one
+// cluster of C CTAs per slot runs nsteps steps.
+#ifndef PSS_RES_E8
+#define PSS_RES_E8 128
+#endif
+constexpr int kResMaxThreads = 576;    // transform threads of a CTA
+constexpr int kResNoiseWarps = 4;      // and the warps that draw the noise
+struct Res2Args {
+    SysP<float> sp;
+    const FieldP<float> *fps;
+    float2 *state;              // tiled, slot_stride apart
+    size_t slot_stride;
+    const float2 *roots;        // exp(-2 pi i j / kMaxFftN)
+    long long *d_step;
+    int *d_status;
+    GridSync *gs;               // done: CTAs finished (the last one advances *d_step)
+    int nsteps;
+    int C;                      // CTAs per cluster, a power of two
+};
+// Values per thread of a transform of n points there, the points of shared
+// memory it takes, and a CTA's dynamic shared memory (C CTAs per cluster)
+__host__ __device__ constexpr int res_e(int n) { return n <= PSS_RES_E8 ? 8 : 16; }
+__host__ __device__ constexpr int res_xld(int n) { return n + res_e(n) + 2; }
+__host__ __device__ constexpr size_t res2_smem_bytes(int nx, int ny, int C) {
+    const size_t cols = 2 * (size_t)(((nx / 2 + 2) / 2 + C - 1) / C), pairs = (size_t)(ny / 2 / C);
+    return 256 + sizeof(float2) * ((size_t)nx + ny + cols * (ny + 2 + res_xld(ny)) + pairs * res_xld(nx));
+}
+template <int NX> cudaError_t launch_res2_nx(const Res2Args &a, int nslots, cudaStream_t st, int *active);
 template <typename T> cudaError_t launch_init_uniform(T *real, long long nsites, double lo, double hi,
                                                       uint64_t seed, int field_id, cudaStream_t st);
 // product terms with several operators: Q = (first ? 0 : Q) + M(q) Pt over one

@@ -1,0 +1,7 @@
+// pss_kern_res2d_64.cu -- the cluster-resident 2D step for rows of 64 points
+// (a translation unit per row length so that nvcc builds them in parallel).
+#include "pss_resident2d.cuh"
+
+namespace pss {
+template cudaError_t launch_res2_nx<64>(const Res2Args &, int, cudaStream_t, int *);
+}
