@@ -333,12 +333,54 @@ int upload_params(pss_system *s) { return s->prec == PSS_F64 ? upload_params_t<d
 // (more warps to hide latency).  Measured on GB300: the column kernel is
 // faster with radix 16 for 3D pencils and 1024-point columns, the row
 // kernel with radix 8, the 3D y kernel with radix 16.
+//
+// FP64 is bound by its arithmetic: a scheduler issues one FP64 warp
+// instruction in 64 cycles, whatever the number of active lanes, so a step
+// takes as long as its busiest scheduler.  Radix 4 costs the same operations
+// per point as radix 8 and gives every transform twice the threads, the
+// column kernel's CTAs take single columns, and the launch shapes below spread
+// the work over every SM's four schedulers (us per step before -> after:
+// 128^2 60 -> 21, 256^2 80 -> 27, 1024^2 310 -> 256, 64 x 32 x 128 148 -> 70,
+// 32^3 118 -> 29; the normals of noise_mode are a part of it).
+// FP64 radix: transforms of n points, `count` of them in a launch.  Radix 2
+// costs a fifth more operations and doubles the threads again: for launches
+// that would leave schedulers without a warp.  Below 16 points a transform is
+// one pass (the kernels stage no twiddles).
+int f64_radix(const pss_system *s, int n, long long count) {
+    if (n < 16) return 8;
+    return n <= 512 && count * n / 4 <= 32ll * 4 * s->num_sms ? 2 : 4;
+}
 int col_emax(const pss_system *s) {
     if (s->tune_col_radix) return s->tune_col_radix;
     return (s->dim == 3 || s->n_inner >= 1024) ? 16 : 8;
 }
-int row_emax(const pss_system *s) { return s->tune_row_radix ? s->tune_row_radix : 8; }
-int mid_emax(const pss_system *s) { return s->tune_mid_radix ? s->tune_mid_radix : 16; }
+int row_emax(const pss_system *s) {
+    return s->tune_row_radix ? s->tune_row_radix
+         : s->prec == PSS_F64 ? f64_radix(s, s->nx, (long long)(s->rows + 1) / 2 * s->nslots()) : 8;
+}
+// (a y CTA holds at least kTileW transforms and at most 256 threads)
+int mid_emax(const pss_system *s) {
+    return s->tune_mid_radix ? s->tune_mid_radix : s->prec != PSS_F64 ? 16
+         : s->ny < 16 ? 8 : s->ny <= 256 ? 4 : s->ny <= 512 ? 8 : 16;
+}
+// FP64 column kernel on single columns (not the adjoint's modes): at least 16
+// points per column, and a CTA of at most 512 transform threads
+bool col_single(const pss_system *s, int mode) {
+    return s->prec == PSS_F64 && !s->tune_col_radix && !s->tune_col_tiles && mode != COL_ADJ_A && mode != COL_ADJ_B &&
+           mode != COL_ADJ_BA && s->n_inner >= 16;
+}
+// columns per CTA there: as many as leave kF64Ctas CTAs per SM, at most 64
+// transform threads
+constexpr int kF64Ctas = 6;
+long long col_pencils(const pss_system *s) { return (long long)s->hx * (s->dim == 3 ? s->ny / 2 + 1 : 1) * s->nslots(); }
+int col_single_radix(const pss_system *s) { return f64_radix(s, s->n_inner, col_pencils(s) * (s->dim == 3 ? 2 : 1)); }
+int col_singles_per_cta(const pss_system *s) {
+    const int per = (s->dim == 3 ? 2 : 1) * fft_TPF(s->n_inner, col_single_radix(s));
+    const long long ctas = col_pencils(s);
+    int tc = 1;
+    while (tc * 2 * per <= 64 && tc * 2 <= s->hx && (tc * per < 16 || ctas / (2 * tc) >= kF64Ctas * s->num_sms)) tc *= 2;
+    return tc;
+}
 
 // tiles per CTA of the column kernel: a power of two, so that the CTA's
 // FFT count F = tiles * kTileW * NP is one; aims at >= 64 threads per CTA
@@ -366,6 +408,12 @@ int row_G(const pss_system *s) {
     }
     const int want = std::max(1, (s->rows / 2 + 7) / 8);
     int G = 1;
+    if (s->prec == PSS_F64) {
+        // whole warps; up to 128 threads where kF64Ctas CTAs per SM are left
+        while (G * tpf < 32 && G * 2 <= std::max(1, s->rows / 2)) G *= 2;
+        while (G * 2 * tpf <= 128 && (long long)s->rows / (4 * G) * s->nslots() >= kF64Ctas * s->num_sms) G *= 2;
+        return G;
+    }
     while (G * 2 * tpf <= 128 && G * 2 <= want) G *= 2;
     return G;
 }
@@ -379,6 +427,10 @@ int mid_PZ(const pss_system *s) {
         pz = p;
     }
     pz = std::min(pz, s->nz);
+    if (s->prec == PSS_F64 && s->tune_mid_planes <= 0)
+        while (pz > 1 && (kTileW * tpf * pz > 128 ||
+                          (kTileW * tpf * pz > 32 && (long long)s->ntiles * (s->nz / pz) * s->nslots() < kF64Ctas * s->num_sms)))
+            pz /= 2;
     return pz;
 }
 
@@ -649,11 +701,14 @@ template <typename T> struct Seq {
         a.d_step = s->d_step;
         a.d_status = s->d_status;
         a.mode = mode;
-        a.E = col_emax(s);
-        a.tiles_per_cta = col_tiles_per_cta(s);
-        a.F = a.tiles_per_cta * kTileW * (s->dim == 3 ? 2 : 1);
+        const bool single = col_single(s, mode);
+        a.E = single ? col_single_radix(s) : col_emax(s);
+        a.wc = single ? 1 : kTileW;
+        a.tiles_per_cta = single ? col_singles_per_cta(s) : col_tiles_per_cta(s);
+        a.F = a.tiles_per_cta * a.wc * (s->dim == 3 ? 2 : 1);
         a.n_tiles = mode == COL_INV_MASK ? max_kept_tiles(s) : s->ntiles;
-        const int gx = (a.n_tiles + a.tiles_per_cta - 1) / a.tiles_per_cta;
+        const int cols = single ? std::min(a.n_tiles * kTileW, s->hx) : a.n_tiles;
+        const int gx = (cols + a.tiles_per_cta - 1) / a.tiles_per_cta;
         const int gy = s->dim == 3 ? s->ny / 2 + 1 : 1;
         if constexpr (std::is_same<T, float>::value) {
             // the adjoint's column part of the FP32 2D path on FFT groups: one
@@ -1554,6 +1609,44 @@ int grow_arrays(pss_system *s, int old_nf) {
     return PSS_OK;
 }
 
+// Twiddle tables of every transform length and radix cap, the roots of unity
+// and the logarithm tables, built once in FP64 (pss_internal.h has the layout)
+const std::vector<double2> &host_tables() {
+    static const std::vector<double2> tables = [] {
+        std::vector<double2> h(kTwiddleEntries, make_double2(0.0, 0.0));
+        for (int emax : {2, 4, 8, 16, 32})
+            for (int n = 2; n <= kMaxFftN; n *= 2) {
+                const int E = fft_E(n, emax);
+                for (int P = E, R = std::min(E, n / P); P < n; P *= R, R = std::min(E, n / P))
+                    for (int r = 1; r < R; ++r)
+                        for (int k = 0; k < P; ++k) {
+                            const double a = 2 * kPi * (double)(r * k) / (double)(P * R);
+                            h[twiddle_offset(n, emax) + (P - E) + (r - 1) * P + k] = make_double2(std::cos(a), -std::sin(a));
+                        }
+            }
+        for (int j = 0; j < kMaxFftN; ++j) {
+            // by symmetry from the first octant, so that the axes and diagonals are exact
+            const int q = j & (kMaxFftN / 4 - 1), o = std::min(q, kMaxFftN / 4 - q);
+            const double a = 2 * kPi * (double)o / kMaxFftN;
+            double c = std::cos(a), s = std::sin(a);
+            if (o != q) std::swap(c, s);
+            for (int quarter = j / (kMaxFftN / 4); quarter > 0; --quarter) { const double x = c; c = -s; s = x; }
+            h[kRootsOffset + j] = make_double2(c, -s);
+        }
+        // (1/c, ln c) of the interval j of [1, 2), the upper half taken at half its
+        // value; c = 1 for the two intervals next to 1
+        for (int j = 0; j < kLogEntries; ++j) {
+            long double c = 1.0L + (j + 0.5L) / kLogEntries;
+            if (j >= kLogEntries / 2) c /= 2;
+            const double inv = (j == 0 || j == kLogEntries - 1) ? 1.0 : (double)(1.0L / c);
+            h[kLogOffset + j] = make_double2(inv, (double)-std::log((long double)inv));
+        }
+        for (int k = 0; k < 32; ++k) h[kLn2Offset + k] = make_double2((double)(k * std::log(2.0L)), 0.0);
+        return h;
+    }();
+    return tables;
+}
+
 int do_create(pss_system **out, int batch, int dim, int nx, int ny, int nz, double dx, double dy, double dz, double dt,
               const uint64_t *seeds, int precision) {
     if (!out) return fail(nullptr, PSS_EINVAL, "out is NULL");
@@ -1594,24 +1687,9 @@ int do_create(pss_system **out, int batch, int dim, int nx, int ny, int nz, doub
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&s->coop, cudaDevAttrCooperativeLaunch, s->device);
     if (e == cudaSuccess) e = cudaMalloc(&s->gs, sizeof(GridSync));
     if (e == cudaSuccess) e = cudaMemset(s->gs, 0, sizeof(GridSync));
-    // twiddle tables of every transform length and radix cap, built in FP64 on the host
     if (e == cudaSuccess) {
-        const int total = kTwiddleEntries;
-        std::vector<double2> h(total, make_double2(0.0, 0.0));
-        for (int emax : {8, 16, 32})
-            for (int n = 2; n <= kMaxFftN; n *= 2) {
-                const int E = fft_E(n, emax);
-                for (int P = E, R = std::min(E, n / P); P < n; P *= R, R = std::min(E, n / P))
-                    for (int r = 1; r < R; ++r)
-                        for (int k = 0; k < P; ++k) {
-                            const double a = 2 * kPi * (double)(r * k) / (double)(P * R);
-                            h[twiddle_offset(n, emax) + (P - E) + (r - 1) * P + k] = make_double2(std::cos(a), -std::sin(a));
-                        }
-            }
-        for (int j = 0; j < kMaxFftN; ++j) {
-            const double a = 2 * kPi * (double)j / kMaxFftN;
-            h[kRootsOffset + j] = make_double2(std::cos(a), -std::sin(a));
-        }
+        const std::vector<double2> &h = host_tables();
+        const int total = (int)h.size();
         if (precision == PSS_F64) {
             e = cudaMalloc(&s->tw, sizeof(double2) * total);
             if (e == cudaSuccess) e = cudaMemcpy(s->tw, h.data(), sizeof(double2) * total, cudaMemcpyHostToDevice);

@@ -113,17 +113,6 @@ __device__ __forceinline__ float root_approx(float x) {
     return fmul(x, r);
 }
 
-// Box-Muller pair in FP64 (the library calls).  FP32 draws its normals in
-// noise_mode, with the hardware log2 / sqrt / sin / cos approximations
-// (absolute error ~1e-6 on these arguments).
-__device__ __forceinline__ void box_muller(double u0, double u1, double &n1, double &n2) {
-    const double r = sqrt(-2.0 * log(u0));
-    double s, c;
-    sincospi(2.0 * u1, &s, &c);
-    n1 = r * c;
-    n2 = r * s;
-}
-
 // ---------------------------------------------------------------------------
 // 32nd roots of unity: cos(2 pi k / 32) from the exact first-octant values
 // (cos(j pi / 16), j = 0..8) by quadrant symmetry.
@@ -193,7 +182,7 @@ template <int R, int DIR, typename T> __device__ __forceinline__ void dft_reg(cp
 // Stockham radix-R pass with P = product of the radices already done:
 // butterfly i (0 <= i < N/R) reads x[i + r N/R], multiplies by
 // exp(DIR 2 pi i r k / (P R)) with k = i mod P, transforms over r, and writes
-// y[(i / P) P R + k + r P].  N = E^m * RL: m radix-E passes (E = 8 or 16; the
+// y[(i / P) P R + k + r P].  N = E^m * RL: m radix-E passes (E = 2, 4, 8 or 16; the
 // middle ones share one loop body), then one radix-RL pass.  The first pass reads through a source
 // functor and the last pass writes through a sink functor, so that
 // element-wise work (a power, a mask, a scale, a store to global memory)

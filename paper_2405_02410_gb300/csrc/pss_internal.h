@@ -13,7 +13,7 @@ template <> struct CplxOf<double> { using type = double2; };
 template <typename T> using cplx = typename CplxOf<T>::type;
 
 // Twiddle factors: the host builds, in FP64, one table per transform length
-// n = 2, 4, ..., kMaxFftN and radix cap emax (8, 16 or 32).  A length-n FFT runs
+// n = 2, 4, ..., kMaxFftN and radix cap emax (2, 4, 8, 16 or 32).  A length-n FFT runs
 // radix-E passes (E = min(n, emax)) and a last pass of radix n / P (<= E).
 // The pass that follows P > 1 points already transformed, of radix
 // R = min(E, n / P), needs exp(-2 pi i r k / (P R)) for 1 <= r < R, k < P,
@@ -23,11 +23,16 @@ template <typename T> using cplx = typename CplxOf<T>::type;
 // copy.
 constexpr int kMaxFftN = 1024;
 __host__ __device__ constexpr int twiddle_offset(int n, int emax) {
-    return (emax == 32 ? 4 * kMaxFftN : emax == 16 ? 2 * kMaxFftN : 0) + n;
+    return (emax == 2 ? 8 * kMaxFftN : emax == 4 ? 6 * kMaxFftN : emax == 32 ? 4 * kMaxFftN : emax == 16 ? 2 * kMaxFftN : 0) + n;
 }
-// behind the tables: the kMaxFftN-th roots of unity, exp(-2 pi i j / kMaxFftN)
-constexpr int kRootsOffset = 6 * kMaxFftN;
-constexpr int kTwiddleEntries = 7 * kMaxFftN;
+// behind the tables: the kMaxFftN-th roots of unity, exp(-2 pi i j / kMaxFftN),
+// and (FP64) the logarithm tables of noise_mode: kLogEntries pairs (1/c, ln c)
+// and the multiples k ln 2, k < 32 (in x)
+constexpr int kRootsOffset = 10 * kMaxFftN;
+constexpr int kLogOffset = 11 * kMaxFftN;
+constexpr int kLogEntries = 128;
+constexpr int kLn2Offset = kLogOffset + kLogEntries;
+constexpr int kTwiddleEntries = kLn2Offset + 32;
 
 constexpr int kTileW = 4;       // kx columns per tile of every spectral array
 constexpr int kMaxFields = 4;
@@ -103,8 +108,9 @@ template <typename T> struct ColArgs {
     long long *d_step;    // step counter (k2_col advances it)
     int *d_status;
     int mode, tiles_per_cta, n_tiles;
-    int E;                // FFT radix cap (8 or 16), chosen by the host
-    int F;                // FFTs per CTA = tiles_per_cta * kTileW * (2 in 3D, else 1); a power of two
+    int E;                // FFT radix cap (2, 4, 8 or 16), chosen by the host
+    int wc;               // columns of a chunk: kTileW, or 1 (FP64, E <= 4; tiles_per_cta then counts columns)
+    int F;                // FFTs per CTA = tiles_per_cta * wc * (2 in 3D, else 1); a power of two
     // adjoint (COL_ADJ_A): the forward state after the step, its noise step, and
     // the FP64 gradient sums [slot][11] (dO_0..4, dM_0..4, sum Re(conj(mu) xi))
     const cplx<T> *aux;
@@ -137,7 +143,7 @@ template <typename T> struct RowArgs {
     long long *d_step;
     int *d_status;
     int mode, G, inc_step;
-    int E;                // FFT radix cap (8 or 16)
+    int E;                // FFT radix cap (2, 4, 8 or 16)
     int kx_cols_max;      // largest kept half-spectrum column count over the launch's slots
     cplx<T> *noise;       // k2_row: where the unit-amplitude noise of step *d_step goes (null: none)
     int noise_warps;      // k2_row: warps that draw it beside the transform warps
@@ -162,7 +168,7 @@ template <typename T> struct MidArgs {
     long long *d_step;
     int *d_status;
     int mode, PZ, inc_step;
-    int E;                // FFT radix cap (8 or 16)
+    int E;                // FFT radix cap (2, 4, 8 or 16)
 };
 
 // Launch configuration chosen by the host.
@@ -171,7 +177,8 @@ struct RowCfg { int G; };
 struct MidCfg { int PZ; };
 
 // Launchers of the step kernels, one instantiation per precision and FFT
-// radix cap EMAX (pss_kern_{f32,f64}.cu: 8, pss_kern_{f32,f64}_r16.cu: 16).
+// radix cap EMAX (pss_kern_{f32,f64}.cu: 8, pss_kern_{f32,f64}_r16.cu: 16,
+// pss_kern_f64_r4.cu: 4 and pss_kern_f64_r2.cu: 2, FP64 only).
 template <typename T, int EMAX>
 cudaError_t launch_col_e(const ColArgs<T> &a, int nslots, int grid_x, int grid_y, cudaStream_t st);
 template <typename T, int EMAX> cudaError_t launch_row_e(const RowArgs<T> &a, int nslots, cudaStream_t st);
@@ -179,16 +186,24 @@ template <typename T, int EMAX> cudaError_t launch_mid_e(const MidArgs<T> &a, in
 // dynamic shared memory of one column-kernel CTA (0: side not supported)
 template <typename T, int EMAX> size_t col_smem_bytes_e(int n_inner, int F, int mode);
 template <typename T> inline size_t col_smem_bytes(int n_inner, int F, int E, int mode) {
+    if constexpr (sizeof(T) == 8)
+        if (E <= 4) return E == 2 ? col_smem_bytes_e<T, 2>(n_inner, F, mode) : col_smem_bytes_e<T, 4>(n_inner, F, mode);
     return E == 16 ? col_smem_bytes_e<T, 16>(n_inner, F, mode) : col_smem_bytes_e<T, 8>(n_inner, F, mode);
 }
 template <typename T>
 inline cudaError_t launch_col(const ColArgs<T> &a, int nslots, int grid_x, int grid_y, cudaStream_t st) {
+    if constexpr (sizeof(T) == 8)
+        if (a.E <= 4) return a.E == 2 ? launch_col_e<T, 2>(a, nslots, grid_x, grid_y, st) : launch_col_e<T, 4>(a, nslots, grid_x, grid_y, st);
     return a.E == 16 ? launch_col_e<T, 16>(a, nslots, grid_x, grid_y, st) : launch_col_e<T, 8>(a, nslots, grid_x, grid_y, st);
 }
 template <typename T> inline cudaError_t launch_row(const RowArgs<T> &a, int nslots, cudaStream_t st) {
+    if constexpr (sizeof(T) == 8)
+        if (a.E <= 4) return a.E == 2 ? launch_row_e<T, 2>(a, nslots, st) : launch_row_e<T, 4>(a, nslots, st);
     return a.E == 16 ? launch_row_e<T, 16>(a, nslots, st) : launch_row_e<T, 8>(a, nslots, st);
 }
 template <typename T> inline cudaError_t launch_mid(const MidArgs<T> &a, int nslots, int n_tiles, cudaStream_t st) {
+    if constexpr (sizeof(T) == 8)
+        if (a.E <= 4) return a.E == 2 ? launch_mid_e<T, 2>(a, nslots, n_tiles, st) : launch_mid_e<T, 4>(a, nslots, n_tiles, st);
     return a.E == 16 ? launch_mid_e<T, 16>(a, nslots, n_tiles, st) : launch_mid_e<T, 8>(a, nslots, n_tiles, st);
 }
 // The FP32 path with one FFT group per transform (sides 256, 512 or 1024):
@@ -311,7 +326,7 @@ template <typename T> cudaError_t launch_structure_factor(const SysP<T> &sp, con
 // FFT shape helpers visible to the host
 __host__ __device__ constexpr int ilog2(int n) { return n <= 1 ? 0 : 1 + ilog2(n >> 1); }
 // Values per thread and pass of a length-n FFT (the radix of its main
-// passes) when a kernel runs its FFTs with at most emax (8 or 16) values per
+// passes) when a kernel runs its FFTs with at most emax (2, 4, 8 or 16) values per
 // thread: radix 16 means fewer passes, radix 8 twice the threads per FFT.
 __host__ __device__ constexpr int fft_E(int n, int emax) { return n < emax ? n : emax; }
 __host__ __device__ constexpr int fft_TPF(int n, int emax) { return n / fft_E(n, emax); }

@@ -39,15 +39,6 @@ template <typename T> __device__ __forceinline__ T poly5(const T *c, T x) {
 
 __device__ __forceinline__ int signed_k(int k, int n) { return k < (n + 1) / 2 ? k : k - n; }
 
-// sigma0 |q|^p with |q| = sqrt(q2)
-template <typename T> __device__ __forceinline__ T noise_amp(T sigma0, int p, T q2) {
-    if (p == 0) return sigma0;
-    const T qa = fast_sqrt(q2);
-    T amp = sigma0;
-    for (int i = 0; i < p; ++i) amp *= qa;
-    return amp;
-}
-
 // A pair of independent normals of standard deviation sigma0 |q|^p (Box-Muller
 // of two generator words).  FP32: drawing noise is a large part of every
 // step's instructions (issue-bound kernels), so the odd power of |q| goes
@@ -66,11 +57,51 @@ __device__ __forceinline__ float2 noise_mode(uint32_t w0, uint32_t w1, float sig
     __sincosf(fmul(6.283185307179586f, u1), &s, &c);
     return mk<float>(fmul(r, c), fmul(r, s));
 }
-__device__ __forceinline__ double2 noise_mode(uint32_t w0, uint32_t w1, double sigma0, int p, double q2) {
-    double n1, n2;
-    box_muller(uniform24<double>(w0), uniform24<double>(w1), n1, n2);
-    const double amp = noise_amp<double>(sigma0, p, q2);
-    return mk<double>(amp * n1, amp * n2);
+__device__ __forceinline__ float2 noise_mode(uint32_t w0, uint32_t w1, float sigma0, int p, float q2, const float2 *) {
+    return noise_mode(w0, w1, sigma0, p, q2);
+}
+// FP64: a GB300 scheduler issues one FP64 warp instruction in 64 cycles, so
+// the draw is written for few FP64 operations: both uniforms are 25-bit odd
+// integers over 2^25, whose reduction for the logarithm and the sine is
+// integer work, and the reduced arguments are small against a table
+// (table-driven reduction as in Tang, ACM TOMS 15 (1989) and 16 (1990)):
+//   -ln u0 = k ln 2 - ln c - ln(1 + r), c the centre of one of 128 intervals of
+//       [3/4, 3/2) (c = 1 next to 1, so that u0 -> 1 keeps its relative
+//       accuracy), |r| < 2^-7, the series to r^8 (relative remainder 2^-59);
+//   cos, sin of 2 pi u1 = the 1024th roots of unity turned by |d| < 0.0031, the
+//       series to d^4, d^5 (remainder below 2e-18).
+// 35 FP64 operations per mode with the root, against 80 with the library's log,
+// sincospi and two roots.  tw: the system's tables (kRootsOffset, kLogOffset).
+__device__ __forceinline__ double2 noise_mode(uint32_t w0, uint32_t w1, double sigma0, int p, double q2,
+                                              const double2 *__restrict__ tw) {
+    // u0 = n 2^-25 = m 2^-k, m in [3/4, 3/2)
+    const uint32_t n = (w0 >> 7) | 1u;
+    const int lz = __clz((int)n);
+    const uint32_t f = n << lz;                                       // [1, 2) with 31 bits after the point
+    const uint32_t upper = (f >> 30) & 1u;                            // 3/2 and above: halved
+    const int k = lz - 6 - (int)upper;
+    const double m = __hiloint2double((int)(((0x3ffu - upper) << 20) | ((f & 0x7fffffffu) >> 11)), (int)(f << 21));
+    const double2 t = __ldg(tw + kLogOffset + ((f >> 24) & (kLogEntries - 1)));
+    const double r = fma(m, t.x, -1.0);
+    double s = fma(r, -1.0 / 8, 1.0 / 7);
+    s = fma(s, r, -1.0 / 6);
+    s = fma(s, r, 1.0 / 5);
+    s = fma(s, r, -1.0 / 4);
+    s = fma(s, r, 1.0 / 3);
+    s = fma(s, r, -1.0 / 2);
+    double L = (__ldg(&tw[kLn2Offset + k].x) - t.y) - fma(r * r, s, r);
+    // u1 = n1 2^-25 turns = j / 1024 + d / (2 pi)
+    const int n1 = (int)((w1 >> 7) | 1u), j = (n1 + (1 << 14)) >> 15;
+    const double d = (double)(n1 - (j << 15)) * (6.283185307179586 / 33554432.0);      // 2 pi / 2^25
+    const double2 e = __ldg(tw + kRootsOffset + (j & (kMaxFftN - 1)));     // cos, -sin
+    const double z = d * d;
+    const double sd = fma(d * z, fma(z, 1.0 / 120, -1.0 / 6), d), cd = z * fma(z, 1.0 / 24, -0.5);
+    const double c = fma(e.x, cd, fma(e.y, sd, e.x)), si = fma(e.x, sd, fma(-e.y, cd, -e.y));
+    if (p & 1) L *= q2;
+    double amp = 1.4142135623730951 * sigma0;
+    if (p >= 2) amp *= p >= 4 ? q2 * q2 : q2;                          // p is 0 .. 4
+    const double R = sqrt(L) * amp;
+    return mk<double>(R * c, R * si);
 }
 
 // Noise increments xi_q of two neighbouring modes kx0 = 2j, kx1 = 2j + 1 of
@@ -82,10 +113,12 @@ __device__ __forceinline__ double2 noise_mode(uint32_t w0, uint32_t w1, double s
 // A mode that is its own partner is real.  The per-component standard
 // deviations are sigma0 |q|^npow = sqrt(N_sites D~(q) dt / dV); q2a, q2b are
 // the two modes' q^2.  on_plane: kx0 is 0 or Nx/2 (its partner is (kx0, -ky, -kz)).
+// tw: the system's tables (FP64).
 template <typename T>
 __device__ __forceinline__ void noise_pair(bool on_plane, int kx0, int ky, int kz, T sigma0, int npow, T q2a, T q2b,
                                            bool has1, const SysP<T> &sp, uint32_t fid, const PhiloxKey &key,
-                                           uint32_t step, cplx<T> &xi0, cplx<T> &xi1) {
+                                           uint32_t step, cplx<T> &xi0, cplx<T> &xi1,
+                                           const cplx<T> *__restrict__ tw = nullptr) {
     const uint32_t row = (uint32_t)(kz * sp.ny + ky);
     uint32_t crow = row;
     bool cj = false, selfc = false;
@@ -95,7 +128,7 @@ __device__ __forceinline__ void noise_pair(bool on_plane, int kx0, int ky, int k
         if (prow < row) { crow = prow; cj = true; }
     }
     u32x4 r = philox4x32_10(u32x4{(crow * (uint32_t)sp.hxe + (uint32_t)kx0) >> 1, step, fid, 0u}, key);
-    xi0 = noise_mode(r.x, r.y, sigma0, npow, q2a);
+    xi0 = noise_mode(r.x, r.y, sigma0, npow, q2a, tw);
     if (on_plane) {
         if (cj) xi0.y = -xi0.y;
         if (selfc) xi0 = mk<T>(T(1.4142135623730951) * xi0.x, T(0));
@@ -104,8 +137,36 @@ __device__ __forceinline__ void noise_pair(bool on_plane, int kx0, int ky, int k
         // kx1 is odd, so it is never 0 or Nx/2: it is its own canonical member
         if (crow != row)
             r = philox4x32_10(u32x4{(row * (uint32_t)sp.hxe + (uint32_t)kx0) >> 1, step, fid, 0u}, key);
-        xi1 = noise_mode(r.z, r.w, sigma0, npow, q2b);
+        xi1 = noise_mode(r.z, r.w, sigma0, npow, q2b, tw);
     }
+}
+
+// The draw of one mode (kx, ky, kz) alone: its own words of the pair's call.
+template <typename T>
+__device__ __forceinline__ cplx<T> noise_one(bool on_plane, int kx, int ky, int kz, T sigma0, int npow, T q2,
+                                             const SysP<T> &sp, uint32_t fid, const PhiloxKey &key, uint32_t step,
+                                             const cplx<T> *__restrict__ tw) {
+    const uint32_t row = (uint32_t)(kz * sp.ny + ky);
+    uint32_t crow = row;
+    bool cj = false, selfc = false;
+    if (on_plane) {   // kx is 0 or Nx/2, even
+        const uint32_t prow = (uint32_t)(((sp.nz - kz) & (sp.nz - 1)) * sp.ny + ((sp.ny - ky) & (sp.ny - 1)));
+        selfc = prow == row;
+        if (prow < row) { crow = prow; cj = true; }
+    }
+    const u32x4 r = philox4x32_10(u32x4{(crow * (uint32_t)sp.hxe + (uint32_t)kx) >> 1, step, fid, 0u}, key);
+    cplx<T> xi = noise_mode((kx & 1) ? r.z : r.x, (kx & 1) ? r.w : r.y, sigma0, npow, q2, tw);
+    if (cj) xi.y = -xi.y;
+    if (selfc) xi = mk<T>(T(1.4142135623730951) * xi.x, T(0));
+    return xi;
+}
+
+// False for NaN, infinities and values next to overflow.  FP64 looks at the
+// exponents (integer work; 2^997 and above count as overflow).
+__device__ __forceinline__ bool finite_mode(float2 v) { return fabsf(v.x) + fabsf(v.y) <= 3.0e38f; }
+__device__ __forceinline__ bool finite_mode(double2 v) {
+    const int lim = 0x7e400000;
+    return (__double2hiint(v.x) & 0x7fffffff) < lim && (__double2hiint(v.y) & 0x7fffffff) < lim;
 }
 
 // two neighbouring complex values at a 16-byte aligned address (one 16-byte
@@ -278,7 +339,7 @@ __device__ __forceinline__ void col_adjoint(const ColArgs<T> &a, const FieldP<T>
                 const T q2e = qe * qe + qy * qy + qz * qz, q2o = qo * qo + qy * qy + qz * qz;
                 noise_pair<T>(kx0 == 0 || 2 * kx0 == sp.nx, kx0, ky, kz, fp.sigma0, fp.noise_pow, q2e, q2o,
                               kx0 + 1 < sp.hx, sp, (uint32_t)fp.field_id,
-                              key, step, xin[0], xin[1]);
+                              key, step, xin[0], xin[1], a.tw);
             }
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
@@ -370,31 +431,36 @@ __device__ __forceinline__ void col_adjoint(const ColArgs<T> &a, const FieldP<T>
     if (t == 0) bulk_wait_read();
 }
 
-template <typename T, int N> struct ColSmem {
-    static constexpr int CS = N * W + 8;                         // chunk stride (elements)
+template <typename T, int N, int WC = W> struct ColSmem {
+    static constexpr int CS = N * WC + 8;                        // chunk stride (elements)
     __host__ __device__ static int xs(int F) {                   // X / Y size (elements)
-        const int a = F * sf_fft_fastest(N, F), b = (F / W) * CS;
+        const int a = F * sf_fft_fastest(N, F), b = (F / WC) * CS;
         return a > b ? a : b;
     }
     __host__ __device__ static size_t bytes(int F) {
-        return 128 + sizeof(cplx<T>) * ((size_t)twiddle_elems<N>() + (size_t)(F / W) * CS + 2 * (size_t)xs(F));
+        return 128 + sizeof(cplx<T>) * ((size_t)twiddle_elems<N>() + (size_t)(F / WC) * CS + 2 * (size_t)xs(F));
     }
     // the adjoint instantiation also stages COL_ADJ_BA's second product (Z, after Y)
-    __host__ __device__ static size_t bytes_adj(int F) { return bytes(F) + sizeof(cplx<T>) * (size_t)(F / W) * CS; }
+    __host__ __device__ static size_t bytes_adj(int F) { return bytes(F) + sizeof(cplx<T>) * (size_t)(F / WC) * CS; }
 };
 
-template <typename T, int N, int EMAX, bool ADJ>
+template <typename T, int N, int EMAX, bool ADJ, int WC = W>
 __global__ void __launch_bounds__(512, (N >= 512 || ADJ) ? 1 : 2) k_col(const ColArgs<T> a) {
     using C = cplx<T>;
-    using L = ColSmem<T, N>;
+    using L = ColSmem<T, N, WC>;
+    static_assert(WC == W || (WC == 1 && !ADJ), "whole tiles or single columns");
+    constexpr int LOGWC = ilog2(WC), SUB = W / WC;                    // chunks of one tile
+    constexpr bool BULK = WC == W;                                    // a chunk is contiguous in global memory
     constexpr int TPF = FftShape<N, EMAX>::TPF;
     constexpr int CS = L::CS;
-    constexpr int LOGNW = FftShape<N, EMAX>::LOG + 2;                 // log2(N W)
+    constexpr int LOGNW = FftShape<N, EMAX>::LOG + LOGWC;             // log2(N WC)
     extern __shared__ __align__(128) unsigned char smem_raw[];
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw);
     const int F = a.F;                                           // a power of two, multiple of W
     const int logF = __ffs(F) - 1;
-    const int nchunks = F / W, lognch = logF - 2;
+    const int nchunks = F / WC, lognch = logF - LOGWC;
+    // tiles of WC columns, as every "tile" below (single columns: without the padding of the last tile)
+    const int n_tiles = BULK ? a.n_tiles : min(a.n_tiles * SUB, a.sp.hx);
     const int SF = sf_fft_fastest(N, F);
     C *TW = reinterpret_cast<C *>(smem_raw + 128);             // roots of unity of length N
     C *PHI = TW + twiddle_elems<N>();
@@ -413,22 +479,28 @@ __global__ void __launch_bounds__(512, (N >= 512 || ADJ) ? 1 : 2) k_col(const Co
     const int t = threadIdx.x, nthr = blockDim.x;
     const int op = blockIdx.y;
     const int opp = (sp.n_outer - op) & (sp.n_outer - 1);        // partner pencil (-ky)
+    // single columns: a pencil that is its own partner is transformed once (its
+    // second chunk idles); whole tiles compute it twice
+    const bool lone = !BULK && logNP && opp == op;
     const int mode = a.mode;
     const int first_tile = blockIdx.x * a.tiles_per_cta;
     const C *__restrict__ tw = TW;
 
     auto chunk_tile = [&](int ch) { return first_tile + (ch >> logNP); };
     auto chunk_o = [&](int ch) { return (ch & logNP) ? opp : op; };
-    auto chunk_ok = [&](int ch) { return chunk_tile(ch) < a.n_tiles; };
+    auto chunk_ok = [&](int ch) { return chunk_tile(ch) < n_tiles; };
     auto chunk_writes = [&](int ch) { return chunk_ok(ch) && !((ch & logNP) && opp == op); };
-    auto gofs = [&](int ch) { return ((size_t)(chunk_tile(ch) * sp.n_outer + chunk_o(ch)) * N) * W; };
+    auto gofs = [&](int ch) {
+        const int tile = chunk_tile(ch);
+        return ((size_t)((tile / SUB) * sp.n_outer + chunk_o(ch)) * N) * W + (tile & (SUB - 1)) * WC;
+    };
 
     // ---- stage: state chunks -> PHI (not for COL_FWD), product chunks -> X (COL_STEP, COL_FWD)
     constexpr bool adj = ADJ;   // the adjoint modes are a separate instantiation
     const bool need_in = mode == COL_STEP || mode == COL_FWD || adj;
     const bool need_phi = mode != COL_FWD;
     const bool need_in2 = adj && mode == COL_ADJ_BA;
-    const uint32_t chunk_bytes = (uint32_t)(N * W * sizeof(C));
+    const uint32_t chunk_bytes = BULK ? (uint32_t)(N * W * sizeof(C)) : 0u;
     int nvalid = 0;                                              // chunks 0..nvalid-1 lie inside the grid
     for (int ch = 0; ch < nchunks; ++ch) nvalid += chunk_ok(ch) ? 1 : 0;
     pdl_wait();
@@ -441,7 +513,7 @@ __global__ void __launch_bounds__(512, (N >= 512 || ADJ) ? 1 : 2) k_col(const Co
         mbar_expect_tx(bar, chunk_bytes * nvalid * ((need_in ? 1 : 0) + (need_phi ? 1 : 0) + (need_in2 ? 1 : 0)) +
                                 twiddle_bytes<C, N>() + extra);
         if (twiddle_bytes<C, N>()) bulk_g2s(TW, a.tw + twiddle_offset(N, EMAX), twiddle_bytes<C, N>(), bar);
-        for (int ch = 0; ch < nvalid; ++ch) {
+        for (int ch = 0; BULK && ch < nvalid; ++ch) {
             if (need_phi) bulk_g2s(PHI + ch * CS, a.state + sofs + gofs(ch), chunk_bytes, bar);
             if (need_in) bulk_g2s(X + ch * CS, a.in + sofs + gofs(ch), chunk_bytes, bar);
             if (need_in2) bulk_g2s(Z + ch * CS, a.in2 + sofs + gofs(ch), chunk_bytes, bar);
@@ -452,8 +524,16 @@ __global__ void __launch_bounds__(512, (N >= 512 || ADJ) ? 1 : 2) k_col(const Co
         reinterpret_cast<uint32_t *>(&sfp)[i] = reinterpret_cast<const uint32_t *>(&a.fps[slot])[i];
     if (t == 0) sstep = (uint32_t)(*a.d_step);
     __syncthreads();   // the barrier is initialised before anyone polls it
-    for (int i = nvalid * (N * W) + t; i < nchunks * (N * W); i += nthr) {   // chunks past the last tile read as zero
-        const int ch = i >> LOGNW, r = i & (N * W - 1);
+    if constexpr (!BULK) {
+        for (int i = t; i < nvalid * (N * WC); i += nthr) {
+            const int ch = i >> LOGNW, r = i & (N * WC - 1);
+            const size_t g = sofs + gofs(ch) + (size_t)(r >> LOGWC) * W + (r & (WC - 1));
+            if (need_phi) PHI[ch * CS + r] = a.state[g];
+            if (need_in) X[ch * CS + r] = a.in[g];
+        }
+    }
+    for (int i = nvalid * (N * WC) + t; i < nchunks * (N * WC); i += nthr) {   // chunks past the last tile read as zero
+        const int ch = i >> LOGNW, r = i & (N * WC - 1);
         PHI[ch * CS + r] = mk<T>(0, 0);
         X[ch * CS + r] = mk<T>(0, 0);
         if (need_in2) Z[ch * CS + r] = mk<T>(0, 0);
@@ -462,15 +542,15 @@ __global__ void __launch_bounds__(512, (N >= 512 || ADJ) ? 1 : 2) k_col(const Co
 
     // this thread's FFT: column c of chunk ch
     const int f = t & (F - 1), lane = t >> logF;
-    const bool active = lane < TPF;
-    const int ch = f >> 2, c = f & 3;
+    const int ch = f >> LOGWC, c = f & (WC - 1);
+    const bool active = lane < TPF && !(lone && (ch & 1));
     const int my_tile = chunk_tile(ch), my_o = chunk_o(ch);
-    const int kx = my_tile * W + c;
+    const int kx = my_tile * WC + c;
 
     if (need_in) {
         // forward transform along this axis: P_q (the staged chunk is [pos][W],
         // or [W][pos] for a column-major input)
-        const int xstride = a.in_colmajor ? 1 : W;
+        const int xstride = a.in_colmajor ? 1 : WC;
         const C *xb = X + ch * CS + (a.in_colmajor ? c * N : c);
         int which = 0;
         if (!ADJ && mode == COL_STEP && fp.spectral) {
@@ -480,7 +560,7 @@ __global__ void __launch_bounds__(512, (N >= 512 || ADJ) ? 1 : 2) k_col(const Co
 #pragma unroll 1
             for (int i = t; i < N * F; i += nthr) {
                 const int ff = i & (F - 1), pos = i >> logF;
-                Y[ff * SF + spad(pos)] = X[(ff >> 2) * CS + pos * W + (ff & 3)];
+                Y[ff * SF + spad(pos)] = X[(ff >> LOGWC) * CS + pos * WC + (ff & (WC - 1))];
             }
         } else {
             which = fft_run<T, N, EMAX, -1>([&](int p) { return xb[p * xstride]; },
@@ -497,15 +577,16 @@ __global__ void __launch_bounds__(512, (N >= 512 || ADJ) ? 1 : 2) k_col(const Co
         const uint32_t step = sstep;
         // update: each thread keeps one pair of neighbouring columns (they share
         // one Philox draw) of one chunk and walks the positions
-        const int cp = t & 1, chq = (t >> 1) & (nchunks - 1);
-        const int pos_step = nthr >> (1 + lognch);
+        constexpr int LOGCP = WC == 1 ? 0 : LOGWC - 1;              // column pairs of a chunk
+        const int cp = t & ((1 << LOGCP) - 1), chq = (t >> LOGCP) & (nchunks - 1);
+        const int pos_step = nthr >> (LOGCP + lognch);
         const int tile = chunk_tile(chq), o = chunk_o(chq);
-        const int c0 = 2 * cp, kx0 = tile * W + c0;
+        const int c0 = 2 * cp, kx0 = tile * WC + c0;
         const bool has0 = kx0 < sp.hx, has1 = kx0 + 1 < sp.hx;
         const bool on_plane = kx0 == 0 || 2 * kx0 == sp.nx;
         const T qx0 = T(kx0) * sp.gx, qx1 = T(kx0 + 1) * sp.gx;
         const T qx0s = qx0 * qx0, qx1s = qx1 * qx1;
-        const C *P0 = P + (chq * W + c0) * SF, *P1 = P0 + SF;
+        const C *P0 = P + (chq * WC + c0) * SF, *P1 = P0 + (WC == 1 ? 0 : SF);   // (one column: P1 is not used)
         C *phb = PHI + chq * CS + c0;
         bool bad = false;
         T dtO[kPolyTerms], dtM[kPolyTerms];
@@ -514,29 +595,70 @@ __global__ void __launch_bounds__(512, (N >= 512 || ADJ) ? 1 : 2) k_col(const Co
             dtO[i] = sp.dt * fp.O[i];
             dtM[i] = sp.dt * fp.M[i];
         }
+        // operators of degree 2 in q^2 (Models A and B) take the short polynomials
+        const bool low = dtO[3] == T(0) && dtO[4] == T(0) && dtM[3] == T(0) && dtM[4] == T(0);
+        // q^2 of the axis of this kernel's transform, and of the other one (y in 3D)
+        const T gpos = sp.dim == 3 ? sp.gz : (sp.dim == 2 ? sp.gy : T(0));
+        const T qo = sp.dim == 3 ? T(signed_k(o, sp.ny)) * sp.gy : T(0), qo2 = qo * qo;
         const bool has_product = fp.power > 0, noisy = fp.noisy != 0;
         const int noise_pow = fp.noise_pow, fid = fp.field_id;
         const T sigma0 = fp.sigma0;
         const PhiloxKey key = philox_key(fp.seed_lo, fp.seed_hi);
-        if (tile < a.n_tiles) {
+        if (tile < n_tiles && !(lone && (chq & 1))) {
 #pragma unroll 1
-            for (int pos = t >> (1 + lognch); pos < N; pos += pos_step) {
+            for (int pos = t >> (LOGCP + lognch); pos < N; pos += pos_step) {
+                if constexpr (WC == 1) {
+                    // one column: the mode's own half of its pair's draw
+                    C v = P0[spad(pos)];
+                    C *ph = phb + pos;
+                    if (mode == COL_STEP) {
+                        const int ky = sp.dim == 3 ? o : (sp.dim == 2 ? pos : 0);
+                        const int kz = sp.dim == 3 ? pos : 0;
+                        const T qp = T(signed_k(pos, N)) * gpos;
+                        const T q2 = qx0s + (qp * qp + qo2);
+                        C xi = mk<T>(0, 0);
+                        if (noisy)
+                            xi = noise_one<T>(on_plane, kx0, ky, kz, sigma0, noise_pow, q2, sp, (uint32_t)fid, key, step,
+                                              a.tw);
+                        T m, g;
+                        if (low) {
+                            m = ffma(ffma(dtM[2], q2, dtM[1]), q2, dtM[0]);
+                            g = fast_rcp(fadd(T(1), ffma(ffma(dtO[2], q2, dtO[1]), q2, dtO[0])));
+                        } else {
+                            update_factors<T>(q2, dtO, dtM, m, g);
+                        }
+                        v = update_pre<T>(*ph, v, xi, m, g, has_product);
+                        bad |= !finite_mode(v);
+                    }
+                    *ph = has0 ? v : mk<T>(0, 0);
+                    continue;
+                }
                 C v0 = P0[spad(pos)], v1 = P1[spad(pos)];
-                C *ph = phb + pos * W;
+                C *ph = phb + pos * WC;
                 if (mode == COL_STEP) {
                     C f0, f1;
                     ld_pair<T>(ph, f0, f1);
                     const int ky = sp.dim == 3 ? o : (sp.dim == 2 ? pos : 0);
                     const int kz = sp.dim == 3 ? pos : 0;
-                    const T qy = T(signed_k(ky, sp.ny)) * sp.gy, qz = T(signed_k(kz, sp.nz)) * sp.gz;
-                    const T qyz2 = qy * qy + qz * qz;
+                    const T qp = T(signed_k(pos, N)) * gpos;
+                    const T qyz2 = qp * qp + qo2;
                     const T q2a = qx0s + qyz2, q2b = qx1s + qyz2;
                     C xi0 = mk<T>(0, 0), xi1 = mk<T>(0, 0);
                     if (noisy)
                         noise_pair<T>(on_plane, kx0, ky, kz, sigma0, noise_pow, q2a, q2b, has1, sp, (uint32_t)fid, key,
-                                      step, xi0, xi1);
-                    v0 = update_mode<T>(f0, v0, xi0, q2a, dtO, dtM, has_product);
-                    v1 = update_mode<T>(f1, v1, xi1, q2b, dtO, dtM, has_product);
+                                      step, xi0, xi1, a.tw);
+                    T m0, g0, m1, g1;
+                    if (low) {
+                        m0 = ffma(ffma(dtM[2], q2a, dtM[1]), q2a, dtM[0]);
+                        m1 = ffma(ffma(dtM[2], q2b, dtM[1]), q2b, dtM[0]);
+                        g0 = fast_rcp(fadd(T(1), ffma(ffma(dtO[2], q2a, dtO[1]), q2a, dtO[0])));
+                        g1 = fast_rcp(fadd(T(1), ffma(ffma(dtO[2], q2b, dtO[1]), q2b, dtO[0])));
+                    } else {
+                        update_factors<T>(q2a, dtO, dtM, m0, g0);
+                        update_factors<T>(q2b, dtO, dtM, m1, g1);
+                    }
+                    v0 = update_pre<T>(f0, v0, xi0, m0, g0, has_product);
+                    v1 = update_pre<T>(f1, v1, xi1, m1, g1, has_product);
                     // false for NaN and for infinities (or values next to overflow)
                     bad |= !(fabs(v0.x) + fabs(v0.y) + fabs(v1.x) + fabs(v1.y) <= T(sizeof(T) == 4 ? 3.0e38 : 1.0e300));
                 }
@@ -554,8 +676,8 @@ __global__ void __launch_bounds__(512, (N >= 512 || ADJ) ? 1 : 2) k_col(const Co
         if (first_tile == 0) ++npl;
         {
             const int kh = sp.nx / 2, last_tile = first_tile + a.tiles_per_cta;
-            if (kh > 0 && first_tile * W <= kh && kh < last_tile * W) {
-                const int cqh = (kh / W - first_tile) << logNP, cch = kh & (W - 1);
+            if (kh > 0 && first_tile * WC <= kh && kh < last_tile * WC) {
+                const int cqh = (kh / WC - first_tile) << logNP, cch = kh & (WC - 1);
                 if (npl == 0) { pl_cq0 = cqh; pl_cc0 = cch; } else { pl_cq1 = cqh; pl_cc1 = cch; }
                 ++npl;
             }
@@ -567,9 +689,9 @@ __global__ void __launch_bounds__(512, (N >= 512 || ADJ) ? 1 : 2) k_col(const Co
                 const int j = i >> LOGN, pos = i & (N - 1);
                 const int cq = j ? pl_cq1 : pl_cq0, cc = j ? pl_cc1 : pl_cc0;
                 const int ppos = (N - pos) & (N - 1);
-                if (logNP == 0 && ppos < pos) continue;
-                C *p0 = &PHI[cq * CS + pos * W + cc];
-                C *p1 = &PHI[(cq + logNP) * CS + ppos * W + cc];
+                if ((logNP == 0 || lone) && ppos < pos) continue;
+                C *p0 = &PHI[cq * CS + pos * WC + cc];
+                C *p1 = &PHI[(cq + (lone ? 0 : logNP)) * CS + ppos * WC + cc];
                 const C u0 = *p0, u1 = *p1;
                 const C h = mk<T>(T(0.5) * (u0.x + u1.x), T(0.5) * (u0.y - u1.y));
                 *p0 = h;
@@ -578,16 +700,23 @@ __global__ void __launch_bounds__(512, (N >= 512 || ADJ) ? 1 : 2) k_col(const Co
             __syncthreads();
         }
         // write the state back: one bulk copy per chunk (contiguous in global memory)
-        fence_proxy_async();   // every thread's PHI writes, before the copy engine reads them
+        if (BULK) fence_proxy_async();   // every thread's PHI writes, before the copy engine reads them
         __syncthreads();
-        if (t == 0) {
+        if constexpr (!BULK) {
+            cplx<T> *sdst = a.state_out ? a.state_out : a.state;
+            for (int i = t; i < nvalid * (N * WC); i += nthr) {
+                const int cq = i >> LOGNW, r = i & (N * WC - 1);
+                if (chunk_writes(cq))
+                    sdst[sofs + gofs(cq) + (size_t)(r >> LOGWC) * W + (r & (WC - 1))] = PHI[cq * CS + r];
+            }
+        } else if (t == 0) {
             cplx<T> *sdst = a.state_out ? a.state_out : a.state;
             for (int cq = 0; cq < nvalid; ++cq)
                 if (chunk_writes(cq)) bulk_s2g(sdst + sofs + gofs(cq), PHI + cq * CS, chunk_bytes);
             bulk_commit();
         }
         if (mode == COL_FWD) {
-            if (t == 0) bulk_wait_read();
+            if (BULK && t == 0) bulk_wait_read();
             return;
         }
     }
@@ -598,7 +727,7 @@ __global__ void __launch_bounds__(512, (N >= 512 || ADJ) ? 1 : 2) k_col(const Co
     bool skip = false;
     if (!full) {
         const bool ky_kept = sp.dim != 3 || abs(signed_k(op, sp.ny)) <= fp.kmax[1];
-        skip = first_tile * W > fp.kmax[0] || !ky_kept;              // CTA-uniform: nothing kept
+        skip = first_tile * WC > fp.kmax[0] || !ky_kept;              // CTA-uniform: nothing kept
     }
     if (!skip) {
         __syncthreads();   // PHI is final; X and Y are free
@@ -607,7 +736,7 @@ __global__ void __launch_bounds__(512, (N >= 512 || ADJ) ? 1 : 2) k_col(const Co
         const int kmax_pos = full ? N : (sp.dim == 3 ? fp.kmax[2] : (sp.dim == 2 ? fp.kmax[1] : 0));
         const T scale = (kx_keep && o_keep) ? sp.inv_nsites : T(0);
         const C *pb = PHI + ch * CS + c;
-        const bool writes = chunk_writes(ch) && (full || my_tile * W <= fp.kmax[0]);
+        const bool writes = chunk_writes(ch) && (full || my_tile * WC <= fp.kmax[0]);
         C *__restrict__ dst = a.out + sofs + gofs(ch) + c;
         // a product-term factor: op(q) = (i q_d) (-q^2)^l, q_d = 0 at a Nyquist index
         const T gpos = sp.dim == 3 ? sp.gz : sp.gy;
@@ -632,15 +761,15 @@ __global__ void __launch_bounds__(512, (N >= 512 || ADJ) ? 1 : 2) k_col(const Co
         if (a.op_on)
             fft_run<T, N, EMAX, +1>(
                 [&](int p) {
-                    return abs(signed_k(p, N)) <= kmax_pos ? op(p, cscale<T>(pb[p * W], scale)) : mk<T>(0, 0);
+                    return abs(signed_k(p, N)) <= kmax_pos ? op(p, cscale<T>(pb[p * WC], scale)) : mk<T>(0, 0);
                 },
                 sink, X + f * SF, Y + f * SF, lane, active, tw);
         else
             fft_run<T, N, EMAX, +1>(
-                [&](int p) { return abs(signed_k(p, N)) <= kmax_pos ? cscale<T>(pb[p * W], scale) : mk<T>(0, 0); },
+                [&](int p) { return abs(signed_k(p, N)) <= kmax_pos ? cscale<T>(pb[p * WC], scale) : mk<T>(0, 0); },
                 sink, X + f * SF, Y + f * SF, lane, active, tw);
     }
-    if (need_in && t == 0) bulk_wait_read();   // PHI must outlive the state write-back
+    if (BULK && need_in && t == 0) bulk_wait_read();   // PHI must outlive the state write-back
 }
 
 // ---------------------------------------------------------------------------
@@ -1118,9 +1247,22 @@ template <typename T, int N, int EMAX>
 cudaError_t launch_col_n(const ColArgs<T> &a, int nf, int gx, int gy, cudaStream_t st) {
     const int threads = col_threads(N, EMAX, a.F);
     const bool adj = a.mode == COL_ADJ_A || a.mode == COL_ADJ_B || a.mode == COL_ADJ_BA;
-    const size_t smem = a.mode == COL_ADJ_BA ? ColSmem<T, N>::bytes_adj(a.F) : ColSmem<T, N>::bytes(a.F);
-    if (a.F * FftShape<N, EMAX>::TPF > 512 || (a.F & (a.F - 1)) != 0 || a.F % W != 0)
+    if (a.F * FftShape<N, EMAX>::TPF > 512 || (a.F & (a.F - 1)) != 0 || a.F % a.wc != 0)
         return cudaErrorInvalidConfiguration;
+    if (a.wc != W) {
+        if constexpr (EMAX <= 4 && N >= 16) {
+            if (a.wc != 1 || adj || a.in_colmajor) return cudaErrorInvalidConfiguration;
+            const size_t smem = ColSmem<T, N, 1>::bytes(a.F);
+            // many CTAs (radix 4): every thread transforms, since warps that only
+            // join the update would leave their scheduler's FP64 unit idle meanwhile
+            const int ft = a.F * FftShape<N, EMAX>::TPF, threads = EMAX == 2 ? col_threads(N, EMAX, a.F) : ft < 32 ? 32 : ft;
+            cudaError_t e = ensure_smem(k_col<T, N, EMAX, false, 1>, smem);
+            if (e != cudaSuccess) return e;
+            return launch_pdl(k_col<T, N, EMAX, false, 1>, dim3(gx, gy, nf), threads, smem, st, a);
+        }
+        return cudaErrorInvalidConfiguration;
+    }
+    const size_t smem = a.mode == COL_ADJ_BA ? ColSmem<T, N>::bytes_adj(a.F) : ColSmem<T, N>::bytes(a.F);
     cudaError_t e = adj ? ensure_smem(k_col<T, N, EMAX, true>, smem) : ensure_smem(k_col<T, N, EMAX, false>, smem);
     if (e != cudaSuccess) return e;
     if (adj) return launch_pdl(k_col<T, N, EMAX, true>, dim3(gx, gy, nf), threads, smem, st, a);
