@@ -251,13 +251,15 @@ int pss_time_kernels(pss_system *s, int64_t n, double *avg_ms);
  *                 and row phases (1, default) or as two launches a step on
  *                 the "fast2d" kernels (0); the same bits at the same FFT
  *                 radix;
- *   "resident"    FP32 2D systems with sides of 32..512 and power products, at
- *                 least one side below 256 (or 256 x 256 batches that fill the
- *                 GPU), take a run of steps as one launch in which a cluster
- *                 of CTAs holds each slot on chip (1, default) or the kernels
- *                 pss_step_path names (0); they agree to FP32 rounding, and
- *                 the other launch-shape keys do not act on such a run;
- *                 "fast2d" 0 also turns it off;
+ *   "resident"    runs of steps as one launch with every slot's state on chip
+ *                 (1, default) or the kernels pss_step_path names (0): FP32 2D
+ *                 systems with sides of 32..512 and power products, at least
+ *                 one side below 256 (or 256 x 256 batches that fill the GPU),
+ *                 a cluster of CTAs per slot ("fast2d" 0 also turns these
+ *                 off); 1D systems of 64..1024 sites whose fields each have at
+ *                 most one explicit product, of one factor of the field
+ *                 itself, with or without boundary frames.  They agree to
+ *                 rounding; the other launch-shape keys do not act on them;
  *   "res_ctas"    CTAs per cluster of that launch (a power of two <= 16; 0:
  *                 automatic); the same bits whatever their number;
  *   "persist_blocks" CTAs of that launch (0: automatic, one per SM and at

@@ -538,6 +538,33 @@ bool resident2d(const pss_system *s) {
     }
     return s->res256_on;
 }
+// A run of steps of a 1D system of 64..1024 sites is one launch of one CTA per
+// slot (k_line) where every field's explicit part is one product of itself:
+// its power term, or one product term of one factor of the field (KPZ's
+// (d_x h)^2 is one).  Boundary frames included.
+bool line_field(const pss_system *s, int fi, GFactor *out) {
+    const Field &f = s->fields[fi];
+    *out = {fi, f.power, -1, 0};
+    if (!f.general) return true;
+    if (f.power != 0) return false;
+    int n = 0;
+    for (const GTerm &t : s->gterms)
+        if (t.target == fi) {
+            if (++n > 1 || t.factors.size() != 1 || t.factors[0].field != fi) return false;
+            *out = t.factors[0];
+        }
+    return n == 1;
+}
+bool line1d(const pss_system *s) {
+    if (!(s->tune_resident && s->dim == 1 && s->nx >= 64 && !s->tune_real_state && !s->tune_test_timeout)) return false;
+    GFactor f;
+    for (int i = 0; i < (int)s->fields.size(); ++i)
+        if (!line_field(s, i, &f)) return false;
+    return true;
+}
+// runs of steps as one launch that keeps the state on chip
+bool resident(const pss_system *s) { return line1d(s) || resident2d(s); }
+
 // CTAs per cluster: the most that still run every slot at once and leave a CTA
 // kResSitesPerCta sites (64^2 on 1 .. 16 CTAs: 4.3, 3.8, 3.1, 3.2, 3.7 us per
 // step; 128^2: 13.0, 8.3, 5.4, 4.3, 4.1), else the fewest that hold one slot
@@ -1242,7 +1269,7 @@ template <typename T> int step_once(pss_system *s, cudaStream_t st) {
 int launch_resident(pss_system *s, int nsteps, cudaStream_t st);
 
 int record_steps(pss_system *s, cudaStream_t st, int64_t n) {
-    if (resident2d(s)) {
+    if (resident(s)) {
         // (in a graph: a list with a system twice, recorded step by step)
         int rc = PSS_OK;
         for (int64_t k = 0; k < n && rc == PSS_OK; ++k) rc = launch_resident(s, 1, st);
@@ -1406,11 +1433,36 @@ int run_persist(pss_system *s, int64_t n, cudaStream_t st) {
     return PSS_OK;
 }
 
-// The cluster-resident path: one launch per run of at most kMaxPersistSteps
-// steps.  It reads and writes only the state and the step counter; the work
+// The resident paths (k_res2d, k_line): one launch per run of at most
+// kMaxPersistSteps steps.  It reads and writes only the state and the step counter; the work
 // arrays then hold nothing of the new state (stale), for the paths that use
 // them.
+template <typename T> int launch_line_run(pss_system *s, int nsteps, cudaStream_t st) {
+    LineArgs<T> a{};
+    a.sp = sys_params<T>(s);
+    a.fps = (const FieldP<T> *)s->fps;
+    a.state = (cplx<T> *)s->state;
+    a.slot_stride = s->field_elems;
+    a.tw = (const cplx<T> *)s->tw;
+    a.d_step = s->d_step;
+    a.d_status = s->d_status;
+    a.gs = s->gs;
+    a.nsteps = nsteps;
+    a.nf = (int)s->fields.size();
+    for (int i = 0; i < a.nf; ++i) {
+        GFactor f;
+        line_field(s, i, &f);
+        const Field &fd = s->fields[i];
+        a.fld[i] = {f.power, f.deriv, f.lap, fd.frame_w, T(fd.frame_lo), T(fd.frame_hi)};
+    }
+    cudaError_t e = launch_line<T>(a, s->nslots(), st);
+    s->launches++;
+    if (e != cudaSuccess) return cuda_fail(s, e, "k_line launch");
+    return PSS_OK;
+}
+
 int launch_resident(pss_system *s, int nsteps, cudaStream_t st) {
+    if (s->dim == 1) return s->prec == PSS_F64 ? launch_line_run<double>(s, nsteps, st) : launch_line_run<float>(s, nsteps, st);
     Res2Args a{};
     a.sp = sys_params<float>(s);
     a.fps = (const FieldP<float> *)s->fps;
@@ -1481,7 +1533,7 @@ int join_resident(pss_system *s0, const std::vector<pss_system *> &res) {
 // and kept), so that the launches per step do not depend on n.
 int run_steps(pss_system *s, int64_t n) {
     if (persist2d(s)) return run_persist(s, n, s->stream);
-    if (resident2d(s)) return run_resident(s, n, s->stream);
+    if (resident(s)) return run_resident(s, n, s->stream);
     const int chunk = s->tune_graph_steps > 0 ? s->tune_graph_steps : kDefaultGraphSteps;
     if (!s->graph_valid) {
         drop_graphs(s);
@@ -2164,8 +2216,10 @@ int pss_step(pss_system *s, int64_t n) {
     if (n == 0) return PSS_OK;
     int rc = upload_params(s);
     if (rc) return rc;
-    if (round_trip(s) && (rc = ensure_real(s))) return rc;
-    if (!resident2d(s) && (rc = prologue(s, persist2d(s)))) return rc;
+    if (!resident(s)) {
+        if (round_trip(s) && (rc = ensure_real(s))) return rc;
+        if ((rc = prologue(s, persist2d(s)))) return rc;
+    }
     if ((rc = run_steps(s, n))) return rc;
     s->step += n;
     return PSS_OK;
@@ -2184,8 +2238,8 @@ int pss_step_many(pss_system **systems, int n, int64_t steps) {
             if (rc) return fail(s0, rc, "%s", s->err.c_str());
         }
         int rc = upload_params(s);
-        if (!rc && round_trip(s)) rc = ensure_real(s);
-        if (!rc && !resident2d(s)) rc = prologue(s);
+        if (!rc && round_trip(s) && !resident(s)) rc = ensure_real(s);
+        if (!rc && !resident(s)) rc = prologue(s);
         if (rc) return i == 0 ? rc : fail(s0, rc, "%s", s->err.c_str());
     }
     if (steps == 0) return PSS_OK;
@@ -2196,7 +2250,7 @@ int pss_step_many(pss_system **systems, int n, int64_t steps) {
     bool twice = false;
     for (int i = 0; i < n; ++i)
         for (int j = 0; j < i; ++j) twice |= systems[i] == systems[j];
-    for (int i = 0; i < n; ++i) (!twice && resident2d(systems[i]) ? res : rest).push_back(systems[i]);
+    for (int i = 0; i < n; ++i) (!twice && resident(systems[i]) ? res : rest).push_back(systems[i]);
     if (int rc = run_resident_beside(s0, res, !rest.empty(), steps)) return rc;
     pss_system **all = systems;
     const int n_all = n;
@@ -2248,7 +2302,7 @@ int pss_step_many(pss_system **systems, int n, int64_t steps) {
     if (int rc = join_resident(s0, res)) return rc;
     for (int i = 0; i < n_all; ++i) {
         all[i]->step += steps;
-        if (resident2d(all[i])) all[i]->stale = true;
+        if (resident(all[i])) all[i]->stale = true;
     }
     return PSS_OK;
 }

@@ -236,6 +236,19 @@ __device__ __forceinline__ void stockham_pass(Src src, Dst dst, int logP, int la
         cplx<T> u[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) u[r] = src(i + r * STRIDE);
+        if constexpr (R == 2 && sizeof(T) == 8) {
+            // FP64 radix 2: u0 +- w u1 in fused multiply-adds (the same operations,
+            // two roundings a component and the shorter chain)
+            if (P > 1) {
+                cplx<T> w = tw[P - FftShape<N, EMAX>::E + k];
+                if (DIR > 0) w.y = -w.y;
+                const cplx<T> x = u[0], y = u[1];
+                const int j = ((i - k) << LOGR) + k;
+                dst(j, mk<T>(ffma(w.x, y.x, ffma(-w.y, y.y, x.x)), ffma(w.x, y.y, ffma(w.y, y.x, x.y))));
+                dst(j + P, mk<T>(ffma(-w.x, y.x, ffma(w.y, y.y, x.x)), ffma(-w.x, y.y, ffma(-w.y, y.x, x.y))));
+                continue;
+            }
+        }
         if (P > 1) {
             // this pass's twiddles exp(-2 pi i r k / (P R)), stored [r - 1][k] from
             // entry P - E on; consecutive lanes read consecutive entries

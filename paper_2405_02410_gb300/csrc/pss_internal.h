@@ -293,8 +293,29 @@ struct Res2Args {
     int nsteps;
     int C;                      // CTAs per cluster, a power of two
 };
-// Values per thread of a transform of n points there, the points of shared
-// memory it takes, and a CTA's dynamic shared memory (C CTAs per cluster)
+// A run of steps of a 1D system (k_line: 64..1024 sites), one CTA per slot.
+// Per field: its explicit term M(q) F[(F^-1[op(q) m phi])^power] (power 0:
+// none; op as in ColArgs), and its boundary frame.
+template <typename T> struct LineField {
+    int power, deriv, lap, frame_w;
+    T frame_lo, frame_hi;
+};
+template <typename T> struct LineArgs {
+    SysP<T> sp;
+    const FieldP<T> *fps;
+    cplx<T> *state;
+    size_t slot_stride;
+    const cplx<T> *tw;
+    long long *d_step;
+    int *d_status;
+    GridSync *gs;               // done: CTAs finished (the last one advances *d_step)
+    int nsteps, nf;
+    LineField<T> fld[kMaxFields];
+};
+template <typename T> cudaError_t launch_line(const LineArgs<T> &a, int nslots, cudaStream_t st);
+
+// Values per thread of k_res2d's transforms of n points, the points of shared
+// memory one takes, and a CTA's dynamic shared memory (C CTAs per cluster)
 __host__ __device__ constexpr int res_e(int n) { return n <= PSS_RES_E8 ? 8 : 16; }
 __host__ __device__ constexpr int res_xld(int n) { return n + res_e(n) + 2; }
 __host__ __device__ constexpr size_t res2_smem_bytes(int nx, int ny, int C) {
