@@ -49,9 +49,11 @@ __device__ __forceinline__ int signed_k(int k, int n) { return k < (n + 1) / 2 ?
 __device__ __forceinline__ float2 noise_mode(uint32_t w0, uint32_t w1, float sigma0, int p, float q2) {
     const float u0 = ffma(float(w0 >> 8), 5.9604644775390625e-08f, 2.98023223876953125e-08f);
     const float u1 = ffma(float(w1 >> 8), 5.9604644775390625e-08f, 2.98023223876953125e-08f);
-    const float L = fmul(fmul(-2.0f, __logf(u0)), (p & 1) ? q2 : 1.0f);
-    float amp = sigma0;
-    if (p >= 2) amp = fmul(amp, p >= 4 ? fmul(q2, q2) : q2);   // p is 0 .. 4
+    float L = fmul(-2.0f, __logf(u0)), amp = sigma0;
+    if (p != 0) {                                              // p is 0 .. 4
+        if (p & 1) L = fmul(L, q2);
+        if (p >= 2) amp = fmul(amp, p >= 4 ? fmul(q2, q2) : q2);
+    }
     const float r = fmul(root_approx(L), amp);
     float s, c;
     __sincosf(fmul(6.283185307179586f, u1), &s, &c);
@@ -129,10 +131,7 @@ __device__ __forceinline__ void noise_pair(bool on_plane, int kx0, int ky, int k
     }
     u32x4 r = philox4x32_10(u32x4{(crow * (uint32_t)sp.hxe + (uint32_t)kx0) >> 1, step, fid, 0u}, key);
     xi0 = noise_mode(r.x, r.y, sigma0, npow, q2a, tw);
-    if (on_plane) {
-        if (cj) xi0.y = -xi0.y;
-        if (selfc) xi0 = mk<T>(T(1.4142135623730951) * xi0.x, T(0));
-    }
+    xi0 = selfc ? mk<T>(T(1.4142135623730951) * xi0.x, T(0)) : mk<T>(xi0.x, cj ? -xi0.y : xi0.y);
     if (has1) {
         // kx1 is odd, so it is never 0 or Nx/2: it is its own canonical member
         if (crow != row)
