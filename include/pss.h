@@ -260,6 +260,11 @@ int pss_time_kernels(pss_system *s, int64_t n, double *avg_ms);
  *                 most one explicit product, of one factor of the field
  *                 itself, with or without boundary frames.  They agree to
  *                 rounding; the other launch-shape keys do not act on them;
+ *   "fuse_terms"  FP32 1D and 2D systems with product terms whose terms of one
+ *                 field share an operator (or whose operators are multiples of
+ *                 one power of q^2), with at most 6 distinct factors, evaluate
+ *                 them in one row kernel per step (1, default) or factor by
+ *                 factor (0); they agree to FP32 rounding;
  *   "res_ctas"    CTAs per cluster of that launch (a power of two <= 16; 0:
  *                 automatic); the same bits whatever their number;
  *   "persist_blocks" CTAs of that launch (0: automatic, one per SM and at

@@ -17,6 +17,7 @@
 #include <cstdio>
 #include <cstring>
 #include <atomic>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <type_traits>
@@ -67,6 +68,8 @@ constexpr double kPi = 3.14159265358979323846;
 
 }  // namespace
 
+namespace { struct TermPlan; }
+
 struct pss_system {
     int dim = 0, nx = 1, ny = 1, nz = 1;
     double dx[3] = {1, 1, 1};
@@ -92,6 +95,12 @@ struct pss_system {
     void *tw = nullptr;                      // roots of unity, precision of the system
     void *real = nullptr;                    // real scratch [nz][ny][nx] (one slot)
     void *GS = nullptr;                      // product terms: factor / product spectrum [slot][field_elems]
+    void *term_extra = nullptr;              // fused product terms: further y-inverses [extra][slot][field_elems]
+    size_t term_extra_bytes = 0;
+    float *term_coef = nullptr;              // their real-space coefficients [slot][kMaxTerms]
+    int coef_slots = 0;
+    mutable std::shared_ptr<TermPlan> plan;  // made for generation plan_gen
+    mutable uint64_t plan_gen = 0;
     void *real_acc = nullptr;                // product terms: sum of the products in real space (one slot)
     void *real_tp = nullptr;                 // product terms: running product of one term (one slot)
     void *half = nullptr;                    // half-spectrum scratch (one slot)
@@ -136,6 +145,7 @@ struct pss_system {
     int tune_adj_col2 = 1;
     int tune_adj_radix = 0;                  // FFT radix of that backward pass (8 or 16; 0: the forward's)
     int tune_persist_adj = 1;                // FP32 2D adjoint on the persistent path: a segment's backward pass in one launch                   // FP32 2D adjoint: column parts on FFT groups (0: generic kernel)
+    int tune_fuse_terms = 1;                 // FP32 1D/2D product terms in one row kernel (0: factor by factor)
     int tune_resident = 1;                   // FP32 2D sides of 32..512: a run of steps with every slot in one cluster
     int tune_res_ctas = 0;                   // its CTAs per cluster (0 = automatic)
     int res_ctas_auto = 0, res_ctas_slots = 0;   // the automatic choice, for that many slots
@@ -275,6 +285,74 @@ std::vector<std::vector<GTerm>> term_groups(const pss_system *s, int fi) {
     return groups;
 }
 
+// The product terms of an FP32 1D or 2D system as one row kernel (k_row_terms),
+// where each field's terms need one forward transform: they share one
+// operator, or every operator is a multiple of the same power of q^2 (the
+// multiples go into real space, M(q) keeps the power).
+struct TermPlan {
+    bool ok = false;
+    TermProg prog{};
+    struct Extra { int field, dy, lap; };
+    std::vector<Extra> extras;               // y-inverses beyond the plain ones
+    int common_pow[kMaxFields];              // the shared power of q^2 (-1: one operator, as it is)
+    std::vector<std::vector<Mono>> coef[kMaxFields];   // per term: the monomials whose sum is its coefficient (empty: 1)
+};
+TermPlan make_term_plan(const pss_system *s) {
+    TermPlan pl;
+    if (s->prec != PSS_F32 || s->dim > 2 || !any_general(s) || !s->tune_fuse_terms) return pl;
+    for (int fi = 0; fi < (int)s->fields.size(); ++fi) {
+        const auto groups = term_groups(s, fi);
+        pl.common_pow[fi] = -1;
+        if (groups.size() > 1) {
+            int pw = groups[0][0].M[0].pow;
+            for (const auto &g : groups)
+                for (const Mono &m : g[0].M)
+                    if (m.pow != pw) return pl;
+            pl.common_pow[fi] = pw;
+        }
+        for (const auto &g : groups)
+            for (const GTerm &t : g) {
+                int &n = pl.prog.nterm[fi];
+                if (n >= kMaxTerms || (int)t.factors.size() > kMaxTermProduct) return pl;
+                TermP &tp = pl.prog.term[fi][n++];
+                pl.coef[fi].push_back(groups.size() > 1 ? t.M : std::vector<Mono>{});
+                tp.n = (int)t.factors.size();
+                for (int k = 0; k < tp.n; ++k) {
+                    const GFactor &f = t.factors[k];
+                    const int dx = f.deriv == 0, dy = f.deriv == 1;
+                    int arr = -1;
+                    if (dy || f.lap > 0) {
+                        for (size_t e = 0; e < pl.extras.size(); ++e)
+                            if (pl.extras[e].field == f.field && pl.extras[e].dy == dy && pl.extras[e].lap == f.lap) arr = (int)e;
+                        if (arr < 0) { arr = (int)pl.extras.size(); pl.extras.push_back({f.field, dy, f.lap}); }
+                    }
+                    int c = -1;
+                    for (int i = 0; i < pl.prog.nfac; ++i)
+                        if (pl.prog.fac[i].field == f.field && pl.prog.fac[i].arr == arr && pl.prog.fac[i].dx == dx) c = i;
+                    if (c < 0) {
+                        if (pl.prog.nfac >= kMaxTermFactors) return pl;
+                        c = pl.prog.nfac++;
+                        pl.prog.fac[c] = {f.field, arr, dx};
+                    }
+                    tp.fac[k] = c;
+                    tp.power[k] = f.power;
+                }
+            }
+    }
+    // an extra array per y-inverse, of every slot
+    pl.ok = pl.prog.nfac > 0 && pl.extras.size() <= 4;
+    return pl;
+}
+// (made once per change of the terms: graphs, parameters and buffers follow it)
+const TermPlan &term_plan(const pss_system *s) {
+    if (!s->plan || s->plan_gen != s->gen) {
+        s->plan = std::make_shared<TermPlan>(make_term_plan(s));
+        s->plan_gen = s->gen;
+    }
+    return *s->plan;
+}
+bool fused_terms(const pss_system *s) { return any_general(s) && term_plan(s).ok; }
+
 template <typename T> FieldP<T> field_params(const pss_system *s, int inst, int fi) {
     const Field &f = s->fields[fi];
     FieldP<T> p{};
@@ -282,7 +360,10 @@ template <typename T> FieldP<T> field_params(const pss_system *s, int inst, int 
     for (const Mono &m : f.lhs) O[m.pow] += m.scale * pval(s, inst, m.param);
     p.power = f.power;
     p.spectral = 0;
-    if (f.general) {
+    if (f.general && fused_terms(s) && term_plan(s).common_pow[fi] >= 0) {
+        p.power = 1;
+        M[term_plan(s).common_pow[fi]] = 1.0;
+    } else if (f.general) {
         // one operator: the column kernel applies it after its own transform;
         // several: the products arrive summed in Fourier space with theirs
         const auto groups = term_groups(s, fi);
@@ -320,6 +401,27 @@ template <typename T> int upload_params_t(pss_system *s) {
     h.reserve(s->nslots());
     for (int b = 0; b < s->batch; ++b)
         for (int fi = 0; fi < (int)s->fields.size(); ++fi) h.push_back(field_params<T>(s, b, fi));
+    if (std::is_same<T, float>::value && fused_terms(s)) {
+        // the coefficients of the terms' sums in real space, [slot][kMaxTerms]
+        const TermPlan &pl = term_plan(s);
+        std::vector<float> c((size_t)s->nslots() * kMaxTerms, 1.0f);
+        for (int b = 0; b < s->batch; ++b)
+            for (int fi = 0; fi < (int)s->fields.size(); ++fi)
+                for (size_t i = 0; i < pl.coef[fi].size(); ++i)
+                    if (!pl.coef[fi][i].empty()) {
+                        double v = 0.0;
+                        for (const Mono &m : pl.coef[fi][i]) v += m.scale * pval(s, b, m.param);
+                        c[((size_t)b * s->fields.size() + fi) * kMaxTerms + i] = (float)v;
+                    }
+        if (s->coef_slots != s->nslots()) {
+            cudaFree(s->term_coef);
+            s->term_coef = nullptr;
+            s->coef_slots = 0;
+            CK(cudaMalloc(&s->term_coef, sizeof(float) * c.size()));
+            s->coef_slots = s->nslots();
+        }
+        CK(cudaMemcpyAsync(s->term_coef, c.data(), sizeof(float) * c.size(), cudaMemcpyHostToDevice, s->stream));
+    }
     if (!h.empty()) CK(cudaMemcpyAsync(s->fps, h.data(), sizeof(FieldP<T>) * h.size(), cudaMemcpyHostToDevice, s->stream));
     s->fps_dirty = false;
     return PSS_OK;
@@ -415,6 +517,17 @@ int row_G(const pss_system *s) {
         return G;
     }
     while (G * 2 * tpf <= 128 && G * 2 <= want) G *= 2;
+    return G;
+}
+
+// Row pairs per CTA of the product terms' row kernel: whole warps, up to 128
+// threads where every SM keeps a CTA, within shared memory
+int terms_G(const pss_system *s) {
+    const int tpf = fft_TPF(s->nx, 8), pairs = (s->rows + 1) / 2, nfac = term_plan(s).prog.nfac;
+    auto bytes = [&](int G) { return sizeof(float2) * ((size_t)s->nx + (size_t)G * (2 * sf_row_h(s->nx) + (size_t)nfac * s->nx)); };
+    int G = 1;
+    while (G * tpf < 32 && G * 2 <= pairs) G *= 2;
+    while (G * 2 * tpf <= 128 && (long long)pairs / (2 * G) * s->batch >= s->num_sms && bytes(2 * G) <= 100 * 1024) G *= 2;
     return G;
 }
 
@@ -1042,9 +1155,55 @@ template <typename T> struct Seq {
         return PSS_OK;
     }
 
+    // A (the plain y-inverses of every slot) -> B: all product terms of every
+    // instance, after the further y-inverses they need
+    int fused_products(bool inc) {
+        if constexpr (std::is_same<T, float>::value) {
+            const TermPlan &pl = term_plan(s);
+            const int nf = (int)s->fields.size();
+            const size_t all = s->field_elems * (size_t)s->nslots();
+            float2 *extra = (float2 *)s->term_extra;
+            for (size_t e = 0; e < pl.extras.size(); ++e) {
+                const auto &x = pl.extras[e];
+                // one instance: the field's own slot; a batch: every slot in one launch
+                Seq<T> q{s, st, s->batch == 1 ? x.field : 0, s->batch == 1 ? 1 : s->nslots()};
+                q.op_on = 1;
+                q.op_deriv = x.dy ? 1 : -1;
+                q.op_lap = x.lap;
+                if (int rc = q.col_ptrs(COL_INV_MASK, q.state(), nullptr, extra + e * all, nullptr, 0)) return rc;
+            }
+            TermArgs a{};
+            a.sp = sys_params<float>(s);
+            a.fps = (const FieldP<float> *)s->fps;
+            a.in = (const float2 *)A();
+            a.extra = extra;
+            a.extra_stride = all;
+            a.out = (float2 *)B();
+            a.slot_stride = s->field_elems;
+            a.coef = s->term_coef;
+            a.tw = (const float2 *)s->tw;
+            a.d_step = s->d_step;
+            a.nf = nf;
+            a.inc_step = inc ? 1 : 0;
+            a.prog = pl.prog;
+            a.G = terms_G(s);
+            cudaError_t e = launch_terms(a, s->batch, st);
+            s->launches++;
+            if (e != cudaSuccess) return cuda_fail(s, e, "k_row_terms launch");
+            return PSS_OK;
+        } else {
+            (void)inc;
+            return fail(s, PSS_EUNSUPPORTED, "the fused product terms are FP32 only");
+        }
+    }
+
     // B <- x-transformed product of the current state (start of a run)
     int prologue() {
         int rc;
+        if (fused_terms(s)) {
+            if ((rc = col(COL_INV_MASK, false, true))) return rc;                 // state -> A
+            return fused_products(false);                                          // A -> B
+        }
         if (fast2d(s)) {
             if ((rc = col2(COL_INV_MASK))) return rc;                             // state -> A (column-major)
             return row2(false);                                                    // A -> B (column-major)
@@ -1060,6 +1219,10 @@ template <typename T> struct Seq {
 
     int one_step() {
         int rc;
+        if (fused_terms(s)) {
+            if ((rc = col(COL_STEP, true, true))) return rc;                       // B, state -> state, A
+            return fused_products(true);                                           // A -> B, step++
+        }
         if (fast2d(s)) {
             if ((rc = col2(COL_STEP))) return rc;                                 // B, state -> state, A
             return row2(true);                                                     // A -> B, step++
@@ -1192,7 +1355,7 @@ template <typename T> int general_products(pss_system *s, cudaStream_t st) {
 
 template <typename T> int full_prologue(pss_system *s, cudaStream_t st) {
     int rc = Seq<T>{s, st, 0, s->nslots()}.prologue();
-    if (rc || !any_general(s)) return rc;
+    if (rc || !any_general(s) || fused_terms(s)) return rc;
     return general_products<T>(s, st);
 }
 
@@ -1200,6 +1363,17 @@ template <typename T> int run_prologue(pss_system *s) { return full_prologue<T>(
 
 int alloc_term_scratch(pss_system *s) {
     if (!any_general(s)) return PSS_OK;
+    if (fused_terms(s)) {
+        const size_t need = term_plan(s).extras.size() * csize(s) * s->field_elems * (size_t)s->nslots();
+        if (s->term_extra_bytes < need) {
+            cudaFree(s->term_extra);
+            s->term_extra = nullptr;
+            s->term_extra_bytes = 0;
+            CK(cudaMalloc(&s->term_extra, need));
+            s->term_extra_bytes = need;
+        }
+        if (!persist2d(s)) return PSS_OK;    // (the persistent KPZ step keeps its second array in GS)
+    }
     if (!s->GS) CK(cudaMalloc(&s->GS, csize(s) * s->field_elems * (size_t)s->nslots()));
     if (!s->real) CK(cudaMalloc(&s->real, rsize(s) * (size_t)s->nsites));
     if (!s->real_acc) CK(cudaMalloc(&s->real_acc, rsize(s) * (size_t)s->nsites));
@@ -1247,7 +1421,7 @@ bool round_trip(const pss_system *s) {
 template <typename T> int step_once(pss_system *s, cudaStream_t st) {
     int rc = Seq<T>{s, st, 0, s->nslots()}.one_step();
     if (rc) return rc;
-    if (!round_trip(s)) return any_general(s) ? general_products<T>(s, st) : PSS_OK;
+    if (!round_trip(s)) return any_general(s) && !fused_terms(s) ? general_products<T>(s, st) : PSS_OK;
     // per slot: the full real field, its frame, and back to the spectrum
     const int nf = (int)s->fields.size();
     for (int slot = 0; slot < s->nslots(); ++slot) {
@@ -1944,6 +2118,8 @@ int pss_destroy_system(pss_system *s) {
     cudaFree(s->GS);
     cudaFree(s->real_acc);
     cudaFree(s->real_tp);
+    cudaFree(s->term_extra);
+    cudaFree(s->term_coef);
     cudaFree(s->fps);
     cudaFree(s->tw);
     cudaFree(s->real);
@@ -2088,6 +2264,7 @@ int pss_add_term(pss_system *s, int field_id, int implicit, int n_mono, const in
     }
     s->stale = true;
     s->fps_dirty = true;
+    if (any_general(s)) invalidate(s);   // the fused terms are launch arguments
     return PSS_OK;
 }
 
@@ -2437,6 +2614,11 @@ int pss_set_tuning(pss_system *s, const char *key, int value) {
     else if (k == "real_state") s->tune_real_state = value ? 1 : 0;
     else if (k == "test_timeout") s->tune_test_timeout = value ? 1 : 0;
     else if (k == "persist") s->tune_persist = value ? 1 : 0;
+    else if (k == "fuse_terms") {
+        s->tune_fuse_terms = value ? 1 : 0;
+        s->fps_dirty = true;   // the operators and the product's layout follow it
+        s->stale = true;
+    }
     else if (k == "resident") s->tune_resident = value ? 1 : 0;
     else if (k == "res_ctas") {
         if (value > 16) return fail(s, PSS_EINVAL, "res_ctas is at most 16 (0 = automatic)");

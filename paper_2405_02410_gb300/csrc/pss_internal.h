@@ -293,6 +293,35 @@ struct Res2Args {
     int nsteps;
     int C;                      // CTAs per cluster, a power of two
 };
+// The product terms of an FP32 1D or 2D instance as k_row_terms takes them:
+// distinct factors psi = F^-1[(i q_x if dx) Y m phi_field], Y the y-inverse in
+// array `arr` (-1: the column kernel's plain one, else an extra one), and per
+// target field its terms, coefficient times a product of powers of factors.
+constexpr int kMaxTermFactors = 6, kMaxTerms = 6, kMaxTermProduct = 4;
+struct TermFactor { int field, arr, dx; };
+struct TermP { int n; int fac[kMaxTermProduct], power[kMaxTermProduct]; };
+struct TermProg {
+    int nfac;
+    TermFactor fac[kMaxTermFactors];
+    int nterm[kMaxFields];
+    TermP term[kMaxFields][kMaxTerms];
+};
+struct TermArgs {
+    SysP<float> sp;
+    const FieldP<float> *fps;
+    const float2 *in;           // plain y-inverses, tiled [slot]
+    const float2 *extra;        // further y-inverses, arrays of all slots extra_stride apart
+    size_t extra_stride;
+    float2 *out;                // the sums transformed along x, tiled [slot]
+    size_t slot_stride;
+    const float *coef;          // [slot][kMaxTerms] coefficients of the field's terms
+    const float2 *tw;
+    long long *d_step;
+    int nf, G, inc_step;        // fields per instance, row pairs per CTA
+    TermProg prog;
+};
+cudaError_t launch_terms(const TermArgs &a, int batch, cudaStream_t st);
+
 // A run of steps of a 1D system (k_line: 64..1024 sites), one CTA per slot.
 // Per field: its explicit term M(q) F[(F^-1[op(q) m phi])^power] (power 0:
 // none; op as in ColArgs), and its boundary frame.
@@ -357,6 +386,7 @@ __host__ __device__ constexpr int col_threads(int n, int emax, int F) {
     return 2 * F * fft_TPF(n, emax) <= 512 ? (2 * F * fft_TPF(n, emax) < 32 ? 32 : 2 * F * fft_TPF(n, emax))
                                             : F * fft_TPF(n, emax);
 }
+inline int sf_row_h(int n) { return n + n / 16 + 16; }   // at least the row kernels' buffer slice per transform
 inline int fft_smem_elems_h(int n, int F) { return (n + n / 16) * F; }
 
 }  // namespace pss
