@@ -3042,6 +3042,19 @@ int pss_load_state(pss_system *s, const void *buf, size_t len) {
     return device_errors(s);
 }
 
+// Bin means, counts and L = 2 pi sum S / sum |q| S from the accumulator (the
+// last word is sum S times |q| in units of pi / (nbins dx))
+static void finish_structure_factor(const pss_system *s, const double *h, int nbins, double *S_out, double *count_out,
+                                    double *L_out) {
+    double sum = 0.0;
+    for (int b = 0; b < nbins; ++b) {
+        S_out[b] = h[nbins + b] > 0 ? h[b] / h[nbins + b] : 0.0;
+        if (count_out) count_out[b] = h[nbins + b];
+        sum += h[b];
+    }
+    if (L_out) *L_out = h[2 * nbins] > 0 ? 2.0 * nbins * s->dx[0] * sum / h[2 * nbins] : 0.0;
+}
+
 int pss_structure_factor(pss_system *s, int field_id, int nbins, double *S_out, double *count_out, double *L_out) {
     int rc = check_field(s, field_id);
     if (rc) return rc;
@@ -3058,19 +3071,15 @@ int pss_structure_factor(pss_system *s, int field_id, int nbins, double *S_out, 
     const size_t ofs = csize(s) * s->field_elems * (size_t)cur_slot(s, field_id);
     cudaError_t e = s->prec == PSS_F64
         ? launch_structure_factor<double>(sys_params<double>(s), s->dx, (const double2 *)((char *)s->state + ofs), nbins,
-                                          s->sq, s->stream)
+                                          s->sq, s->num_sms, s->stream)
         : launch_structure_factor<float>(sys_params<float>(s), s->dx, (const float2 *)((char *)s->state + ofs), nbins,
-                                         s->sq, s->stream);
+                                         s->sq, s->num_sms, s->stream);
     s->launches++;
     if (e != cudaSuccess) return cuda_fail(s, e, "structure factor kernel");
     std::vector<double> h(need);
     CK(cudaMemcpyAsync(h.data(), s->sq, sizeof(double) * need, cudaMemcpyDeviceToHost, s->stream));
     if ((rc = device_errors(s))) return rc;
-    for (int b = 0; b < nbins; ++b) {
-        S_out[b] = h[nbins + b] > 0 ? h[b] / h[nbins + b] : 0.0;
-        if (count_out) count_out[b] = h[nbins + b];
-    }
-    if (L_out) *L_out = h[2 * nbins + 1] > 0 ? 2 * kPi * h[2 * nbins] / h[2 * nbins + 1] : 0.0;
+    finish_structure_factor(s, h.data(), nbins, S_out, count_out, L_out);
     return PSS_OK;
 }
 
@@ -3123,19 +3132,15 @@ int pss_structure_factor_noalloc(pss_system *s, int field_id, int nbins, double 
     const size_t ofs = csize(s) * s->field_elems * (size_t)cur_slot(s, field_id);
     cudaError_t e = s->prec == PSS_F64
         ? launch_structure_factor<double>(sys_params<double>(s), s->dx, (const double2 *)((char *)s->state + ofs), nbins,
-                                          acc, s->stream)
+                                          acc, s->num_sms, s->stream)
         : launch_structure_factor<float>(sys_params<float>(s), s->dx, (const float2 *)((char *)s->state + ofs), nbins,
-                                         acc, s->stream);
+                                         acc, s->num_sms, s->stream);
     s->launches++;
     if (e != cudaSuccess) return cuda_fail(s, e, "structure factor kernel");
     double h[kNoAllocSlots];   // host copy on the stack: no heap allocation either
     CK(cudaMemcpyAsync(h, acc, sizeof(double) * need, cudaMemcpyDeviceToHost, s->stream));
     if ((rc = device_errors(s))) return rc;
-    for (int b = 0; b < nbins; ++b) {
-        S_out[b] = h[nbins + b] > 0 ? h[b] / h[nbins + b] : 0.0;
-        if (count_out) count_out[b] = h[nbins + b];
-    }
-    if (L_out) *L_out = h[2 * nbins + 1] > 0 ? 2 * kPi * h[2 * nbins] / h[2 * nbins + 1] : 0.0;
+    finish_structure_factor(s, h, nbins, S_out, count_out, L_out);
     return PSS_OK;
 }
 

@@ -371,7 +371,7 @@ template <typename T> cudaError_t launch_segment_begin(cplx<T> *dst, const cplx<
 cudaError_t launch_set_i64(long long *dst, long long value, cudaStream_t st);
 template <typename T> cudaError_t launch_structure_factor(const SysP<T> &sp, const double dx[3],
                                                           const cplx<T> *tiles, int nbins,
-                                                          double *acc /* 2*nbins + 2 */, cudaStream_t st);
+                                                          double *acc /* 2*nbins + 1 */, int num_sms, cudaStream_t st);
 
 // FFT shape helpers visible to the host
 __host__ __device__ constexpr int ilog2(int n) { return n <= 1 ? 0 : 1 + ilog2(n >> 1); }

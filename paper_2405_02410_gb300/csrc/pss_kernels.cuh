@@ -1135,82 +1135,99 @@ cudaError_t launch_segment_begin(cplx<T> *dst, const cplx<T> *ck, size_t slot_el
 }
 
 // S(q) accumulation: acc[0..nbins) sum S, acc[nbins..2nbins) counts,
-// acc[2nbins] sum S, acc[2nbins+1] sum |q| S.  Bin arithmetic in FP64 with
-// explicit round-to-nearest operations (no contraction).
+// acc[2nbins] sum |q| S nbins dx / pi (the host sums the bins for sum S).  Bin
+// arithmetic in FP64 with explicit round-to-nearest operations (no
+// contraction), sums in FP64.
+//
+// Bound by FP64 operations (one warp instruction per scheduler in 64 cycles),
+// so the kernel counts them: a warp takes 32 neighbouring kx and up to 32 rows,
+// computes each axis' term of s^2 = (|q| nbins dx / pi)^2 once per kx and once
+// per row (lane r for row r, handed out by shuffles), and per mode is left with
+// the sum, one root (the bin and |q|), |z|^2 and two accumulations: 17
+// operations where each mode took about a hundred.  A lane adds up the modes
+// of one bin as it walks down the rows and adds a run to the CTA's bins when
+// the bin changes; the counts are integers.  (The sums of 32 lanes by shuffles
+// took 5 additions per bin and 32 modes, which at 128^2 are 32 bins.)
+// us per call of pss_structure_factor before -> after: 1024^2 164 -> 67, 128^2
+// 70 -> 41 (20 of them the copies and the wait).
+constexpr int kSqWarps = 4;
 template <typename T>
-__global__ void k_structure_factor(SysP<T> sp, double dx0, double dx1, double dx2, const cplx<T> *tiles,
-                                   int nbins, double *acc) {
+__global__ void __launch_bounds__(32 * kSqWarps)
+k_structure_factor(SysP<T> sp, double dx0, double dx1, double dx2, const cplx<T> *tiles, int nbins, int nrow,
+                   double *acc) {
     extern __shared__ double sacc[];
-    for (int i = threadIdx.x; i < 2 * nbins + 2; i += blockDim.x) sacc[i] = 0.0;
+    uint32_t *scnt = reinterpret_cast<uint32_t *>(sacc + nbins);
+    for (int i = threadIdx.x; i < nbins; i += blockDim.x) {
+        sacc[i] = 0.0;
+        scnt[i] = 0u;
+    }
     __syncthreads();
-    const long long n = (long long)sp.nz * sp.ny * sp.hx;
     const double inv_ns = 1.0 / ((double)sp.nx * sp.ny * sp.nz);
-    const double dxs[3] = {dx0, dx1, dx2};
-    const int Ns[3] = {sp.nx, sp.ny, sp.nz};
     const int lane = threadIdx.x & 31;
-    double tS = 0.0, tQ = 0.0;   // the thread's share of the two totals
-    // the warps step through the modes 32 at a time (neighbouring kx of one row, a
-    // handful of bins at most): lanes in one bin are summed with shuffles and one
-    // lane adds the sums to the CTA's bins
-    for (long long i0 = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < n;
-         i0 += (long long)gridDim.x * blockDim.x) {
-        const long long i = i0 + lane;
+    const int nkb = (sp.hx + 31) >> 5, nrb = (sp.rows + nrow - 1) / nrow;
+    // (2 nbins k dx0 / (N dx))^2
+    auto axis = [&](int k, int n, double dx) {
+        const double t = __ddiv_rn(__dmul_rn(__dmul_rn(__dmul_rn(2.0, (double)nbins), (double)k), dx0),
+                                   __dmul_rn((double)n, dx));
+        return __dmul_rn(t, t);
+    };
+    double tQ = 0.0;
+    for (int w = blockIdx.x * kSqWarps + (threadIdx.x >> 5); w < nkb * nrb; w += gridDim.x * kSqWarps) {
+        const int kb = w % nkb, r0 = (w / nkb) * nrow, nr = min(nrow, sp.rows - r0);
+        const int kx = kb * 32 + lane;
+        const bool in = kx < sp.hx;
+        const double ax = sp.nx == 1 ? 0.0 : __dadd_rn(0.0, axis(kx, sp.nx, dx0));
+        double ay = 0.0, az = 0.0;                            // of row r0 + lane
+        {
+            const int row = min(r0 + lane, sp.rows - 1);
+            const int ky = sp.dim == 3 ? row / sp.nz : row, kz = sp.dim == 3 ? row % sp.nz : 0;
+            if (sp.ny > 1) ay = axis(signed_k(ky, sp.ny), sp.ny, dx1);
+            if (sp.nz > 1) az = axis(signed_k(kz, sp.nz), sp.nz, dx2);
+        }
+        const bool plane = kx == 0 || 2 * kx == sp.nx;
+        const cplx<T> *z0 = tiles + ((size_t)(kx >> 2) * sp.rows + r0) * W + (kx & 3);
         int b = -1;
-        double vS = 0.0, vW = 0.0;
-        if (i < n) {
-            const int kx = (int)(i % sp.hx);
-            const long long r2 = i / sp.hx;
-            const int ky = (int)(r2 % sp.ny), kz = (int)(r2 / sp.ny);
-            const int ks[3] = {kx, signed_k(ky, sp.ny), signed_k(kz, sp.nz)};
-            double s2 = 0.0, qq = 0.0;
-            for (int j = 0; j < 3; ++j) {
-                if (Ns[j] == 1) continue;
-                const double num = __dmul_rn(__dmul_rn(__dmul_rn(2.0, (double)nbins), (double)ks[j]), dx0);
-                const double tj = __ddiv_rn(num, __dmul_rn((double)Ns[j], dxs[j]));
-                s2 = __dadd_rn(s2, __dmul_rn(tj, tj));
-                const double qj = 6.283185307179586 * ks[j] / (Ns[j] * dxs[j]);
-                qq += qj * qj;
+        uint32_t cnt = 0u;
+        double run = 0.0;
+        auto flush = [&]() {
+            if (b >= 0) {
+                atomicAdd(&sacc[b], run);
+                atomicAdd(&scnt[b], cnt);
             }
+            run = 0.0;
+            cnt = 0u;
+        };
+#pragma unroll 1
+        for (int r = 0; r < nr; ++r) {
+            const double y = __shfl_sync(0xffffffffu, ay, r), zz = __shfl_sync(0xffffffffu, az, r);
+            if (!in) continue;
+            double s2 = ax;
+            if (sp.ny > 1) s2 = __dadd_rn(s2, y);
+            if (sp.nz > 1) s2 = __dadd_rn(s2, zz);
             const double s = __dsqrt_rn(s2);
-            if (s2 != 0.0 && s <= (double)nbins) {
-                b = (int)ceil(s) - 1;
-                const int row = sp.dim == 3 ? ky * sp.nz + kz : ky;
-                const cplx<T> z = tiles[((size_t)(kx / W) * sp.rows + row) * W + kx % W];
-                const double S = ((double)z.x * z.x + (double)z.y * z.y) * inv_ns;
-                vW = (kx == 0 || 2 * kx == sp.nx) ? 1.0 : 2.0;
-                vS = vW * S;
-                tS += vS;
-                tQ += vW * sqrt(qq) * S;
+            if (!(s2 != 0.0 && s <= (double)nbins)) continue;
+            const int nb = (int)ceil(s) - 1;
+            if (nb != b) {
+                flush();
+                b = nb;
             }
+            const cplx<T> z = z0[(size_t)r * W];
+            double v = ((double)z.x * z.x + (double)z.y * z.y) * inv_ns;
+            if (!plane) v += v;
+            cnt += plane ? 1u : 2u;
+            run += v;
+            tQ += s * v;
         }
-        unsigned todo = __ballot_sync(0xffffffffu, b >= 0);
-        while (todo) {
-            const int src = __ffs(todo) - 1;
-            const int b0 = __shfl_sync(0xffffffffu, b, src);
-            const bool mine = b == b0;
-            double sv = mine ? vS : 0.0, wv = mine ? vW : 0.0;
-            for (int o = 16; o > 0; o >>= 1) {
-                sv += __shfl_xor_sync(0xffffffffu, sv, o);
-                wv += __shfl_xor_sync(0xffffffffu, wv, o);
-            }
-            if (lane == src) {
-                atomicAdd(&sacc[b0], sv);
-                atomicAdd(&sacc[nbins + b0], wv);
-            }
-            todo &= ~__ballot_sync(0xffffffffu, mine);
-        }
+        flush();
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        tS += __shfl_xor_sync(0xffffffffu, tS, o);
-        tQ += __shfl_xor_sync(0xffffffffu, tQ, o);
-    }
-    if (lane == 0) {
-        if (tS != 0.0) atomicAdd(&sacc[2 * nbins], tS);
-        if (tQ != 0.0) atomicAdd(&sacc[2 * nbins + 1], tQ);
-    }
+    for (int o = 16; o > 0; o >>= 1) tQ += __shfl_xor_sync(0xffffffffu, tQ, o);
+    if (lane == 0 && tQ != 0.0) atomicAdd(&acc[2 * nbins], tQ);
     __syncthreads();
-    for (int i = threadIdx.x; i < 2 * nbins + 2; i += blockDim.x)
-        if (sacc[i] != 0.0) atomicAdd(&acc[i], sacc[i]);
+    for (int i = threadIdx.x; i < nbins; i += blockDim.x)
+        if (scnt[i]) {
+            atomicAdd(&acc[i], sacc[i]);
+            atomicAdd(&acc[nbins + i], (double)scnt[i]);
+        }
 }
 
 // ---------------------------------------------------------------------------
@@ -1403,15 +1420,18 @@ cudaError_t launch_half_to_tiles(const SysP<T> &sp, const cplx<T> *half, cplx<T>
 
 template <typename T>
 cudaError_t launch_structure_factor(const SysP<T> &sp, const double dx[3], const cplx<T> *tiles, int nbins,
-                                    double *acc, cudaStream_t st) {
-    const long long n = (long long)sp.nz * sp.ny * sp.hx;
-    // at most 512 CTAs: each adds its 2 nbins + 2 sums to the same global words
-    long long blocks = (n + 255) / 256;
-    if (blocks > 512) blocks = 512;
-    const size_t smem = sizeof(double) * (size_t)(2 * nbins + 2);
+                                    double *acc, int num_sms, cudaStream_t st) {
+    // rows per warp: the fewest (4 .. 32) that leave the schedulers two warps each
+    const long long nkb = (sp.hx + 31) / 32;
+    int nrow = 4;
+    while (nrow < 32 && nkb * sp.rows / nrow > 8ll * num_sms) nrow *= 2;
+    const long long warps = nkb * ((sp.rows + nrow - 1) / nrow);
+    long long blocks = (warps + kSqWarps - 1) / kSqWarps;
+    if (blocks > 8ll * num_sms) blocks = 8ll * num_sms;   // each adds its bins to the same global words
+    const size_t smem = (sizeof(double) + sizeof(uint32_t)) * (size_t)nbins;
     cudaError_t e = ensure_smem(k_structure_factor<T>, smem);
     if (e != cudaSuccess) return e;
-    k_structure_factor<T><<<(int)blocks, 256, smem, st>>>(sp, dx[0], dx[1], dx[2], tiles, nbins, acc);
+    k_structure_factor<T><<<(int)blocks, 32 * kSqWarps, smem, st>>>(sp, dx[0], dx[1], dx[2], tiles, nbins, nrow, acc);
     return cudaGetLastError();
 }
 
@@ -1433,6 +1453,6 @@ cudaError_t launch_structure_factor(const SysP<T> &sp, const double dx[3], const
     template cudaError_t launch_segment_begin<T>(cplx<T> *, const cplx<T> *, size_t, const long long *, long long, \
                                                  long long, long long *, long long *, cudaStream_t);             \
     template cudaError_t launch_structure_factor<T>(const SysP<T> &, const double *, const cplx<T> *, int,   \
-                                                    double *, cudaStream_t);
+                                                    double *, int, cudaStream_t);
 
 }  // namespace pss
