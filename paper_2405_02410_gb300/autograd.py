@@ -42,8 +42,8 @@ class PSSRun(torch.autograd.Function):
             raise ValueError("h0 must be a CUDA tensor (the half spectrum stays on the device)")
         sys_ = system
         sys_.set_stream(torch.cuda.current_stream(h0.device))
-        for i, pid in enumerate(param_ids):
-            sys_.set_param(pid, float(params[i]))
+        for pid, value in zip(param_ids, params.detach().tolist()):   # one copy to the host
+            sys_.set_param(pid, value)
         sys_.set_step(step0)
         sys_.set_spectrum(0, h0.detach().to(_cdtype(sys_)).contiguous())
         sys_.adjoint_forward(int(nsteps))
@@ -79,18 +79,22 @@ def binned_structure_factor(h: torch.Tensor, shape, nbins: int = 64, dx: float =
     the bin of a mode is ceil(|q| nbins dx / pi) - 1.  Returns (S[nbins], counts[nbins])."""
     shape = tuple(shape)
     n = int(np.prod(shape))
-    ks = [np.fft.fftfreq(m) * m for m in shape[:-1]] + [np.arange(shape[-1] // 2 + 1)]
-    grids = np.meshgrid(*ks, indexing="ij")
-    s2 = sum((2.0 * nbins * k / m) ** 2 for k, m in zip(grids, shape))
-    s = np.sqrt(s2)
-    b = np.ceil(s).astype(np.int64) - 1
+    # the bins on h's device, in FP64 (the same operations as on the host, each
+    # correctly rounded)
+    s2, w = 0.0, None
+    for axis, m in enumerate(shape):
+        last = axis == len(shape) - 1
+        i = torch.arange(m // 2 + 1 if last else m, device=h.device)
+        k = (i if last else torch.where(i < (m + 1) // 2, i, i - m)).to(torch.float64)
+        view = [1] * len(shape)
+        view[axis] = -1
+        s2 = s2 + ((2.0 * nbins * k / m) ** 2).view(view)
+        if last:
+            w = torch.where((i == 0) | ((2 * i == m) if m % 2 == 0 else (i < 0)), 1.0, 2.0).to(torch.float64).view(view)
+    s = torch.sqrt(s2)
     valid = (s2 > 0) & (s <= nbins)
-    w = np.where(grids[-1] == 0, 1.0, 2.0)
-    if shape[-1] % 2 == 0:
-        w = np.where(grids[-1] == shape[-1] // 2, 1.0, w)
-    w = np.where(valid, w, 0.0)
-    bidx = torch.from_numpy(np.where(valid, b, 0).reshape(-1)).to(h.device)
-    wt = torch.from_numpy(w.reshape(-1)).to(device=h.device, dtype=torch.float64)
+    bidx = torch.where(valid, torch.ceil(s) - 1, torch.zeros_like(s)).to(torch.int64).reshape(-1)
+    wt = torch.where(valid, w, torch.zeros_like(s)).reshape(-1)
     p = (h.reshape(-1).abs().to(torch.float64) ** 2) * wt / n
     sums = torch.zeros(nbins, dtype=torch.float64, device=h.device).index_add(0, bidx, p)
     cnt = torch.zeros(nbins, dtype=torch.float64, device=h.device).index_add(0, bidx, wt)

@@ -169,6 +169,7 @@ struct pss_system {
     void *seg_noise = nullptr;               // their unit noise [K + 1][slot] (the persistent path)
     double *d_grad = nullptr;                // [11]
     long long *d_seg = nullptr;              // [2]: segment index, step of its first step (device)
+    int64_t ck_cap = 0, seg_cap = 0;         // checkpoints, steps of a segment they hold
     int64_t adj_n = 0, adj_step0 = 0, adj_K = 0, adj_nck = 0;
     bool adj_ready = false;
     cudaGraphExec_t adj_graph = nullptr;     // one full segment of the backward pass
@@ -1236,27 +1237,29 @@ template <typename T> struct Seq {
         return row(ROW_FUSED, true, true, true, nullptr, 0);                        // A -> B, step++
     }
 
-    // real scratch -> state of the sequence's slots
-    int forward_from_real() {
+    // real field (by default the scratch) -> state of the sequence's slots
+    int forward_from_real(const void *real = nullptr) {
         int rc;
+        const T *r = (const T *)(real ? real : s->real);
         if (s->dim == 3) {
-            if ((rc = row(ROW_R2C, true, false, false, s->real, 0))) return rc;   // real -> A
+            if ((rc = row_ptrs(ROW_R2C, A(), A(), false, r, nullptr, 0))) return rc;   // real -> A
             if ((rc = mid(MID_FWD, true, false))) return rc;                      // A -> B
         } else {
-            if ((rc = row(ROW_R2C, true, true, false, s->real, 0))) return rc;    // real -> B
+            if ((rc = row_ptrs(ROW_R2C, A(), B(), false, r, nullptr, 0))) return rc;   // real -> B
         }
         return col(COL_FWD, true, true);                                          // B -> state
     }
 
-    // state -> real scratch
-    int inverse_to_real() {
+    // state -> real field (by default the scratch)
+    int inverse_to_real(void *real = nullptr) {
         int rc;
+        void *r = real ? real : s->real;
         if ((rc = col(COL_INV_FULL, false, true))) return rc;                     // state -> A
         if (s->dim == 3) {
             if ((rc = mid(MID_INV_FULL, true, false))) return rc;                 // A -> B
-            return row(ROW_C2R, false, false, false, s->real, 0);                 // B -> real
+            return row(ROW_C2R, false, false, false, r, 0);                       // B -> real
         }
-        return row(ROW_C2R, true, false, false, s->real, 0);                      // A -> real
+        return row(ROW_C2R, true, false, false, r, 0);                            // A -> real
     }
 
     // Recompute of one forward step for the adjoint: phi_n (st_in) -> phi_n+1
@@ -1783,10 +1786,17 @@ int ensure_half(pss_system *s) {
     return PSS_OK;
 }
 
+int report_status(pss_system *s, int st);
+
 int device_errors(pss_system *s) {
     int st = 0;
     CK(cudaMemcpyAsync(&st, s->d_status, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
+    return report_status(s, st);
+}
+
+// the status word of the device as an error of this call (cleared)
+int report_status(pss_system *s, int st) {
     if (st) {
         CK(cudaMemsetAsync(s->d_status, 0, sizeof(int), s->stream));
         if (st & 2) {
@@ -1936,41 +1946,53 @@ int do_create(pss_system **out, int batch, int dim, int nx, int ny, int nz, doub
 }
 
 // per-slot real-space transfers go through the one-slot scratch
-template <typename T> int forward_slot(pss_system *s, int slot) {
-    return Seq<T>{s, s->stream, slot, 1}.forward_from_real();
+template <typename T> int forward_slot(pss_system *s, int slot, const void *real) {
+    return Seq<T>{s, s->stream, slot, 1}.forward_from_real(real);
 }
-template <typename T> int inverse_slot(pss_system *s, int slot) {
-    return Seq<T>{s, s->stream, slot, 1}.inverse_to_real();
+template <typename T> int inverse_slot(pss_system *s, int slot, void *real) {
+    return Seq<T>{s, s->stream, slot, 1}.inverse_to_real(real);
 }
 
-int forward_field(pss_system *s, int field_id) {
+int forward_field(pss_system *s, int field_id, const void *real = nullptr) {
     int rc = upload_params(s);
     if (rc) return rc;
     const int slot = cur_slot(s, field_id);
-    rc = s->prec == PSS_F64 ? forward_slot<double>(s, slot) : forward_slot<float>(s, slot);
+    rc = s->prec == PSS_F64 ? forward_slot<double>(s, slot, real) : forward_slot<float>(s, slot, real);
     s->stale = true;
     return rc;
 }
 
+// The checkpoints and a segment's arrays, kept from one adjoint run to the next
+// and grown when a run needs more (cudaMalloc and cudaFree of all of them, and
+// capturing the segment again, were 0.5 ms of every run).  The segment's graph
+// holds the run's first step and segment length, and these buffers.
 int adj_alloc(pss_system *s, int64_t nck, int64_t K) {
     const size_t slot_bytes = csize(s) * s->field_elems;
-    cudaFree(s->ck);
-    cudaFree(s->seg);
-    cudaFree(s->seg_prod);
-    cudaFree(s->seg_real);
-    cudaFree(s->seg_noise);
-    s->ck = s->seg = s->seg_prod = s->seg_real = s->seg_noise = nullptr;
-    CK(cudaMalloc(&s->ck, slot_bytes * (size_t)(nck + 1)));
-    CK(cudaMalloc(&s->seg, slot_bytes * (size_t)(K + 1)));
-    CK(cudaMalloc(&s->seg_prod, slot_bytes * (size_t)(K + 1)));
-    CK(cudaMalloc(&s->seg_real, rsize(s) * (size_t)s->nsites * (size_t)(K + 1)));
-    if (persist2d_ok(s)) CK(cudaMalloc(&s->seg_noise, slot_bytes * (size_t)(K + 1)));
+    const bool noise = persist2d_ok(s);
+    const bool grow_seg = K > s->seg_cap || (noise && !s->seg_noise);
+    if (nck > s->ck_cap || grow_seg || s->adj_K != K || s->adj_step0 != s->step) s->adj_graph_valid = false;
+    if (nck > s->ck_cap) {
+        cudaFree(s->ck);
+        s->ck = nullptr;
+        s->ck_cap = 0;
+        CK(cudaMalloc(&s->ck, slot_bytes * (size_t)(nck + 1)));
+        s->ck_cap = nck;
+    }
+    if (grow_seg) {
+        for (void **p : {&s->seg, &s->seg_prod, &s->seg_real, &s->seg_noise}) {
+            cudaFree(*p);
+            *p = nullptr;
+        }
+        s->seg_cap = 0;
+        CK(cudaMalloc(&s->seg, slot_bytes * (size_t)(K + 1)));
+        CK(cudaMalloc(&s->seg_prod, slot_bytes * (size_t)(K + 1)));
+        CK(cudaMalloc(&s->seg_real, rsize(s) * (size_t)s->nsites * (size_t)(K + 1)));
+        if (noise) CK(cudaMalloc(&s->seg_noise, slot_bytes * (size_t)(K + 1)));
+        s->seg_cap = K;
+    }
     if (!s->L) CK(cudaMalloc(&s->L, slot_bytes));
     if (!s->d_grad) CK(cudaMalloc(&s->d_grad, sizeof(double) * 11));
     if (!s->d_seg) CK(cudaMalloc(&s->d_seg, sizeof(long long) * 2));
-    if (s->adj_graph) cudaGraphExecDestroy(s->adj_graph);
-    s->adj_graph = nullptr;
-    s->adj_graph_valid = false;
     return PSS_OK;
 }
 
@@ -2366,6 +2388,9 @@ int pss_set_field(pss_system *s, int field_id, const void *real, int where) {
     int rc = check_field(s, field_id);
     if (rc) return rc;
     if (!real) return fail(s, PSS_EINVAL, "real is NULL");
+    // the row kernel reads a device field where it is (its bulk copies want 16-byte
+    // alignment); host fields and others go through the scratch
+    if (where != PSS_HOST && (uintptr_t)real % 16 == 0) return forward_field(s, field_id, real);
     if ((rc = ensure_real(s))) return rc;
     const size_t bytes = rsize(s) * (size_t)s->nsites;
     CK(cudaMemcpyAsync(s->real, real, bytes, where == PSS_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice,
@@ -2858,9 +2883,9 @@ int pss_get_step(pss_system *s, int64_t *step) {
 int pss_set_step(pss_system *s, int64_t step) {
     if (!s) return PSS_EINVAL;
     if (step < 0) return fail(s, PSS_EINVAL, "step must be >= 0");
-    long long v = step;
-    CK(cudaMemcpyAsync(s->d_step, &v, sizeof v, cudaMemcpyHostToDevice, s->stream));
-    CK(cudaStreamSynchronize(s->stream));
+    cudaError_t e = launch_set_i64(s->d_step, (long long)step, s->stream);   // in stream order, no host wait
+    s->launches++;
+    if (e != cudaSuccess) return cuda_fail(s, e, "step counter kernel");
     s->step = step;
     s->stale = true;   // the fast 2D path keeps the next step's noise drawn ahead
     return PSS_OK;
@@ -2870,15 +2895,19 @@ int pss_get_field(pss_system *s, int field_id, void *real_out, int where) {
     int rc = check_field(s, field_id);
     if (rc) return rc;
     if (!real_out) return fail(s, PSS_EINVAL, "real_out is NULL");
-    if ((rc = ensure_real(s))) return rc;
+    // the row kernel writes a device field where it is wanted
+    const bool direct = where != PSS_HOST && (uintptr_t)real_out % rsize(s) == 0;
+    if (!direct && (rc = ensure_real(s))) return rc;
     if ((rc = upload_params(s))) return rc;
     const int slot = cur_slot(s, field_id);
-    rc = s->prec == PSS_F64 ? inverse_slot<double>(s, slot) : inverse_slot<float>(s, slot);
+    void *dst = direct ? real_out : s->real;
+    rc = s->prec == PSS_F64 ? inverse_slot<double>(s, slot, dst) : inverse_slot<float>(s, slot, dst);
     if (rc) return rc;
     if (s->dim == 3) s->stale = true;   // the y pass reused B
     const size_t bytes = rsize(s) * (size_t)s->nsites;
-    CK(cudaMemcpyAsync(real_out, s->real, bytes, where == PSS_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice,
-                       s->stream));
+    if (!direct)
+        CK(cudaMemcpyAsync(real_out, s->real, bytes, where == PSS_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice,
+                           s->stream));
     return device_errors(s);
 }
 
@@ -2886,18 +2915,21 @@ int pss_get_spectrum(pss_system *s, int field_id, void *half_out, int where) {
     int rc = check_field(s, field_id);
     if (rc) return rc;
     if (!half_out) return fail(s, PSS_EINVAL, "half_out is NULL");
-    if ((rc = ensure_half(s))) return rc;
+    const bool direct = where != PSS_HOST && (uintptr_t)half_out % csize(s) == 0;
+    if (!direct && (rc = ensure_half(s))) return rc;
+    void *dst = direct ? half_out : s->half;
     const size_t ofs = csize(s) * s->field_elems * (size_t)cur_slot(s, field_id);
     cudaError_t e = s->prec == PSS_F64
-        ? launch_tiles_to_half<double>(sys_params<double>(s), (const double2 *)((char *)s->state + ofs),
-                                       (double2 *)s->half, s->stream)
-        : launch_tiles_to_half<float>(sys_params<float>(s), (const float2 *)((char *)s->state + ofs), (float2 *)s->half,
+        ? launch_tiles_to_half<double>(sys_params<double>(s), (const double2 *)((char *)s->state + ofs), (double2 *)dst,
+                                       s->stream)
+        : launch_tiles_to_half<float>(sys_params<float>(s), (const float2 *)((char *)s->state + ofs), (float2 *)dst,
                                       s->stream);
     s->launches++;
     if (e != cudaSuccess) return cuda_fail(s, e, "layout kernel");
     const size_t bytes = csize(s) * (size_t)s->hx * s->ny * s->nz;
-    CK(cudaMemcpyAsync(half_out, s->half, bytes, where == PSS_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice,
-                       s->stream));
+    if (!direct)
+        CK(cudaMemcpyAsync(half_out, s->half, bytes, where == PSS_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice,
+                           s->stream));
     return device_errors(s);
 }
 
@@ -2905,15 +2937,19 @@ int pss_set_spectrum(pss_system *s, int field_id, const void *half_in, int where
     int rc = check_field(s, field_id);
     if (rc) return rc;
     if (!half_in) return fail(s, PSS_EINVAL, "half_in is NULL");
-    if ((rc = ensure_half(s))) return rc;
     const size_t bytes = csize(s) * (size_t)s->hx * s->ny * s->nz;
-    CK(cudaMemcpyAsync(s->half, half_in, bytes, where == PSS_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice,
-                       s->stream));
+    const void *src = half_in;
+    if (where == PSS_HOST || (uintptr_t)half_in % csize(s) != 0) {
+        if ((rc = ensure_half(s))) return rc;
+        CK(cudaMemcpyAsync(s->half, half_in, bytes, where == PSS_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice,
+                           s->stream));
+        src = s->half;
+    }
     const size_t ofs = csize(s) * s->field_elems * (size_t)cur_slot(s, field_id);
     cudaError_t e = s->prec == PSS_F64
-        ? launch_half_to_tiles<double>(sys_params<double>(s), (const double2 *)s->half,
-                                       (double2 *)((char *)s->state + ofs), s->stream)
-        : launch_half_to_tiles<float>(sys_params<float>(s), (const float2 *)s->half, (float2 *)((char *)s->state + ofs),
+        ? launch_half_to_tiles<double>(sys_params<double>(s), (const double2 *)src, (double2 *)((char *)s->state + ofs),
+                                       s->stream)
+        : launch_half_to_tiles<float>(sys_params<float>(s), (const float2 *)src, (float2 *)((char *)s->state + ofs),
                                       s->stream);
     s->launches++;
     if (e != cudaSuccess) return cuda_fail(s, e, "layout kernel");
@@ -3076,9 +3112,14 @@ int pss_structure_factor(pss_system *s, int field_id, int nbins, double *S_out, 
                                          s->sq, s->num_sms, s->stream);
     s->launches++;
     if (e != cudaSuccess) return cuda_fail(s, e, "structure factor kernel");
+    // the status word rides in the last word of the accumulator: one copy, one wait
     std::vector<double> h(need);
+    CK(cudaMemcpyAsync(s->sq + need - 1, s->d_status, sizeof(int), cudaMemcpyDeviceToDevice, s->stream));
     CK(cudaMemcpyAsync(h.data(), s->sq, sizeof(double) * need, cudaMemcpyDeviceToHost, s->stream));
-    if ((rc = device_errors(s))) return rc;
+    CK(cudaStreamSynchronize(s->stream));
+    int st = 0;
+    std::memcpy(&st, &h[need - 1], sizeof st);
+    if ((rc = report_status(s, st))) return rc;
     finish_structure_factor(s, h.data(), nbins, S_out, count_out, L_out);
     return PSS_OK;
 }
@@ -3138,8 +3179,12 @@ int pss_structure_factor_noalloc(pss_system *s, int field_id, int nbins, double 
     s->launches++;
     if (e != cudaSuccess) return cuda_fail(s, e, "structure factor kernel");
     double h[kNoAllocSlots];   // host copy on the stack: no heap allocation either
+    CK(cudaMemcpyAsync(acc + need - 1, s->d_status, sizeof(int), cudaMemcpyDeviceToDevice, s->stream));
     CK(cudaMemcpyAsync(h, acc, sizeof(double) * need, cudaMemcpyDeviceToHost, s->stream));
-    if ((rc = device_errors(s))) return rc;
+    CK(cudaStreamSynchronize(s->stream));
+    int st = 0;
+    std::memcpy(&st, &h[need - 1], sizeof st);
+    if ((rc = report_status(s, st))) return rc;
     finish_structure_factor(s, h, nbins, S_out, count_out, L_out);
     return PSS_OK;
 }
