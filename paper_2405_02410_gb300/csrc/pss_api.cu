@@ -146,6 +146,7 @@ struct pss_system {
     int tune_adj_radix = 0;                  // FFT radix of that backward pass (8 or 16; 0: the forward's)
     int tune_persist_adj = 1;                // FP32 2D adjoint on the persistent path: a segment's backward pass in one launch                   // FP32 2D adjoint: column parts on FFT groups (0: generic kernel)
     int tune_fuse_terms = 1;                 // FP32 1D/2D product terms in one row kernel (0: factor by factor)
+    int tune_regs3d = 1;                     // FP32 3D: z and y passes with their points in registers (0: staged kernels)
     int tune_resident = 1;                   // FP32 2D sides of 32..512: a run of steps with every slot in one cluster
     int tune_res_ctas = 0;                   // its CTAs per cluster (0 = automatic)
     int res_ctas_auto = 0, res_ctas_slots = 0;   // the automatic choice, for that many slots
@@ -702,6 +703,30 @@ int res_ctas(pss_system *s) {
     return c;
 }
 
+// The register z and y passes of FP32 3D systems (k3_col, k3_mid) where the
+// side has their shape and no launch shape of the staged kernels is asked for.
+// Faster at every size measured (us per step, staged -> registers: 32^3 20.4 ->
+// 13.3, 64^3 pair 22.0 -> 15.7, 256 z x 64 x 32 22.0 -> 18.6, 16 z x 128 x 64
+// 22.3 -> 14.3, 256^3 pair 351 -> 282).  Product terms keep the staged kernels
+// (factors and summed spectra are modes of theirs), and so do the adjoint's modes.
+bool regs3d(const pss_system *s) {
+    return s->tune_regs3d && s->prec == PSS_F32 && s->dim == 3 && !any_general(s) && !s->tune_test_timeout;
+}
+bool regs3d_col(const pss_system *s, int mode) {
+    return regs3d(s) && r3_side(s->nz) && !s->tune_col_radix && !s->tune_col_tiles && mode != COL_ADJ_A &&
+           mode != COL_ADJ_B && mode != COL_ADJ_BA;
+}
+bool regs3d_mid(const pss_system *s) {
+    return regs3d(s) && r3_side(s->ny) && !s->tune_mid_radix && !s->tune_mid_planes;
+}
+// z-planes per CTA of k3_mid: 256 threads, fewer (at least four planes: whole
+// 128-byte lines) where that leaves SMs without a CTA
+int mid3_PZ(const pss_system *s) {
+    int pz = std::min(s->nz, 64 / (s->ny >= 128 ? s->ny / 16 : s->ny >= 32 ? s->ny / 8 : s->ny / 4));
+    while (pz > 4 && (long long)s->ntiles * (s->nz / pz) * s->nslots() < 2 * s->num_sms) pz /= 2;
+    return pz;
+}
+
 // Defaults of the FP32 2D two-kernel path.  A batch of 8 or more instances is
 // throughput-bound rather than latency-bound; measured on GB300 (us per step,
 // single-instance defaults -> batch defaults): 256^2 x 8 11.4 -> 9.5, x 32
@@ -864,6 +889,16 @@ template <typename T> struct Seq {
                 return PSS_OK;
             }
         }
+        if constexpr (std::is_same<T, float>::value) {
+            if (regs3d_col(s, mode) && !op_on) {
+                if (timer) timer->begin(0, st);
+                cudaError_t e = launch_col3(a, nslots, st);
+                if (timer) timer->begin(0, st);
+                s->launches++;
+                if (e != cudaSuccess) return cuda_fail(s, e, "k3_col launch");
+                return PSS_OK;
+            }
+        }
         if (timer) timer->begin(0, st);
         cudaError_t e = launch_col<T>(a, nslots, gx, gy, st);
         if (timer) timer->begin(0, st);
@@ -931,6 +966,17 @@ template <typename T> struct Seq {
         a.inc_step = inc ? 1 : 0;
         const int nt = mode == MID_INV_MASK ? max_kept_tiles(s) : s->ntiles;
         const int kind = mode == MID_FWD ? 3 : 1;
+        if constexpr (std::is_same<T, float>::value) {
+            if (regs3d_mid(s)) {
+                a.PZ = mid3_PZ(s);
+                if (timer) timer->begin(kind, st);
+                cudaError_t e = launch_mid3(a, nslots, nt, st);
+                if (timer) timer->begin(kind, st);
+                s->launches++;
+                if (e != cudaSuccess) return cuda_fail(s, e, "k3_mid launch");
+                return PSS_OK;
+            }
+        }
         if (timer) timer->begin(kind, st);
         cudaError_t e = launch_mid<T>(a, nslots, nt, st);
         if (timer) timer->begin(kind, st);
@@ -2635,6 +2681,7 @@ int pss_set_tuning(pss_system *s, const char *key, int value) {
     else if (k == "graph_steps") s->tune_graph_steps = value;
     else if (k == "fast2d") s->tune_fast2d = value ? 1 : 0;
     else if (k == "fast3d") s->tune_fast3d = value ? 1 : 0;
+    else if (k == "regs3d") s->tune_regs3d = value ? 1 : 0;
     else if (k == "fuse_adjoint") s->tune_fuse_adj = value ? 1 : 0;
     else if (k == "real_state") s->tune_real_state = value ? 1 : 0;
     else if (k == "test_timeout") s->tune_test_timeout = value ? 1 : 0;

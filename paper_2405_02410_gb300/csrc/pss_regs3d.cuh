@@ -1,0 +1,305 @@
+// pss_regs3d.cuh -- the z and y passes of FP32 3D systems with their points in
+// registers (arXiv:2405.02410, section "What cuPSS calculates", Eq. timeupdate).
+//
+// k_col and k_mid stage their tiles in shared memory and run every phase from
+// there; in 3D both are bound by instructions and barriers, not by HBM (k_col
+// at 256^3: 257 instructions per mode, 73 % issue-active, 35 % of the DRAM
+// rate).  Here a thread keeps E points of a transform of N = R1 E points in
+// registers: loads come straight from global memory (consecutive threads take
+// a tile's columns and neighbouring positions, whole 128-byte lines), a
+// transform is two passes with one exchange through shared memory, and the
+// forward transform's outputs (positions lane + r R1) are what the inverse
+// one's first pass reads, so the update runs in registers between them.  The
+// noise is drawn into shared memory while the loads are in flight, a pair of
+// columns per Philox call.  us, staged -> here: 256^3, two fields: z pass 153
+// -> 111 (466 MB: 4.2 TB/s), y inverse 52 -> 37, y forward 63 -> 52 (270 MB:
+// 5.2 TB/s), the step 351 -> 282; whole steps of 128^3 35 -> 28, 256 x 256 x 64
+// 54 -> 41, 64^3 (two fields) 22.0 -> 15.7, 32^3 20.4 -> 13.3.  Forcing 6 CTAs
+// per SM on the step's z pass would leave 80 registers to the 64 that hold its
+// points; 5 take 96.
+#pragma once
+
+#include "pss_kernels.cuh"
+
+namespace pss {
+
+// N = R1 E: R1 threads per transform, E points each; passes of radix R1 (the
+// forward transform's first, BPT butterflies per thread) and E
+template <int N> struct R3Shape {
+    static constexpr int E = N >= 128 ? 16 : N >= 32 ? 8 : 4;
+    static constexpr int R1 = N / E;
+    static constexpr int BPT = E / R1;
+    static constexpr int TILES = 16 / R1;                // k3_col: tiles per CTA
+    static constexpr int THREADS = 8 * TILES * R1;       //   two pencils of each, 128 threads
+    static constexpr int CHUNKS = 2 * TILES;
+    static constexpr int BUF = (N + E) * W;              //   exchange buffer of one chunk, one pad position per butterfly
+    static constexpr int TWN = R1 == E ? N : 2 * N;      // twiddles [r - 1][k] of the radix-E pass, of the radix-R1 one
+    static_assert(R1 <= E && THREADS == 128, "shape");
+};
+
+// twiddles exp(-2 pi i r k / N): of the radix-E pass after R1 points [r - 1][k < R1], and of
+// the radix-R1 pass after E points [r - 1][k < E] at twi (the same where R1 = E)
+template <int N> __device__ __forceinline__ void r3_twiddles(float2 *TW, const float2 *__restrict__ tw, int t, int nthr) {
+    using S = R3Shape<N>;
+    for (int i = t; i < N; i += nthr) {
+        if constexpr (S::R1 == S::E) {
+            TW[i] = tw[twiddle_offset(N, S::E) + i];
+        } else {
+            TW[i] = tw[kRootsOffset + ((i / S::R1 + 1) % S::E) * (i % S::R1) * (kMaxFftN / N)];
+            TW[N + i] = tw[twiddle_offset(N, S::E) + i];
+        }
+    }
+}
+
+// Modes of k3_col: the step, forward only (COL_FWD), inverse only (COL_INV_MASK, COL_INV_FULL)
+enum { R3_STEP = 0, R3_FWD = 1, R3_INV = 2 };
+
+// The z pass.  A CTA takes TILES tiles of the pencils ky and -ky (a kx = 0 mode
+// and its Hermitian partner are in one CTA); thread: column c, lane, chunk.
+template <int N, int MODE> __global__ void __launch_bounds__(128, MODE == R3_STEP ? 5 : 6) k3_col(const ColArgs<float> a) {
+    using S = R3Shape<N>;
+    using C = float2;
+    constexpr int E = S::E, R1 = S::R1;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ FieldP<float> fp;
+    C *TW = reinterpret_cast<C *>(smem_raw);
+    C *XCH = TW + S::TWN;
+    C *XI = XCH + S::CHUNKS * S::BUF;                            // R3_STEP: the noise, [chunk][pos][W]
+    const SysP<float> &sp = a.sp;
+    const int t = threadIdx.x, c = t & (W - 1), lane = (t >> 2) % R1, ch = t / (W * R1);
+    const int slot = a.slot0 + blockIdx.z;
+    const int op = blockIdx.y, opp = (sp.ny - op) & (sp.ny - 1);
+    const bool lone = op == opp;                                 // its own partner: the second chunk is a copy
+    const int first_tile = blockIdx.x * S::TILES, tile = first_tile + (ch >> 1);
+    const int o = (ch & 1) ? opp : op, kx = tile * W + c;
+    const bool ok = tile < a.n_tiles, writes = ok && !((ch & 1) && lone);
+    const size_t ofs = (size_t)slot * a.slot_stride + ((size_t)tile * sp.ny + o) * N * W + c;
+    C *xb = XCH + ch * S::BUF + c;
+    r3_twiddles<N>(TW, a.tw, t, S::THREADS);
+    for (int i = t; i < (int)(sizeof(FieldP<float>) / 4); i += S::THREADS)
+        reinterpret_cast<uint32_t *>(&fp)[i] = reinterpret_cast<const uint32_t *>(&a.fps[slot])[i];
+    __syncthreads();
+    const int oy = signed_k(o, sp.ny);
+    const bool full = a.mode == COL_INV_FULL;
+    // CTA-uniform: nothing of the inverse is kept
+    const bool inverse = MODE != R3_FWD && (full || (first_tile * W <= fp.kmax[0] && abs(signed_k(op, sp.ny)) <= fp.kmax[1]));
+    pdl_wait();
+    pdl_trigger();
+    if (MODE == R3_INV && !inverse) return;
+    const bool keep = kx < sp.hx && (full || (kx <= fp.kmax[0] && abs(oy) <= fp.kmax[1]));
+    const int kmax_pos = full ? N : fp.kmax[2];
+    C v[E];                                                      // from the forward transform on: positions lane + r R1
+    if constexpr (MODE != R3_INV) {
+        const C *__restrict__ in = a.in + ofs;
+#pragma unroll
+        for (int s = 0; s < S::BPT; ++s)
+#pragma unroll
+            for (int r = 0; r < R1; ++r) v[s * R1 + r] = ok ? in[(lane + s * R1 + r * E) * W] : mk<float>(0, 0);
+        if (MODE == R3_STEP && fp.noisy) {
+            const int u = t & (W * R1 - 1), cp = u & 1, kx0 = tile * W + 2 * cp;
+            const float qx0 = (float)kx0 * sp.gx, qx1 = (float)(kx0 + 1) * sp.gx, qo = (float)oy * sp.gy;
+            const float qx0s = qx0 * qx0, qx1s = qx1 * qx1, qo2 = qo * qo;
+            const PhiloxKey key = philox_key(fp.seed_lo, fp.seed_hi);
+            const uint32_t step = (uint32_t)(*a.d_step), fid = (uint32_t)fp.field_id;
+            const bool on_plane = kx0 == 0 || 2 * kx0 == sp.nx, has1 = kx0 + 1 < sp.hx;
+            const int npow = fp.noise_pow;
+            const float sigma0 = fp.sigma0;
+            C *xi = XI + ch * (N * W) + 2 * cp;
+#pragma unroll 1
+            for (int pos = u >> 1; pos < N; pos += 2 * R1) {
+                const float qp = (float)signed_k(pos, N) * sp.gz, qyz2 = qp * qp + qo2;
+                C x0, x1 = mk<float>(0, 0);
+                noise_pair<float>(on_plane, kx0, o, pos, sigma0, npow, qx0s + qyz2, qx1s + qyz2, has1, sp, fid, key, step,
+                                  x0, x1);
+                st_pair<float>(xi + pos * W, x0, x1);
+            }
+        }
+#pragma unroll
+        for (int s = 0; s < S::BPT; ++s) {
+            dft_reg<R1, -1, float>(v + s * R1);
+#pragma unroll
+            for (int r = 0; r < R1; ++r) xb[((lane + s * R1) * (R1 + 1) + r) * W] = v[s * R1 + r];
+        }
+        C ph[E];
+        if (MODE == R3_STEP) {
+#pragma unroll
+            for (int r = 0; r < E; ++r) ph[r] = ok ? a.state[ofs + (lane + r * R1) * W] : mk<float>(0, 0);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+            v[r] = xb[(lane + r * (R1 + 1)) * W];
+            if (r > 0) v[r] = cmul<float>(v[r], TW[(r - 1) * R1 + lane]);
+        }
+        dft_reg<E, -1, float>(v);
+        if constexpr (MODE == R3_STEP) {
+            const bool has_product = fp.power > 0, noisy = fp.noisy != 0;
+            const float qx = (float)kx * sp.gx, qo = (float)oy * sp.gy;
+            const float qxs = qx * qx, qo2 = qo * qo;
+            const C *xi = XI + ch * (N * W) + c;
+            float dtO[kPolyTerms], dtM[kPolyTerms];
+#pragma unroll
+            for (int i = 0; i < kPolyTerms; ++i) {
+                dtO[i] = sp.dt * fp.O[i];
+                dtM[i] = sp.dt * fp.M[i];
+            }
+            bool bad = false;
+            auto update = [&](auto degree2) {
+#pragma unroll
+                for (int r = 0; r < E; ++r) {
+                    const float qp = (float)(lane + r * R1 - (2 * r >= E ? N : 0)) * sp.gz;
+                    const float q2 = qxs + (qp * qp + qo2);
+                    float m, g;
+                    if (decltype(degree2)::value) {
+                        m = ffma(ffma(dtM[2], q2, dtM[1]), q2, dtM[0]);
+                        g = fast_rcp(fadd(1.0f, ffma(ffma(dtO[2], q2, dtO[1]), q2, dtO[0])));
+                    } else {
+                        update_factors<float>(q2, dtO, dtM, m, g);
+                    }
+                    v[r] = update_pre<float>(ph[r], v[r], noisy ? xi[(lane + r * R1) * W] : mk<float>(0, 0), m, g, has_product);
+                    bad |= !finite_mode(v[r]);
+                }
+            };
+            // operators of degree 2 in q^2 (Models A and B) take the short polynomials
+            if (dtO[3] == 0.0f && dtO[4] == 0.0f && dtM[3] == 0.0f && dtM[4] == 0.0f) update(std::true_type{});
+            else update(std::false_type{});
+            if (bad && ok && kx < sp.hx && a.d_status) atomicOr(a.d_status, kStatusNonFinite);
+        }
+        // Hermitian part on the kx = 0 and Nx/2 planes (the field is real): phi(k) <-
+        // (phi(k) + conj phi(-k)) / 2, the partner at position -pos of the partner pencil
+        if (first_tile == 0 || (first_tile * W <= sp.nx / 2 && sp.nx / 2 < (first_tile + S::TILES) * W)) {
+            const bool plane = ok && (kx == 0 || 2 * kx == sp.nx);
+            __syncthreads();
+            if (plane) {
+#pragma unroll
+                for (int r = 0; r < E; ++r) xb[(lane + r * R1) * W] = v[r];
+            }
+            __syncthreads();
+            if (plane) {
+                const C *pb = XCH + (ch ^ 1) * S::BUF + c;
+#pragma unroll
+                for (int r = 0; r < E; ++r) {
+                    const C p = pb[((N - lane - r * R1) & (N - 1)) * W];
+                    v[r] = mk<float>(0.5f * (v[r].x + p.x), 0.5f * (v[r].y - p.y));
+                }
+            }
+        }
+        C *out = (a.state_out ? a.state_out : a.state) + ofs;
+        if (writes) {
+#pragma unroll
+            for (int r = 0; r < E; ++r) out[(lane + r * R1) * W] = kx < sp.hx ? v[r] : mk<float>(0, 0);
+        }
+        if (MODE == R3_FWD || !inverse) return;
+        __syncthreads();                                         // the exchange buffer is free again
+    } else {
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+            const int k = lane + r * R1 - (2 * r >= E ? N : 0);
+            v[r] = ok && keep && abs(k) <= kmax_pos ? a.state[ofs + (lane + r * R1) * W] : mk<float>(0, 0);
+        }
+    }
+    // ---- the inverse of the de-aliased, 1 / N_sites-scaled field
+#pragma unroll
+    for (int r = 0; r < E; ++r) {
+        const int k = lane + r * R1 - (2 * r >= E ? N : 0);
+        v[r] = keep && abs(k) <= kmax_pos ? cscale<float>(v[r], sp.inv_nsites) : mk<float>(0, 0);
+    }
+    dft_reg<E, +1, float>(v);
+#pragma unroll
+    for (int r = 0; r < E; ++r) xb[(lane * (E + 1) + r) * W] = v[r];
+    __syncthreads();
+    const C *TWI = TW + (R1 == E ? 0 : N);
+    C *__restrict__ out = a.out + ofs;
+    const bool stores = writes && (full || tile * W <= fp.kmax[0]);
+#pragma unroll
+    for (int s = 0; s < S::BPT; ++s) {
+        const int i = lane + s * R1;
+        C u[R1];
+#pragma unroll
+        for (int r = 0; r < R1; ++r) {
+            u[r] = xb[(i + r * (E + 1)) * W];
+            if (r > 0) {
+                const C w = TWI[(r - 1) * E + i];
+                u[r] = cmul<float>(u[r], mk<float>(w.x, -w.y));
+            }
+        }
+        dft_reg<R1, +1, float>(u);
+        if (stores) {
+#pragma unroll
+            for (int r = 0; r < R1; ++r) out[(i + r * E) * W] = u[r];
+        }
+    }
+}
+
+// The y pass of one tile and PZ z-planes (F = PZ W transforms, PZ >= 4: a half
+// warp's accesses are one row of the exchange buffer).
+template <int N, int DIR> __global__ void __launch_bounds__(256, 3) k3_mid(const MidArgs<float> a) {
+    using S = R3Shape<N>;
+    using C = float2;
+    constexpr int E = S::E, R1 = S::R1;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    C *TW = reinterpret_cast<C *>(smem_raw);
+    C *XCH = TW + S::TWN;
+    const SysP<float> &sp = a.sp;
+    const int F = a.PZ * W, logF = __ffs(F) - 1;
+    const int t = threadIdx.x, f = t & (F - 1), lane = t >> logF;
+    const int slot = a.slot0 + blockIdx.z, tile = blockIdx.x;
+    r3_twiddles<N>(TW, a.tw, t, blockDim.x);
+    const int kmy = a.mode == MID_INV_MASK ? a.fps[slot].kmax[1] : N;
+    const uint32_t ostride = (uint32_t)sp.nz * W;               // (a field has fewer than 2^32 values)
+    const size_t ofs = (size_t)slot * a.slot_stride + (size_t)tile * N * ostride + (size_t)blockIdx.y * F + f;
+    const C *__restrict__ in = a.in + ofs;
+    C *__restrict__ out = a.out + ofs;
+    pdl_wait();
+    pdl_trigger();
+    C v[E];
+#pragma unroll
+    for (int s = 0; s < S::BPT; ++s)
+#pragma unroll
+        for (int r = 0; r < R1; ++r) {
+            const uint32_t p = lane + s * R1 + r * E;
+            v[s * R1 + r] = DIR < 0 || abs(signed_k((int)p, N)) <= kmy ? in[p * ostride] : mk<float>(0, 0);
+        }
+#pragma unroll
+    for (int s = 0; s < S::BPT; ++s) {
+        dft_reg<R1, DIR, float>(v + s * R1);
+#pragma unroll
+        for (int r = 0; r < R1; ++r) XCH[((lane + s * R1) * R1 + r) * F + f] = v[s * R1 + r];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < E; ++r) {
+        v[r] = XCH[(lane + r * R1) * F + f];
+        if (r > 0) {
+            C w = TW[(r - 1) * R1 + lane];
+            if (DIR > 0) w.y = -w.y;
+            v[r] = cmul<float>(v[r], w);
+        }
+    }
+    dft_reg<E, DIR, float>(v);
+#pragma unroll
+    for (int r = 0; r < E; ++r) out[(uint32_t)(lane + r * R1) * ostride] = v[r];
+    if (a.inc_step && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && t == 0) *a.d_step += 1;
+}
+
+template <int N> cudaError_t launch_col3_n(const ColArgs<float> &a, int nslots, cudaStream_t st) {
+    using S = R3Shape<N>;
+    const dim3 grid((a.n_tiles + S::TILES - 1) / S::TILES, a.sp.ny / 2 + 1, nslots);
+    const size_t base = sizeof(float2) * (size_t)(S::TWN + S::CHUNKS * S::BUF);
+    if (a.mode == COL_STEP) return launch_pdl(k3_col<N, R3_STEP>, grid, S::THREADS, base + sizeof(float2) * S::CHUNKS * N * W, st, a);
+    if (a.mode == COL_FWD) return launch_pdl(k3_col<N, R3_FWD>, grid, S::THREADS, base, st, a);
+    if (a.mode == COL_INV_MASK || a.mode == COL_INV_FULL) return launch_pdl(k3_col<N, R3_INV>, grid, S::THREADS, base, st, a);
+    return cudaErrorInvalidValue;
+}
+
+template <int N> cudaError_t launch_mid3_n(const MidArgs<float> &a, int nslots, int ntiles, cudaStream_t st) {
+    using S = R3Shape<N>;
+    const int F = a.PZ * W, threads = F * S::R1;
+    if (a.PZ < 4 || (a.PZ & (a.PZ - 1)) || a.sp.nz % a.PZ || threads > 256) return cudaErrorInvalidConfiguration;
+    const dim3 grid(ntiles, a.sp.nz / a.PZ, nslots);
+    const size_t smem = sizeof(float2) * (size_t)(S::TWN + N * F);
+    if (a.mode == MID_FWD) return launch_pdl(k3_mid<N, -1>, grid, threads, smem, st, a);
+    return launch_pdl(k3_mid<N, +1>, grid, threads, smem, st, a);
+}
+
+}  // namespace pss
