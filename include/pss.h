@@ -234,11 +234,12 @@ int pss_time_kernels(pss_system *s, int64_t n, double *avg_ms);
  *   "fast3d"      FP32 3D systems whose x side is 256, 512 or 1024 points
  *                 run their x pass on FFT groups (1, default) or on the
  *                 generic row kernel (0);
- *   "regs3d"      FP32 3D systems without product terms run the z and y
- *                 passes of 16..256 points with the points in registers (1,
- *                 default) or on the staged kernels (0; also where "col_radix"
- *                 or "col_tiles", or "mid_radix" or "mid_planes", ask for a
- *                 launch shape of theirs); they agree to FP32 rounding;
+ *   "regs3d"      FP32 3D systems without product terms run their passes of
+ *                 16..256 points with the points in registers (1, default) or
+ *                 on the staged kernels (0; also where "col_radix" or
+ *                 "col_tiles", "mid_radix" or "mid_planes", or "row_radix",
+ *                 "row_pairs", "row2_radix" or "fast3d" 0 ask for a launch
+ *                 shape of theirs); they agree to FP32 rounding;
  *   "col2_radix", "row2_radix"
  *                 radix of that path's FFT passes (8 or 16);
  *   "real_state"  every step ends with each field taken to real space and

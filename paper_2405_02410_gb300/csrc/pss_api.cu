@@ -703,11 +703,11 @@ int res_ctas(pss_system *s) {
     return c;
 }
 
-// The register z and y passes of FP32 3D systems (k3_col, k3_mid) where the
+// The register passes of FP32 3D systems (k3_col, k3_mid, k3_row) where the
 // side has their shape and no launch shape of the staged kernels is asked for.
 // Faster at every size measured (us per step, staged -> registers: 32^3 20.4 ->
-// 13.3, 64^3 pair 22.0 -> 15.7, 256 z x 64 x 32 22.0 -> 18.6, 16 z x 128 x 64
-// 22.3 -> 14.3, 256^3 pair 351 -> 282).  Product terms keep the staged kernels
+// 9.9, 64^3 pair 22.0 -> 12.1, 256 z x 64 x 32 22.2 -> 15.0, 16 z x 128 x 64
+// 22.1 -> 11.2, 256^3 pair 351 -> 246).  Product terms keep the staged kernels
 // (factors and summed spectra are modes of theirs), and so do the adjoint's modes.
 bool regs3d(const pss_system *s) {
     return s->tune_regs3d && s->prec == PSS_F32 && s->dim == 3 && !any_general(s) && !s->tune_test_timeout;
@@ -718,6 +718,18 @@ bool regs3d_col(const pss_system *s, int mode) {
 }
 bool regs3d_mid(const pss_system *s) {
     return regs3d(s) && r3_side(s->ny) && !s->tune_mid_radix && !s->tune_mid_planes;
+}
+bool regs3d_row(const pss_system *s, int mode) {
+    return regs3d(s) && r3_side(s->nx) && !s->tune_row_radix && !s->tune_row_pairs && !s->tune_row2_radix && s->tune_fast3d &&
+           (mode == ROW_FUSED || mode == ROW_R2C || mode == ROW_C2R);
+}
+// row pairs per CTA of k3_row (E points per thread): 128 threads, fewer (a
+// warp at least) where that leaves SMs without a CTA
+int row3_G(const pss_system *s) {
+    const int per = s->nx >= 128 ? s->nx / 16 : s->nx >= 32 ? s->nx / 8 : s->nx / 4;
+    int threads = 128;
+    while (threads > 32 && (long long)s->rows / 2 * per / threads * s->nslots() < 2 * s->num_sms) threads /= 2;
+    return threads / per;
 }
 // z-planes per CTA of k3_mid: 256 threads, fewer (at least four planes: whole
 // 128-byte lines) where that leaves SMs without a CTA
@@ -939,6 +951,18 @@ template <typename T> struct Seq {
         a.fac_first_factor = fac_first_factor;
         a.fac_last_factor = fac_last_factor;
         a.fac_first_term = fac_first_term;
+        if constexpr (std::is_same<T, float>::value) {
+            // (real rows that are stored on the way, the adjoint's, are a mode of k_row)
+            if (regs3d_row(s, mode) && !fac_acc && !(mode == ROW_FUSED && real_out) && !inc) {
+                a.G = row3_G(s);
+                if (timer) timer->begin(2, st);
+                cudaError_t e = launch_row3(a, nslots, st);
+                if (timer) timer->begin(2, st);
+                s->launches++;
+                if (e != cudaSuccess) return cuda_fail(s, e, "k3_row launch");
+                return PSS_OK;
+            }
+        }
         if (timer) timer->begin(2, st);
         cudaError_t e = launch_row<T>(a, nslots, st);
         if (timer) timer->begin(2, st);
@@ -1128,7 +1152,7 @@ template <typename T> struct Seq {
         }
     }
 
-    int x_pass_3d() { return fast3d_rows(s) ? row3() : row(ROW_FUSED, false, false, false, nullptr, 0); }  // B -> A
+    int x_pass_3d() { return fast3d_rows(s) && !regs3d_row(s, ROW_FUSED) ? row3() : row(ROW_FUSED, false, false, false, nullptr, 0); }  // B -> A
 
     // The explicit part of general field fi of instance inst, for the
     // sequence's one slot (section "Writing models": N = M prod_k psi_k^n_k,

@@ -213,11 +213,12 @@ template <typename T> inline cudaError_t launch_mid(const MidArgs<T> &a, int nsl
 // generic kernels (the x pass of the 3D step).
 cudaError_t launch_col2(const ColArgs<float> &a, int nslots, int ntiles, cudaStream_t st);
 cudaError_t launch_row2(const RowArgs<float> &a, int nslots, cudaStream_t st, bool tiled);
-// The register z and y passes of FP32 3D systems (k3_col, k3_mid; r3_side: the
+// The register passes of FP32 3D systems (k3_col, k3_mid, k3_row; r3_side: the
 // transform lengths they take): k3_col over a.n_tiles tiles of every pencil.
 constexpr bool r3_side(int n) { return n >= 16 && n <= 256 && (n & (n - 1)) == 0; }
 cudaError_t launch_col3(const ColArgs<float> &a, int nslots, cudaStream_t st);
 cudaError_t launch_mid3(const MidArgs<float> &a, int nslots, int ntiles, cudaStream_t st);
+cudaError_t launch_row3(const RowArgs<float> &a, int nslots, cudaStream_t st);
 // the adjoint's column part (COL_ADJ_A / _B / _BA) of an FP32 2D system with
 // 256..1024-point columns on FFT groups, one column pair per CTA
 cudaError_t launch_col2_adj(const ColArgs<float> &a, int nslots, cudaStream_t st);

@@ -1,4 +1,4 @@
-// pss_kern_regs3d.cu -- the register z and y passes of FP32 3D systems.
+// pss_kern_regs3d.cu -- the register z, y and x passes of FP32 3D systems.
 #include <type_traits>
 
 #include "pss_regs3d.cuh"
@@ -21,6 +21,16 @@ cudaError_t launch_mid3(const MidArgs<float> &a, int nslots, int ntiles, cudaStr
         case 64: return launch_mid3_n<64>(a, nslots, ntiles, st);
         case 128: return launch_mid3_n<128>(a, nslots, ntiles, st);
         case 256: return launch_mid3_n<256>(a, nslots, ntiles, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
+cudaError_t launch_row3(const RowArgs<float> &a, int nslots, cudaStream_t st) {
+    switch (a.sp.nx) {
+        case 16: return launch_row3_n<16>(a, nslots, st);
+        case 32: return launch_row3_n<32>(a, nslots, st);
+        case 64: return launch_row3_n<64>(a, nslots, st);
+        case 128: return launch_row3_n<128>(a, nslots, st);
+        case 256: return launch_row3_n<256>(a, nslots, st);
         default: return cudaErrorInvalidValue;
     }
 }

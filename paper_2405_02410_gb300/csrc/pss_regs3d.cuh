@@ -1,8 +1,8 @@
-// pss_regs3d.cuh -- the z and y passes of FP32 3D systems with their points in
+// pss_regs3d.cuh -- the passes of FP32 3D systems with their points in
 // registers (arXiv:2405.02410, section "What cuPSS calculates", Eq. timeupdate).
 //
-// k_col and k_mid stage their tiles in shared memory and run every phase from
-// there; in 3D both are bound by instructions and barriers, not by HBM (k_col
+// k_col, k_mid and k_row stage their tiles in shared memory and run every phase from
+// there; in 3D they are bound by instructions and barriers, not by HBM (k_col
 // at 256^3: 257 instructions per mode, 73 % issue-active, 35 % of the DRAM
 // rate).  Here a thread keeps E points of a transform of N = R1 E points in
 // registers: loads come straight from global memory (consecutive threads take
@@ -13,8 +13,9 @@
 // noise is drawn into shared memory while the loads are in flight, a pair of
 // columns per Philox call.  us, staged -> here: 256^3, two fields: z pass 153
 // -> 111 (466 MB: 4.2 TB/s), y inverse 52 -> 37, y forward 63 -> 52 (270 MB:
-// 5.2 TB/s), the step 351 -> 282; whole steps of 128^3 35 -> 28, 256 x 256 x 64
-// 54 -> 41, 64^3 (two fields) 22.0 -> 15.7, 32^3 20.4 -> 13.3.  Forcing 6 CTAs
+// 5.2 TB/s), x pass 104 -> 66 (225 MB: 3.4 TB/s), the step 351 -> 246; whole
+// steps of 128^3 35 -> 22, 256 x 256 x 64 54 -> 36, 64^3 (two fields) 22.0 ->
+// 12.1, 32^3 20.4 -> 9.9.  Forcing 6 CTAs
 // per SM on the step's z pass would leave 80 registers to the 64 that hold its
 // points; 5 take 96.
 #pragma once
@@ -280,6 +281,180 @@ template <int N, int DIR> __global__ void __launch_bounds__(256, 3) k3_mid(const
 #pragma unroll
     for (int r = 0; r < E; ++r) out[(uint32_t)(lane + r * R1) * ostride] = v[r];
     if (a.inc_step && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && t == 0) *a.d_step += 1;
+}
+
+// The x pass: pairs of rows a, b on one complex transform z = a + i b, as in
+// k_row (C2R of Z_k = A_k + i B_k, the power, R2C with A_k = (W_k + conj
+// W_{N-k}) / 2, B_k = (W_k - conj W_{N-k}) / (2i)).  The R1 threads of a pair
+// are neighbours in one warp, so its exchanges need no CTA barrier, and the
+// mirrored modes N - k change hands by shuffles: thread `lane` holds modes
+// lane + s R1 + r E, whose mirrors are thread R1 - lane's in reverse order
+// (thread 0's are its own, one further on).
+enum { R3_FUSED = 0, R3_R2C = 1, R3_C2R = 2 };
+
+template <int N> struct R3Row {
+    using S = R3Shape<N>;
+    // exchange buffer of a pair: the pairs of a half warp fall in different banks
+    static constexpr int BUF = (N + S::E + 15) / 16 * 16 + S::R1 % 16;
+    // index of mode N - k of thread 0, k at s R1 + r
+    static constexpr __host__ __device__ int own(int s, int r) {
+        return s == 0 ? (S::R1 - r) % S::R1 : (S::BPT - s) * S::R1 + S::R1 - 1 - r;
+    }
+};
+
+template <int N, int MODE> __global__ void __launch_bounds__(128, 6) k3_row(const RowArgs<float> a) {
+    using S = R3Shape<N>;
+    using L = R3Row<N>;
+    using C = float2;
+    constexpr int E = S::E, R1 = S::R1, H = R1 / 2;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    C *TW = reinterpret_cast<C *>(smem_raw);
+    const SysP<float> &sp = a.sp;
+    const int t = threadIdx.x, lane = t % R1, g = t / R1;
+    C *xb = TW + S::TWN + g * L::BUF;
+    const int slot = a.slot0 + blockIdx.y;
+    const int r0 = 2 * (blockIdx.x * a.G + g);                   // rows r0 and r0 + 1
+    const bool ok = r0 < sp.rows;
+    const int mirror = (t & 31 & ~(R1 - 1)) | ((R1 - lane) & (R1 - 1));
+    const size_t sofs = (size_t)slot * a.slot_stride;
+    // mode lane + s R1 + r E of row r0 (row r0 + 1: W further on); a field has fewer than 2^32 values
+    auto ofs = [&](int s, int r) {
+        const int k = lane + s * R1 + r * E;
+        return ((uint32_t)(k >> 2) * (uint32_t)sp.rows + (uint32_t)r0) * W + (uint32_t)(k & (W - 1));
+    };
+    r3_twiddles<N>(TW, a.tw, t, blockDim.x);
+    const C *TWI = TW + (R1 == E ? 0 : N);
+    __syncthreads();
+    pdl_wait();
+    pdl_trigger();
+    C v[E];
+    if constexpr (MODE != R3_R2C) {
+        const C *__restrict__ in = a.in + sofs;
+        const int kxc = MODE == R3_FUSED ? a.fps[slot].kx_cols : sp.hx;
+        C m[E / 2];                                              // Z_{N-k} for the thread that holds it
+#pragma unroll
+        for (int s = 0; s < S::BPT; ++s)
+#pragma unroll
+            for (int r = 0; r < H; ++r) {
+                C A = mk<float>(0, 0), B = A;
+                if (ok && lane + s * R1 + r * E < kxc) {
+                    const uint32_t p = ofs(s, r);
+                    A = in[p];
+                    B = in[p + W];
+                    if (s == 0 && r == 0 && lane == 0) A.y = B.y = 0.0f;
+                }
+                v[s * R1 + r] = mk<float>(A.x - B.y, A.y + B.x);
+                m[s * H + r] = mk<float>(A.x + B.y, B.x - A.y);
+            }
+#pragma unroll
+        for (int s = 0; s < S::BPT; ++s)
+#pragma unroll
+            for (int r = H; r < R1; ++r) {
+                const C x = m[(S::BPT - 1 - s) * H + R1 - 1 - r];
+                C z = mk<float>(__shfl_sync(0xffffffffu, x.x, mirror), __shfl_sync(0xffffffffu, x.y, mirror));
+                if (s == 0 && r == H) {
+                    if (lane == 0) {
+                        z = mk<float>(0, 0);
+                        if (ok && N / 2 < kxc) {
+                            const uint32_t p = ofs(0, H);
+                            z = mk<float>(in[p].x, in[p + W].x);
+                        }
+                    }
+                } else if (lane == 0) {
+                    z = m[s == 0 ? R1 - r : (S::BPT - s) * H + R1 - 1 - r];
+                }
+                v[s * R1 + r] = z;
+            }
+#pragma unroll
+        for (int s = 0; s < S::BPT; ++s) {
+            dft_reg<R1, +1, float>(v + s * R1);
+#pragma unroll
+            for (int r = 0; r < R1; ++r) xb[(lane + s * R1) * (R1 + 1) + r] = v[s * R1 + r];
+        }
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+            v[r] = xb[lane + r * (R1 + 1)];
+            if (r > 0) {
+                const C w = TW[(r - 1) * R1 + lane];
+                v[r] = cmul<float>(v[r], mk<float>(w.x, -w.y));
+            }
+        }
+        dft_reg<E, +1, float>(v);                                // sites lane + r R1
+    }
+    if constexpr (MODE == R3_FUSED) {
+        const int p = a.fps[slot].power;
+        if (p == 3) {
+#pragma unroll
+            for (int r = 0; r < E; ++r) v[r] = mk<float>(v[r].x * v[r].x * v[r].x, v[r].y * v[r].y * v[r].y);
+        } else {
+#pragma unroll
+            for (int r = 0; r < E; ++r) v[r] = mk<float>(ipow<float>(v[r].x, p), ipow<float>(v[r].y, p));
+        }
+    } else if (ok) {
+        const size_t ra = (size_t)slot * a.real_stride + real_row_offset(sp, r0) + lane;
+        const size_t rb = (size_t)slot * a.real_stride + real_row_offset(sp, r0 + 1) + lane;
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+            if (MODE == R3_C2R) {
+                a.real_out[ra + r * R1] = v[r].x;
+                a.real_out[rb + r * R1] = v[r].y;
+            } else {
+                v[r] = mk<float>(a.real_in[ra + r * R1], a.real_in[rb + r * R1]);
+            }
+        }
+    } else if (MODE == R3_R2C) {
+#pragma unroll
+        for (int r = 0; r < E; ++r) v[r] = mk<float>(0, 0);
+    }
+    if constexpr (MODE != R3_C2R) {
+        dft_reg<E, -1, float>(v);
+        __syncwarp();                                            // the buffer is free again
+#pragma unroll
+        for (int r = 0; r < E; ++r) xb[lane * (E + 1) + r] = v[r];
+        __syncwarp();
+#pragma unroll
+        for (int s = 0; s < S::BPT; ++s) {
+            const int i = lane + s * R1;
+#pragma unroll
+            for (int r = 0; r < R1; ++r) {
+                v[s * R1 + r] = xb[i + r * (E + 1)];
+                if (r > 0) v[s * R1 + r] = cmul<float>(v[s * R1 + r], TWI[(r - 1) * E + i]);
+            }
+            dft_reg<R1, -1, float>(v + s * R1);
+        }
+        C *__restrict__ out = a.out + sofs;
+#pragma unroll
+        for (int s = 0; s < S::BPT; ++s)
+#pragma unroll
+            for (int r = 0; r < H; ++r) {
+                const C x = v[s * R1 + r], y = v[E - 1 - (s * R1 + r)];
+                C z = mk<float>(__shfl_sync(0xffffffffu, y.x, mirror), __shfl_sync(0xffffffffu, y.y, mirror));
+                if (lane == 0) z = v[L::own(s, r)];
+                if (ok) {
+                    const uint32_t p = ofs(s, r);
+                    out[p] = mk<float>(0.5f * (x.x + z.x), 0.5f * (x.y - z.y));
+                    out[p + W] = mk<float>(0.5f * (x.y + z.y), -0.5f * (x.x - z.x));
+                }
+            }
+        if (ok && lane < W) {                                    // mode N / 2 and the last tile's padding
+            const uint32_t p = ofs(0, H);
+            out[p] = mk<float>(lane == 0 ? v[H].x : 0.0f, 0.0f);
+            out[p + W] = mk<float>(lane == 0 ? v[H].y : 0.0f, 0.0f);
+        }
+    }
+}
+
+template <int N> cudaError_t launch_row3_n(const RowArgs<float> &a, int nslots, cudaStream_t st) {
+    using S = R3Shape<N>;
+    const int threads = a.G * S::R1;
+    if (threads % 32 || threads > 128 || a.sp.rows % 2) return cudaErrorInvalidConfiguration;
+    const dim3 grid((a.sp.rows / 2 + a.G - 1) / a.G, nslots);
+    const size_t smem = sizeof(float2) * (size_t)(S::TWN + a.G * R3Row<N>::BUF);
+    if (a.mode == ROW_FUSED) return launch_pdl(k3_row<N, R3_FUSED>, grid, threads, smem, st, a);
+    if (a.mode == ROW_R2C) return launch_pdl(k3_row<N, R3_R2C>, grid, threads, smem, st, a);
+    if (a.mode == ROW_C2R) return launch_pdl(k3_row<N, R3_C2R>, grid, threads, smem, st, a);
+    return cudaErrorInvalidValue;
 }
 
 template <int N> cudaError_t launch_col3_n(const ColArgs<float> &a, int nslots, cudaStream_t st) {

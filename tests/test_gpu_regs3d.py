@@ -1,6 +1,6 @@
-"""The register z and y passes of FP32 3D systems (tuning key "regs3d") against
+"""The register z, y and x passes of FP32 3D systems (tuning key "regs3d") against
 the staged kernels over the sides, orders, operators and batches the rule that
-selects them accepts (and sides where only one of the two passes is taken),
+selects them accepts (and sides where only some of the passes are taken),
 and against the oracle.
 
 Bars: rel-L2 <= 1e-5 against the staged kernels (FP32 rounding of two transform
@@ -60,6 +60,8 @@ def _results(s, fields):
     ((128, 16, 32), dict(order=0)), ((256, 8, 16), dict(noisy=False)), ((4, 256, 8), {}), ((8, 128, 64), dict(fields=2)),
     ((64, 128, 4), dict(batch=3, fields=2)), ((512, 16, 4), {}), ((16, 512, 4), {}), ((32, 32, 64), dict(power=0)),
     ((16, 32, 128), dict(power=2, order=1)), ((256, 64, 32), dict(fields=2)),
+    ((8, 4, 256), dict(order=0)), ((16, 16, 512), {}), ((4, 4, 32), dict(power=1, order=4)), ((4, 8, 16), dict(batch=2)),
+    ((16, 64, 256), dict(fields=2)),
 ])
 def test_against_the_staged_kernels(shape, kw):
     fields = kw.get("fields", 1)
