@@ -234,12 +234,15 @@ int pss_time_kernels(pss_system *s, int64_t n, double *avg_ms);
  *   "fast3d"      FP32 3D systems whose x side is 256, 512 or 1024 points
  *                 run their x pass on FFT groups (1, default) or on the
  *                 generic row kernel (0);
- *   "regs3d"      FP32 3D systems without product terms run their passes of
- *                 16..256 points with the points in registers (1, default) or
- *                 on the staged kernels (0; also where "col_radix" or
- *                 "col_tiles", "mid_radix" or "mid_planes", or "row_radix",
- *                 "row_pairs", "row2_radix" or "fast3d" 0 ask for a launch
- *                 shape of theirs); they agree to FP32 rounding;
+ *   "regs"        FP32 2D and 3D passes with their points in registers (1,
+ *                 default) or the staged kernels (0): 3D systems without
+ *                 product terms, sides of 16..256 points; 2D systems of 16..1024
+ *                 points a side for fields in and out, and for the steps of
+ *                 those with enough sites to fill the GPU (2: of all but
+ *                 product terms and frames, where no run-in-one-launch path
+ *                 takes them).  The launch-shape keys of the staged kernels
+ *                 select those where they are set.  The two agree to FP32
+ *                 rounding;
  *   "col2_radix", "row2_radix"
  *                 radix of that path's FFT passes (8 or 16);
  *   "real_state"  every step ends with each field taken to real space and

@@ -17,10 +17,10 @@ LIBDIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(LIBDIR, "libpss.so")
 SOURCES = ["pss_api.cu", "pss_kern_f32.cu", "pss_kern_f64.cu", "pss_kern_f32_r16.cu", "pss_kern_f64_r16.cu", "pss_kern_f64_r4.cu", "pss_kern_f64_r2.cu",
            "pss_kern_fast2d.cu", "pss_kern_persist.cu", "pss_kern_persist_kpz.cu", "pss_kern_persist_adj.cu",
-           "pss_kern_line_f32.cu", "pss_kern_line_f64.cu", "pss_kern_terms_f32.cu", "pss_kern_regs3d.cu",
+           "pss_kern_line_f32.cu", "pss_kern_line_f64.cu", "pss_kern_terms_f32.cu", "pss_kern_regs.cu",
            *[f"pss_kern_res2d_{n}.cu" for n in (32, 64, 128, 256, 512)]]
 HEADERS = ["pss_device.cuh", "pss_internal.h", "pss_kernels.cuh", "pss_fast2d.cuh", "pss_persist2d.cuh", "pss_adj2d.cuh", "pss_persist_adj.cuh",
-           "pss_resident2d.cuh", "pss_line.cuh", "pss_terms.cuh", "pss_regs3d.cuh"]
+           "pss_resident2d.cuh", "pss_line.cuh", "pss_terms.cuh", "pss_regs.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-fno-strict-aliasing",
               "--expt-relaxed-constexpr"]

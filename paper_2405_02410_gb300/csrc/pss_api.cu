@@ -146,7 +146,7 @@ struct pss_system {
     int tune_adj_radix = 0;                  // FFT radix of that backward pass (8 or 16; 0: the forward's)
     int tune_persist_adj = 1;                // FP32 2D adjoint on the persistent path: a segment's backward pass in one launch                   // FP32 2D adjoint: column parts on FFT groups (0: generic kernel)
     int tune_fuse_terms = 1;                 // FP32 1D/2D product terms in one row kernel (0: factor by factor)
-    int tune_regs3d = 1;                     // FP32 3D: z and y passes with their points in registers (0: staged kernels)
+    int tune_regs = 1;                       // FP32 2D and 3D: passes with their points in registers (0: staged kernels; 2: all 2D systems they take)
     int tune_resident = 1;                   // FP32 2D sides of 32..512: a run of steps with every slot in one cluster
     int tune_res_ctas = 0;                   // its CTAs per cluster (0 = automatic)
     int res_ctas_auto = 0, res_ctas_slots = 0;   // the automatic choice, for that many slots
@@ -552,10 +552,36 @@ int mid_PZ(const pss_system *s) {
 // The FP32 2D path with one warp per transform serves sides of 256, 512 and
 // 1024 points; everything else runs the generic kernels.
 
-bool fast2d(const pss_system *s) {
+bool round_trip(const pss_system *s);
+bool side_res(int n);
+bool fast2d_shape(const pss_system *s) {
     auto side = [](int n) { return n == 256 || n == 512 || n == 1024; };
     return s->tune_fast2d && s->prec == PSS_F32 && s->dim == 2 && side(s->nx) && side(s->ny) && !any_general(s);
 }
+// The register passes (k3_col, k3_row) are what FP32 2D systems step with where
+// there are enough sites to fill the chip with them: 512 and 1024 points take
+// 32 of them per thread, so a launch lasts about 10 us however small.  us per
+// step, the FFT-group kernels (or cluster-resident run) -> here: 512^2 x 8 24.0
+// -> 24.8, x 12 34.3 -> 28.2, x 32 85 -> 68; 512 x 256 x 16 23.2 -> 22.2, x 32
+// 40 -> 32; 256^2 x 32 17.8 -> 17.4, x 64 35 -> 28, x 128 70 -> 48; with a side
+// of 1024 from fewer sites on: 1024 x 512 x 2 20 -> 24, x 3 30 -> 24, 1024^2 x 2
+// 29.5 -> 25.5, x 8 107 -> 67; against the generic kernels (a side of 1024, the
+// other below 256) 1024 x 128 x 8 18.3 -> 18.2, x 16 29.4 -> 22.5, 128 x 1024 x
+// 32 54 -> 29.  One field of one instance (the adjoint's systems) stays below
+// these.
+bool r3_side(int n) { return n >= 16 && n <= 1024; }
+bool regs2d_step(const pss_system *s) {
+    if (!(s->tune_regs && s->prec == PSS_F32 && s->dim == 2 && r3_side(s->nx) && r3_side(s->ny) && !any_general(s) &&
+          !round_trip(s) && !s->tune_test_timeout && !s->tune_col_radix && !s->tune_col_tiles && !s->tune_row_radix &&
+          !s->tune_row_pairs && !s->tune_col2_radix && !s->tune_row2_radix && !s->tune_col2_warps && !s->tune_row2_pairs &&
+          !s->tune_row2_noise))
+        return false;
+    if (s->tune_regs > 1) return true;
+    const long long sites = s->nsites * s->nslots();
+    if (fast2d_shape(s)) return std::max(s->nx, s->ny) == 1024 ? sites >= 3ll << 19 : sites > 1ll << 21;
+    return !(side_res(s->nx) && side_res(s->ny)) && sites >= 1ll << 20;
+}
+bool fast2d(const pss_system *s) { return fast2d_shape(s) && !regs2d_step(s); }
 // Launch shape of the fast path, measured on GB300.  2D: radix-16 passes for
 // sides of 512 and 1024 (two warps per 1024-point transform, three passes),
 // radix 8 for 256 (one warp per transform: the 256^2 step is latency-bound,
@@ -563,7 +589,6 @@ bool fast2d(const pss_system *s) {
 // pass takes radix 16 at every side: at 256 points that is half a warp per
 // transform and two passes instead of three, and there the passes are bound
 // by shared-memory bandwidth (x pass of the 256^3 pair 130 -> 113 us).
-bool round_trip(const pss_system *s);
 
 // A run of steps of a square FP32 2D system with one field and one instance
 // on the FFT-group path is one persistent launch (k2p_step), where the
@@ -638,14 +663,15 @@ int res_active(const pss_system *s, int C) {
 // 512 x 128 12.6 -> 8.4).  With both sides of 256 or more the two-kernel step
 // spreads one slot over the whole chip: 256^2 x 8 8.8 -> 10.1, x 32 20.7 ->
 // 17.6, x 128 73 -> 68, 512 x 256 8.2 -> 12.2, 512^2 x 32 85 -> 100; only
-// 256^2 gains, when its clusters of four fill most of the chip (36 at a time).
+// 256^2 gains, when its clusters of four fill most of the chip (36 at a time) and
+// there are too few sites for the register passes.
 constexpr int kRes256Fill = 29;   // slots per wave of 256^2 clusters from which it gains
 bool resident2d(const pss_system *s) {
     if (!(s->tune_resident && s->tune_fast2d && s->prec == PSS_F32 && s->dim == 2 && side_res(s->nx) &&
           side_res(s->ny) && !any_general(s) && !round_trip(s) && !s->tune_test_timeout))
         return false;
     if (s->nx < 256 || s->ny < 256) return true;
-    if (s->nx != 256 || s->ny != 256 || s->nslots() < kRes256Fill) return false;
+    if (s->nx != 256 || s->ny != 256 || s->nslots() < kRes256Fill || regs2d_step(s)) return false;
     if (s->res256_slots != s->nslots()) {
         const int active = res_active(s, 4);
         s->res256_on = active > 0 && s->nslots() >= kRes256Fill * ((s->nslots() + active - 1) / active);
@@ -703,38 +729,53 @@ int res_ctas(pss_system *s) {
     return c;
 }
 
-// The register passes of FP32 3D systems (k3_col, k3_mid, k3_row) where the
-// side has their shape and no launch shape of the staged kernels is asked for.
-// Faster at every size measured (us per step, staged -> registers: 32^3 20.4 ->
-// 9.9, 64^3 pair 22.0 -> 12.1, 256 z x 64 x 32 22.2 -> 15.0, 16 z x 128 x 64
-// 22.1 -> 11.2, 256^3 pair 351 -> 246).  Product terms keep the staged kernels
-// (factors and summed spectra are modes of theirs), and so do the adjoint's modes.
-bool regs3d(const pss_system *s) {
-    return s->tune_regs3d && s->prec == PSS_F32 && s->dim == 3 && !any_general(s) && !s->tune_test_timeout;
+// The register passes of FP32 2D and 3D systems (k3_col, k3_mid, k3_row) where
+// the side has their shape and no launch shape of the staged kernels is asked
+// for.  3D: faster at every size measured (us per step, staged -> registers: 32^3
+// 20.4 -> 9.9, 64^3 pair 22.0 -> 12.1, 256 z x 64 x 32 22.2 -> 15.0, 16 z x 128
+// x 64 22.1 -> 11.2, 256^3 pair 351 -> 246).  2D: the step by regs2d_step, and
+// fields in and out at every size (set_field: 256^2 12.4 -> 8.5, 1024 x 64 14.5
+// -> 10.5, 512^2 12.5 -> 12.7, 1024^2 16.5 -> 14.6).  Product terms evaluated
+// factor by factor keep the staged kernels (factors and summed spectra are
+// modes of theirs), and so do the adjoint's modes.
+bool regs(const pss_system *s) {
+    return s->tune_regs && s->prec == PSS_F32 && s->dim >= 2 && !s->tune_test_timeout && (!any_general(s) || fused_terms(s));
 }
-bool regs3d_col(const pss_system *s, int mode) {
-    return regs3d(s) && r3_side(s->nz) && !s->tune_col_radix && !s->tune_col_tiles && mode != COL_ADJ_A &&
-           mode != COL_ADJ_B && mode != COL_ADJ_BA;
+// (3D sides above 256 points keep theirs: measured up to there)
+bool r3_side_of(const pss_system *s, int n) { return r3_side(n) && (s->dim == 2 || n <= 256); }
+bool regs_col(const pss_system *s, int mode) {
+    return regs(s) && r3_side_of(s, s->n_inner) && !s->tune_col_radix && !s->tune_col_tiles &&
+           (mode == COL_FWD || mode == COL_INV_FULL ||
+            ((mode == COL_STEP || mode == COL_INV_MASK) && (s->dim == 3 ? !any_general(s) : regs2d_step(s))));
 }
-bool regs3d_mid(const pss_system *s) {
-    return regs3d(s) && r3_side(s->ny) && !s->tune_mid_radix && !s->tune_mid_planes;
+bool regs_mid(const pss_system *s) {
+    return regs(s) && r3_side_of(s, s->ny) && !s->tune_mid_radix && !s->tune_mid_planes;
 }
-bool regs3d_row(const pss_system *s, int mode) {
-    return regs3d(s) && r3_side(s->nx) && !s->tune_row_radix && !s->tune_row_pairs && !s->tune_row2_radix && s->tune_fast3d &&
-           (mode == ROW_FUSED || mode == ROW_R2C || mode == ROW_C2R);
+bool regs_row(const pss_system *s, int mode) {
+    return regs(s) && r3_side_of(s, s->nx) && !s->tune_row_radix && !s->tune_row_pairs && !s->tune_row2_radix &&
+           (s->dim == 2 || s->tune_fast3d) &&
+           (mode == ROW_R2C || mode == ROW_C2R || (mode == ROW_FUSED && (s->dim == 3 || regs2d_step(s))));
 }
-// row pairs per CTA of k3_row (E points per thread): 128 threads, fewer (a
-// warp at least) where that leaves SMs without a CTA
-int row3_G(const pss_system *s) {
-    const int per = s->nx >= 128 ? s->nx / 16 : s->nx >= 32 ? s->nx / 8 : s->nx / 4;
+// Threads per CTA of k3_col and k3_row for `units` transforms (pairs of pencils
+// in 3D) of `per` threads: 128, fewer (whole warps) where that leaves SMs without
+// a CTA
+int r3_per(int n) { return n >= 512 ? n / 32 : n >= 128 ? n / 16 : n >= 32 ? n / 8 : n / 4; }
+int r3_threads(const pss_system *s, int per, long long units) {
     int threads = 128;
-    while (threads > 32 && (long long)s->rows / 2 * per / threads * s->nslots() < 2 * s->num_sms) threads /= 2;
-    return threads / per;
+    while (threads > 32 && threads > per && units * per / threads < 2 * s->num_sms) threads /= 2;
+    return threads;
+}
+int col3_threads(const pss_system *s, int n_tiles, int nslots) {
+    if (s->dim == 3) return 128;
+    return r3_threads(s, kTileW * r3_per(s->n_inner), (long long)n_tiles * nslots);
+}
+int row3_G(const pss_system *s, int nslots) {
+    return r3_threads(s, r3_per(s->nx), (long long)s->rows / 2 * nslots) / r3_per(s->nx);
 }
 // z-planes per CTA of k3_mid: 256 threads, fewer (at least four planes: whole
 // 128-byte lines) where that leaves SMs without a CTA
 int mid3_PZ(const pss_system *s) {
-    int pz = std::min(s->nz, 64 / (s->ny >= 128 ? s->ny / 16 : s->ny >= 32 ? s->ny / 8 : s->ny / 4));
+    int pz = std::min(s->nz, 64 / r3_per(s->ny));
     while (pz > 4 && (long long)s->ntiles * (s->nz / pz) * s->nslots() < 2 * s->num_sms) pz /= 2;
     return pz;
 }
@@ -902,7 +943,8 @@ template <typename T> struct Seq {
             }
         }
         if constexpr (std::is_same<T, float>::value) {
-            if (regs3d_col(s, mode) && !op_on) {
+            if (regs_col(s, mode) && !op_on) {
+                a.F = col3_threads(s, a.n_tiles, nslots);
                 if (timer) timer->begin(0, st);
                 cudaError_t e = launch_col3(a, nslots, st);
                 if (timer) timer->begin(0, st);
@@ -953,8 +995,8 @@ template <typename T> struct Seq {
         a.fac_first_term = fac_first_term;
         if constexpr (std::is_same<T, float>::value) {
             // (real rows that are stored on the way, the adjoint's, are a mode of k_row)
-            if (regs3d_row(s, mode) && !fac_acc && !(mode == ROW_FUSED && real_out) && !inc) {
-                a.G = row3_G(s);
+            if (regs_row(s, mode) && !fac_acc && !(mode == ROW_FUSED && real_out)) {
+                a.G = row3_G(s, nslots);
                 if (timer) timer->begin(2, st);
                 cudaError_t e = launch_row3(a, nslots, st);
                 if (timer) timer->begin(2, st);
@@ -991,7 +1033,7 @@ template <typename T> struct Seq {
         const int nt = mode == MID_INV_MASK ? max_kept_tiles(s) : s->ntiles;
         const int kind = mode == MID_FWD ? 3 : 1;
         if constexpr (std::is_same<T, float>::value) {
-            if (regs3d_mid(s)) {
+            if (regs_mid(s)) {
                 a.PZ = mid3_PZ(s);
                 if (timer) timer->begin(kind, st);
                 cudaError_t e = launch_mid3(a, nslots, nt, st);
@@ -1152,7 +1194,7 @@ template <typename T> struct Seq {
         }
     }
 
-    int x_pass_3d() { return fast3d_rows(s) && !regs3d_row(s, ROW_FUSED) ? row3() : row(ROW_FUSED, false, false, false, nullptr, 0); }  // B -> A
+    int x_pass_3d() { return fast3d_rows(s) && !regs_row(s, ROW_FUSED) ? row3() : row(ROW_FUSED, false, false, false, nullptr, 0); }  // B -> A
 
     // The explicit part of general field fi of instance inst, for the
     // sequence's one slot (section "Writing models": N = M prod_k psi_k^n_k,
@@ -2705,7 +2747,7 @@ int pss_set_tuning(pss_system *s, const char *key, int value) {
     else if (k == "graph_steps") s->tune_graph_steps = value;
     else if (k == "fast2d") s->tune_fast2d = value ? 1 : 0;
     else if (k == "fast3d") s->tune_fast3d = value ? 1 : 0;
-    else if (k == "regs3d") s->tune_regs3d = value ? 1 : 0;
+    else if (k == "regs") s->tune_regs = std::min(value, 2);
     else if (k == "fuse_adjoint") s->tune_fuse_adj = value ? 1 : 0;
     else if (k == "real_state") s->tune_real_state = value ? 1 : 0;
     else if (k == "test_timeout") s->tune_test_timeout = value ? 1 : 0;
@@ -2779,7 +2821,7 @@ struct TuneKnob {
 std::vector<TuneKnob> tune_space(const pss_system *s) {
     std::vector<TuneKnob> k;
     const auto radix_list = [](int side) { return side == 1024 ? std::vector<int>{8, 16, 32} : std::vector<int>{8, 16}; };
-    if (fast2d(s)) {
+    if (fast2d_shape(s)) {
         // the persistent launch against the two-kernel step, where the system qualifies
         if (persist2d_ok(s)) k.push_back({"persist", &pss_system::tune_persist, {1, 0}});
         k.push_back({"col2_radix", &pss_system::tune_col2_radix, radix_list(s->ny)});
@@ -3270,7 +3312,7 @@ const char *pss_last_error(const pss_system *s) { return s ? s->err.c_str() : g_
 int64_t pss_launch_count(const pss_system *s) { return s ? s->launches : 0; }
 
 int pss_step_path(const pss_system *s) {
-    return s ? (persist2d(s) ? 3 : fast2d(s) ? 1 : fast3d_rows(s) ? 2 : 0) : PSS_EINVAL;
+    return s ? (persist2d(s) ? 3 : fast2d_shape(s) ? 1 : fast3d_rows(s) ? 2 : 0) : PSS_EINVAL;
 }
 
 }  // extern "C"

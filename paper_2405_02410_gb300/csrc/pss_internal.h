@@ -213,9 +213,8 @@ template <typename T> inline cudaError_t launch_mid(const MidArgs<T> &a, int nsl
 // generic kernels (the x pass of the 3D step).
 cudaError_t launch_col2(const ColArgs<float> &a, int nslots, int ntiles, cudaStream_t st);
 cudaError_t launch_row2(const RowArgs<float> &a, int nslots, cudaStream_t st, bool tiled);
-// The register passes of FP32 3D systems (k3_col, k3_mid, k3_row; r3_side: the
-// transform lengths they take): k3_col over a.n_tiles tiles of every pencil.
-constexpr bool r3_side(int n) { return n >= 16 && n <= 256 && (n & (n - 1)) == 0; }
+// The register passes of FP32 2D and 3D systems: k3_col (a.F threads per CTA)
+// over a.n_tiles tiles of every pencil, k3_mid, k3_row
 cudaError_t launch_col3(const ColArgs<float> &a, int nslots, cudaStream_t st);
 cudaError_t launch_mid3(const MidArgs<float> &a, int nslots, int ntiles, cudaStream_t st);
 cudaError_t launch_row3(const RowArgs<float> &a, int nslots, cudaStream_t st);

@@ -1,16 +1,18 @@
-// pss_kern_regs3d.cu -- the register z, y and x passes of FP32 3D systems.
+// pss_kern_regs3d.cu -- the register passes of FP32 2D and 3D systems.
 #include <type_traits>
 
-#include "pss_regs3d.cuh"
+#include "pss_regs.cuh"
 
 namespace pss {
 cudaError_t launch_col3(const ColArgs<float> &a, int nslots, cudaStream_t st) {
-    switch (a.sp.nz) {
+    switch (a.sp.n_inner) {
         case 16: return launch_col3_n<16>(a, nslots, st);
         case 32: return launch_col3_n<32>(a, nslots, st);
         case 64: return launch_col3_n<64>(a, nslots, st);
         case 128: return launch_col3_n<128>(a, nslots, st);
         case 256: return launch_col3_n<256>(a, nslots, st);
+        case 512: return launch_col3_n<512>(a, nslots, st);
+        case 1024: return launch_col3_n<1024>(a, nslots, st);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -31,6 +33,8 @@ cudaError_t launch_row3(const RowArgs<float> &a, int nslots, cudaStream_t st) {
         case 64: return launch_row3_n<64>(a, nslots, st);
         case 128: return launch_row3_n<128>(a, nslots, st);
         case 256: return launch_row3_n<256>(a, nslots, st);
+        case 512: return launch_row3_n<512>(a, nslots, st);
+        case 1024: return launch_row3_n<1024>(a, nslots, st);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -1,9 +1,9 @@
-// pss_regs3d.cuh -- the passes of FP32 3D systems with their points in
+// pss_regs.cuh -- the passes of FP32 2D and 3D systems with their points in
 // registers (arXiv:2405.02410, section "What cuPSS calculates", Eq. timeupdate).
 //
 // k_col, k_mid and k_row stage their tiles in shared memory and run every phase from
-// there; in 3D they are bound by instructions and barriers, not by HBM (k_col
-// at 256^3: 257 instructions per mode, 73 % issue-active, 35 % of the DRAM
+// there; they are bound by instructions and barriers, not by HBM (k_col at
+// 256^3: 257 instructions per mode, 73 % issue-active, 35 % of the DRAM
 // rate).  Here a thread keeps E points of a transform of N = R1 E points in
 // registers: loads come straight from global memory (consecutive threads take
 // a tile's columns and neighbouring positions, whole 128-byte lines), a
@@ -15,9 +15,13 @@
 // -> 111 (466 MB: 4.2 TB/s), y inverse 52 -> 37, y forward 63 -> 52 (270 MB:
 // 5.2 TB/s), x pass 104 -> 66 (225 MB: 3.4 TB/s), the step 351 -> 246; whole
 // steps of 128^3 35 -> 22, 256 x 256 x 64 54 -> 36, 64^3 (two fields) 22.0 ->
-// 12.1, 32^3 20.4 -> 9.9.  Forcing 6 CTAs
-// per SM on the step's z pass would leave 80 registers to the 64 that hold its
-// points; 5 take 96.
+// 12.1, 32^3 20.4 -> 9.9; 2D batches against the FFT-group kernels: 512^2 x 32
+// 85 -> 68, 1024^2 x 8 107 -> 67.  The step's column pass takes 5 CTAs per SM and
+// 96 registers, the state among them; 6 CTAs and 80 registers with the state
+// copied to shared memory asynchronously measured 118 .. 126 us at 256^3 in place
+// of 111.  512 and 1024 points put 32 points on a thread, so there the state
+// goes through shared memory with the noise.
+
 #pragma once
 
 #include "pss_kernels.cuh"
@@ -27,15 +31,15 @@ namespace pss {
 // N = R1 E: R1 threads per transform, E points each; passes of radix R1 (the
 // forward transform's first, BPT butterflies per thread) and E
 template <int N> struct R3Shape {
-    static constexpr int E = N >= 128 ? 16 : N >= 32 ? 8 : 4;
+    static constexpr int E = N >= 512 ? 32 : N >= 128 ? 16 : N >= 32 ? 8 : 4;
     static constexpr int R1 = N / E;
     static constexpr int BPT = E / R1;
-    static constexpr int TILES = 16 / R1;                // k3_col: tiles per CTA
-    static constexpr int THREADS = 8 * TILES * R1;       //   two pencils of each, 128 threads
-    static constexpr int CHUNKS = 2 * TILES;
-    static constexpr int BUF = (N + E) * W;              //   exchange buffer of one chunk, one pad position per butterfly
+    static constexpr int CHUNK = W * R1;                 // k3_col: threads per chunk (a tile of a pencil)
+    static constexpr int BUF = (N + E) * W;              //   its exchange buffer, one pad position per butterfly
     static constexpr int TWN = R1 == E ? N : 2 * N;      // twiddles [r - 1][k] of the radix-E pass, of the radix-R1 one
-    static_assert(R1 <= E && THREADS == 128, "shape");
+    static constexpr bool ALIAS = N >= 512;              //   which then takes the state and noise as well
+    static constexpr int CTAS = N >= 512 ? 4 : 6;        // CTAs of 128 threads per SM the registers are held to
+    static_assert(R1 <= E && CHUNK <= 128, "shape");
 };
 
 // twiddles exp(-2 pi i r k / N): of the radix-E pass after R1 points [r - 1][k < R1], and of
@@ -55,40 +59,48 @@ template <int N> __device__ __forceinline__ void r3_twiddles(float2 *TW, const f
 // Modes of k3_col: the step, forward only (COL_FWD), inverse only (COL_INV_MASK, COL_INV_FULL)
 enum { R3_STEP = 0, R3_FWD = 1, R3_INV = 2 };
 
-// The z pass.  A CTA takes TILES tiles of the pencils ky and -ky (a kx = 0 mode
-// and its Hermitian partner are in one CTA); thread: column c, lane, chunk.
-template <int N, int MODE> __global__ void __launch_bounds__(128, MODE == R3_STEP ? 5 : 6) k3_col(const ColArgs<float> a) {
+// The z pass in 3D, the y pass in 2D.  A CTA takes tiles (in 3D of the pencils
+// ky and -ky: a kx = 0 mode and its Hermitian partner are in one CTA), a chunk
+// of CHUNK threads for each; thread: column c, lane, chunk.
+template <int N, int MODE, int DIM>
+__global__ void __launch_bounds__(128, MODE == R3_STEP && N < 512 ? 5 : R3Shape<N>::CTAS) k3_col(const ColArgs<float> a) {
     using S = R3Shape<N>;
     using C = float2;
     constexpr int E = S::E, R1 = S::R1;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ FieldP<float> fp;
+    const SysP<float> &sp = a.sp;
+    constexpr bool is3 = DIM == 3;
+    const int nthr = is3 ? 128 : blockDim.x;
+    const int t = threadIdx.x, c = t & (W - 1), lane = (t >> 2) % R1, ch = t / S::CHUNK;
+    const int chunks = nthr / S::CHUNK, ctiles = is3 ? chunks >> 1 : chunks;
     C *TW = reinterpret_cast<C *>(smem_raw);
     C *XCH = TW + S::TWN;
-    C *XI = XCH + S::CHUNKS * S::BUF;                            // R3_STEP: the noise, [chunk][pos][W]
-    const SysP<float> &sp = a.sp;
-    const int t = threadIdx.x, c = t & (W - 1), lane = (t >> 2) % R1, ch = t / (W * R1);
+    C *XI = S::ALIAS ? XCH : XCH + chunks * S::BUF;              // R3_STEP: the noise (ALIAS: plus the state), [chunk][pos][W]
+    constexpr int XS = S::ALIAS ? S::BUF : N * W;
     const int slot = a.slot0 + blockIdx.z;
-    const int op = blockIdx.y, opp = (sp.ny - op) & (sp.ny - 1);
-    const bool lone = op == opp;                                 // its own partner: the second chunk is a copy
-    const int first_tile = blockIdx.x * S::TILES, tile = first_tile + (ch >> 1);
-    const int o = (ch & 1) ? opp : op, kx = tile * W + c;
+    const int op = blockIdx.y, opp = (sp.n_outer - op) & (sp.n_outer - 1);
+    const bool lone = is3 && op == opp;                          // its own partner: the second chunk is a copy
+    const int first_tile = blockIdx.x * ctiles, tile = first_tile + (is3 ? ch >> 1 : ch);
+    const int o = is3 && (ch & 1) ? opp : op, kx = tile * W + c;
     const bool ok = tile < a.n_tiles, writes = ok && !((ch & 1) && lone);
-    const size_t ofs = (size_t)slot * a.slot_stride + ((size_t)tile * sp.ny + o) * N * W + c;
+    const size_t ofs = (size_t)slot * a.slot_stride + ((size_t)tile * sp.n_outer + o) * N * W + c;
     C *xb = XCH + ch * S::BUF + c;
-    r3_twiddles<N>(TW, a.tw, t, S::THREADS);
-    for (int i = t; i < (int)(sizeof(FieldP<float>) / 4); i += S::THREADS)
+    r3_twiddles<N>(TW, a.tw, t, nthr);
+    for (int i = t; i < (int)(sizeof(FieldP<float>) / 4); i += nthr)
         reinterpret_cast<uint32_t *>(&fp)[i] = reinterpret_cast<const uint32_t *>(&a.fps[slot])[i];
     __syncthreads();
-    const int oy = signed_k(o, sp.ny);
+    const int oy = is3 ? signed_k(o, sp.ny) : 0;                 // ky of the pencil
     const bool full = a.mode == COL_INV_FULL;
+    auto kept_o = [&](int k) { return !is3 || abs(signed_k(k, sp.ny)) <= fp.kmax[1]; };
     // CTA-uniform: nothing of the inverse is kept
-    const bool inverse = MODE != R3_FWD && (full || (first_tile * W <= fp.kmax[0] && abs(signed_k(op, sp.ny)) <= fp.kmax[1]));
+    const bool inverse = MODE != R3_FWD && (full || (first_tile * W <= fp.kmax[0] && kept_o(op)));
     pdl_wait();
     pdl_trigger();
     if (MODE == R3_INV && !inverse) return;
-    const bool keep = kx < sp.hx && (full || (kx <= fp.kmax[0] && abs(oy) <= fp.kmax[1]));
-    const int kmax_pos = full ? N : fp.kmax[2];
+    const bool keep = kx < sp.hx && (full || (kx <= fp.kmax[0] && kept_o(o)));
+    const int kmax_pos = full ? N : is3 ? fp.kmax[2] : fp.kmax[1];
+    const float gpos = is3 ? sp.gz : sp.gy;
     C v[E];                                                      // from the forward transform on: positions lane + r R1
     if constexpr (MODE != R3_INV) {
         const C *__restrict__ in = a.in + ofs;
@@ -96,33 +108,47 @@ template <int N, int MODE> __global__ void __launch_bounds__(128, MODE == R3_STE
         for (int s = 0; s < S::BPT; ++s)
 #pragma unroll
             for (int r = 0; r < R1; ++r) v[s * R1 + r] = ok ? in[(lane + s * R1 + r * E) * W] : mk<float>(0, 0);
-        if (MODE == R3_STEP && fp.noisy) {
-            const int u = t & (W * R1 - 1), cp = u & 1, kx0 = tile * W + 2 * cp;
+        // the noise of the chunk, a pair of columns per thread (they share a Philox
+        // call); ALIAS: added to the state
+        auto noise = [&]() {
+            const int u = t % S::CHUNK, cp = u & 1, kx0 = tile * W + 2 * cp;
             const float qx0 = (float)kx0 * sp.gx, qx1 = (float)(kx0 + 1) * sp.gx, qo = (float)oy * sp.gy;
             const float qx0s = qx0 * qx0, qx1s = qx1 * qx1, qo2 = qo * qo;
             const PhiloxKey key = philox_key(fp.seed_lo, fp.seed_hi);
             const uint32_t step = (uint32_t)(*a.d_step), fid = (uint32_t)fp.field_id;
-            const bool on_plane = kx0 == 0 || 2 * kx0 == sp.nx, has1 = kx0 + 1 < sp.hx;
+            const bool on_plane = kx0 == 0 || 2 * kx0 == sp.nx, has1 = kx0 + 1 < sp.hx, noisy = !S::ALIAS || fp.noisy != 0;
             const int npow = fp.noise_pow;
             const float sigma0 = fp.sigma0;
-            C *xi = XI + ch * (N * W) + 2 * cp;
+            const C *st = a.state + ofs - c + 2 * cp;
+            C *xi = XI + ch * XS + 2 * cp;
+            C n0 = mk<float>(0, 0), n1 = n0;
+            if (S::ALIAS && ok) ld_pair<float>(st + (u >> 1) * W, n0, n1);
 #pragma unroll 1
             for (int pos = u >> 1; pos < N; pos += 2 * R1) {
-                const float qp = (float)signed_k(pos, N) * sp.gz, qyz2 = qp * qp + qo2;
-                C x0, x1 = mk<float>(0, 0);
-                noise_pair<float>(on_plane, kx0, o, pos, sigma0, npow, qx0s + qyz2, qx1s + qyz2, has1, sp, fid, key, step,
-                                  x0, x1);
+                C x0 = mk<float>(0, 0), x1 = x0;
+                const C f0 = n0, f1 = n1;
+                if (S::ALIAS && ok && pos + 2 * R1 < N) ld_pair<float>(st + (pos + 2 * R1) * W, n0, n1);   // the next one's
+                if (noisy) {
+                    const float qp = (float)signed_k(pos, N) * gpos, qyz2 = qp * qp + qo2;
+                    noise_pair<float>(on_plane, kx0, is3 ? o : pos, is3 ? pos : 0, sigma0, npow, qx0s + qyz2, qx1s + qyz2, has1,
+                                      sp, fid, key, step, x0, x1);
+                }
+                if (S::ALIAS) {
+                    x0 = mk<float>(fadd(f0.x, x0.x), fadd(f0.y, x0.y));
+                    x1 = mk<float>(fadd(f1.x, x1.x), fadd(f1.y, x1.y));
+                }
                 st_pair<float>(xi + pos * W, x0, x1);
             }
-        }
+        };
+        if (MODE == R3_STEP && !S::ALIAS && fp.noisy) noise();
 #pragma unroll
         for (int s = 0; s < S::BPT; ++s) {
             dft_reg<R1, -1, float>(v + s * R1);
 #pragma unroll
             for (int r = 0; r < R1; ++r) xb[((lane + s * R1) * (R1 + 1) + r) * W] = v[s * R1 + r];
         }
-        C ph[E];
-        if (MODE == R3_STEP) {
+        C ph[S::ALIAS ? 1 : E];
+        if (MODE == R3_STEP && !S::ALIAS) {
 #pragma unroll
             for (int r = 0; r < E; ++r) ph[r] = ok ? a.state[ofs + (lane + r * R1) * W] : mk<float>(0, 0);
         }
@@ -132,12 +158,17 @@ template <int N, int MODE> __global__ void __launch_bounds__(128, MODE == R3_STE
             v[r] = xb[(lane + r * (R1 + 1)) * W];
             if (r > 0) v[r] = cmul<float>(v[r], TW[(r - 1) * R1 + lane]);
         }
+        if (MODE == R3_STEP && S::ALIAS) {
+            __syncthreads();                                     // the exchange buffer is free
+            noise();
+            __syncthreads();
+        }
         dft_reg<E, -1, float>(v);
         if constexpr (MODE == R3_STEP) {
             const bool has_product = fp.power > 0, noisy = fp.noisy != 0;
             const float qx = (float)kx * sp.gx, qo = (float)oy * sp.gy;
             const float qxs = qx * qx, qo2 = qo * qo;
-            const C *xi = XI + ch * (N * W) + c;
+            const C *xi = XI + ch * XS + c;
             float dtO[kPolyTerms], dtM[kPolyTerms];
 #pragma unroll
             for (int i = 0; i < kPolyTerms; ++i) {
@@ -148,7 +179,7 @@ template <int N, int MODE> __global__ void __launch_bounds__(128, MODE == R3_STE
             auto update = [&](auto degree2) {
 #pragma unroll
                 for (int r = 0; r < E; ++r) {
-                    const float qp = (float)(lane + r * R1 - (2 * r >= E ? N : 0)) * sp.gz;
+                    const float qp = (float)(lane + r * R1 - (2 * r >= E ? N : 0)) * gpos;
                     const float q2 = qxs + (qp * qp + qo2);
                     float m, g;
                     if (decltype(degree2)::value) {
@@ -157,7 +188,10 @@ template <int N, int MODE> __global__ void __launch_bounds__(128, MODE == R3_STE
                     } else {
                         update_factors<float>(q2, dtO, dtM, m, g);
                     }
-                    v[r] = update_pre<float>(ph[r], v[r], noisy ? xi[(lane + r * R1) * W] : mk<float>(0, 0), m, g, has_product);
+                    // (ALIAS: phi + xi in place of xi; the same sum)
+                    const C f = S::ALIAS ? mk<float>(0, 0) : ph[S::ALIAS ? 0 : r];
+                    const C x = S::ALIAS || noisy ? xi[(lane + r * R1) * W] : mk<float>(0, 0);
+                    v[r] = update_pre<float>(f, v[r], x, m, g, has_product);
                     bad |= !finite_mode(v[r]);
                 }
             };
@@ -167,8 +201,8 @@ template <int N, int MODE> __global__ void __launch_bounds__(128, MODE == R3_STE
             if (bad && ok && kx < sp.hx && a.d_status) atomicOr(a.d_status, kStatusNonFinite);
         }
         // Hermitian part on the kx = 0 and Nx/2 planes (the field is real): phi(k) <-
-        // (phi(k) + conj phi(-k)) / 2, the partner at position -pos of the partner pencil
-        if (first_tile == 0 || (first_tile * W <= sp.nx / 2 && sp.nx / 2 < (first_tile + S::TILES) * W)) {
+        // (phi(k) + conj phi(-k)) / 2, the partner at position -pos (of the partner pencil)
+        if (first_tile == 0 || (first_tile * W <= sp.nx / 2 && sp.nx / 2 < (first_tile + ctiles) * W)) {
             const bool plane = ok && (kx == 0 || 2 * kx == sp.nx);
             __syncthreads();
             if (plane) {
@@ -177,7 +211,7 @@ template <int N, int MODE> __global__ void __launch_bounds__(128, MODE == R3_STE
             }
             __syncthreads();
             if (plane) {
-                const C *pb = XCH + (ch ^ 1) * S::BUF + c;
+                const C *pb = XCH + (is3 ? ch ^ 1 : ch) * S::BUF + c;
 #pragma unroll
                 for (int r = 0; r < E; ++r) {
                     const C p = pb[((N - lane - r * R1) & (N - 1)) * W];
@@ -302,7 +336,7 @@ template <int N> struct R3Row {
     }
 };
 
-template <int N, int MODE> __global__ void __launch_bounds__(128, 6) k3_row(const RowArgs<float> a) {
+template <int N, int MODE> __global__ void __launch_bounds__(128, R3Shape<N>::CTAS) k3_row(const RowArgs<float> a) {
     using S = R3Shape<N>;
     using L = R3Row<N>;
     using C = float2;
@@ -442,6 +476,7 @@ template <int N, int MODE> __global__ void __launch_bounds__(128, 6) k3_row(cons
             out[p] = mk<float>(lane == 0 ? v[H].x : 0.0f, 0.0f);
             out[p + W] = mk<float>(lane == 0 ? v[H].y : 0.0f, 0.0f);
         }
+        if (a.inc_step && blockIdx.x == 0 && blockIdx.y == 0 && t == 0) *a.d_step += 1;
     }
 }
 
@@ -457,14 +492,24 @@ template <int N> cudaError_t launch_row3_n(const RowArgs<float> &a, int nslots, 
     return cudaErrorInvalidValue;
 }
 
-template <int N> cudaError_t launch_col3_n(const ColArgs<float> &a, int nslots, cudaStream_t st) {
+// a.F: threads per CTA (128 in 3D)
+template <int N, int DIM> cudaError_t launch_col3_nd(const ColArgs<float> &a, int nslots, cudaStream_t st) {
     using S = R3Shape<N>;
-    const dim3 grid((a.n_tiles + S::TILES - 1) / S::TILES, a.sp.ny / 2 + 1, nslots);
-    const size_t base = sizeof(float2) * (size_t)(S::TWN + S::CHUNKS * S::BUF);
-    if (a.mode == COL_STEP) return launch_pdl(k3_col<N, R3_STEP>, grid, S::THREADS, base + sizeof(float2) * S::CHUNKS * N * W, st, a);
-    if (a.mode == COL_FWD) return launch_pdl(k3_col<N, R3_FWD>, grid, S::THREADS, base, st, a);
-    if (a.mode == COL_INV_MASK || a.mode == COL_INV_FULL) return launch_pdl(k3_col<N, R3_INV>, grid, S::THREADS, base, st, a);
+    constexpr int np = DIM == 3 ? 2 : 1;
+    if (a.F > 128 || a.F % 32 || a.F % (np * S::CHUNK) || (DIM == 3 && a.F != 128)) return cudaErrorInvalidConfiguration;
+    const int chunks = a.F / S::CHUNK, ctiles = chunks / np;
+    const dim3 grid((a.n_tiles + ctiles - 1) / ctiles, np == 2 ? a.sp.ny / 2 + 1 : 1, nslots);
+    const size_t base = sizeof(float2) * (size_t)(S::TWN + chunks * S::BUF);
+    const size_t xi = S::ALIAS ? 0 : sizeof(float2) * (size_t)chunks * N * W;
+    if (a.mode == COL_STEP) return launch_pdl(k3_col<N, R3_STEP, DIM>, grid, a.F, base + xi, st, a);
+    if (a.mode == COL_FWD) return launch_pdl(k3_col<N, R3_FWD, DIM>, grid, a.F, base, st, a);
+    if (a.mode == COL_INV_MASK || a.mode == COL_INV_FULL) return launch_pdl(k3_col<N, R3_INV, DIM>, grid, a.F, base, st, a);
     return cudaErrorInvalidValue;
+}
+template <int N> cudaError_t launch_col3_n(const ColArgs<float> &a, int nslots, cudaStream_t st) {
+    if constexpr (N <= 256)
+        if (a.sp.dim == 3) return launch_col3_nd<N, 3>(a, nslots, st);
+    return a.sp.dim == 2 ? launch_col3_nd<N, 2>(a, nslots, st) : cudaErrorInvalidValue;
 }
 
 template <int N> cudaError_t launch_mid3_n(const MidArgs<float> &a, int nslots, int ntiles, cudaStream_t st) {

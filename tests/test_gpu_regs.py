@@ -1,4 +1,4 @@
-"""The register z, y and x passes of FP32 3D systems (tuning key "regs3d") against
+"""The register passes of FP32 2D and 3D systems (tuning key "regs") against
 the staged kernels over the sides, orders, operators and batches the rule that
 selects them accepts (and sides where only some of the passes are taken),
 and against the oracle.
@@ -25,7 +25,7 @@ def _gpu():
     build.build()
 
 
-def _system(shape, regs3d, fields=1, batch=1, order=2, noisy=True, power=3):
+def _system(shape, regs, fields=1, batch=1, order=2, noisy=True, power=3):
     from paper_2405_02410_gb300 import pss as P
     s = P.System(shape, dt=0.01, seed=5, batch=batch, precision="f32", dx=(1.0, 0.7, 1.3))
     for i in range(fields):
@@ -38,7 +38,10 @@ def _system(shape, regs3d, fields=1, batch=1, order=2, noisy=True, power=3):
         if noisy:
             s.set_noise(f, pD, up)
         s.set_dealias(f, order)
-    s.set_tuning("regs3d", regs3d)
+    s.set_tuning("regs", regs)
+    if len(shape) == 2 and regs != 1:   # the per-step kernels at every size
+        s.set_tuning("resident", 0)
+        s.set_tuning("persist", 0)
     for b in range(batch):
         s.select_instance(b)
         for f in range(fields):
@@ -75,6 +78,52 @@ def test_against_the_staged_kernels(shape, kw):
     for x, y in zip(*got):
         assert np.isfinite(x).all()
         assert np.linalg.norm(x - y) <= 1e-5 * np.linalg.norm(y)
+
+
+@pytest.mark.parametrize("shape,kw", [
+    ((16, 16), {}), ((32, 64), dict(fields=2)), ((64, 32), dict(order=3)), ((128, 256), dict(order=0)),
+    ((256, 128), dict(batch=3, fields=2)), ((512, 16), dict(noisy=False)), ((16, 512), {}), ((512, 512), dict(fields=2)),
+    ((1024, 32), {}), ((32, 1024), dict(power=2)), ((1024, 1024), dict(order=0)), ((512, 1024), dict(power=0)),
+])
+def test_2d_against_the_staged_kernels(shape, kw):
+    fields = kw.get("fields", 1)
+    got = []
+    for regs in (2, 0):
+        s = _system(shape, regs, **kw)
+        s.step(1)
+        s.step(4)
+        got.append(_results(s, fields))
+        s.close()
+    for x, y in zip(*got):
+        assert np.isfinite(x).all()
+        assert np.linalg.norm(x - y) <= 1e-5 * np.linalg.norm(y)
+
+
+@pytest.mark.parametrize("shape,batch,fields", [((512, 512), 9, 1), ((256, 256), 33, 1), ((512, 1024), 3, 1), ((1024, 1024), 1, 2)])
+def test_2d_systems_that_fill_the_chip(shape, batch, fields):
+    # by the rule's own choice, each instance against the staged kernels
+    s = _system(shape, 1, batch=batch, fields=fields)
+    s.step(3)
+    got = _results(s, fields)
+    s.close()
+    r = _system(shape, 0, batch=batch, fields=fields)
+    r.step(3)
+    for x, y in zip(got, _results(r, fields)):
+        assert np.linalg.norm(x - y) <= 1e-5 * np.linalg.norm(y)
+    r.close()
+
+
+def test_2d_path_changes_between_runs():
+    # the per-step kernels keep the product in another layout than the register passes
+    s, r = _system((256, 256), 2), _system((256, 256), 0)
+    for regs in (0, 2, 0):
+        s.set_tuning("regs", regs)
+        s.step(2)
+        r.step(2)
+    for x, y in zip(_results(s, 1), _results(r, 1)):
+        assert np.linalg.norm(x - y) <= 1e-5 * np.linalg.norm(y)
+    s.close()
+    r.close()
 
 
 @pytest.mark.parametrize("shape", [(16, 32, 16), (64, 16, 8), (128, 4, 16), (8, 64, 32), (16, 16, 256)])
