@@ -756,6 +756,10 @@ bool regs_row(const pss_system *s, int mode) {
            (s->dim == 2 || s->tune_fast3d) &&
            (mode == ROW_R2C || mode == ROW_C2R || (mode == ROW_FUSED && (s->dim == 3 || regs2d_step(s))));
 }
+// product terms' row kernel on the same lines (k3_terms), in 2D
+bool regs_terms(const pss_system *s) {
+    return regs(s) && s->dim == 2 && s->nx >= 16 && s->nx <= 256 && s->ny > 1 && !s->tune_row_radix && !s->tune_row_pairs;
+}
 // Threads per CTA of k3_col and k3_row for `units` transforms (pairs of pencils
 // in 3D) of `per` threads: 128, fewer (whole warps) where that leaves SMs without
 // a CTA
@@ -1299,8 +1303,9 @@ template <typename T> struct Seq {
             a.nf = nf;
             a.inc_step = inc ? 1 : 0;
             a.prog = pl.prog;
-            a.G = terms_G(s);
-            cudaError_t e = launch_terms(a, s->batch, st);
+            const bool reg = regs_terms(s);
+            a.G = reg ? row3_G(s, s->batch) : terms_G(s);
+            cudaError_t e = reg ? launch_terms3(a, s->batch, st) : launch_terms(a, s->batch, st);
             s->launches++;
             if (e != cudaSuccess) return cuda_fail(s, e, "k_row_terms launch");
             return PSS_OK;

@@ -326,6 +326,7 @@ struct TermArgs {
     TermProg prog;
 };
 cudaError_t launch_terms(const TermArgs &a, int batch, cudaStream_t st);
+cudaError_t launch_terms3(const TermArgs &a, int batch, cudaStream_t st);   // k3_terms: 2D rows of 16..256 points
 
 // A run of steps of a 1D system (k_line: 64..1024 sites), one CTA per slot.
 // Per field: its explicit term M(q) F[(F^-1[op(q) m phi])^power] (power 0:

@@ -38,4 +38,14 @@ cudaError_t launch_row3(const RowArgs<float> &a, int nslots, cudaStream_t st) {
         default: return cudaErrorInvalidValue;
     }
 }
+cudaError_t launch_terms3(const TermArgs &a, int batch, cudaStream_t st) {
+    switch (a.sp.nx) {
+        case 16: return launch_terms3_n<16>(a, batch, st);
+        case 32: return launch_terms3_n<32>(a, batch, st);
+        case 64: return launch_terms3_n<64>(a, batch, st);
+        case 128: return launch_terms3_n<128>(a, batch, st);
+        case 256: return launch_terms3_n<256>(a, batch, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
 }  // namespace pss

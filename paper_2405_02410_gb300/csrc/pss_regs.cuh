@@ -336,45 +336,45 @@ template <int N> struct R3Row {
     }
 };
 
-template <int N, int MODE> __global__ void __launch_bounds__(128, R3Shape<N>::CTAS) k3_row(const RowArgs<float> a) {
+// A thread's place in the x pass: its transform lane, its pair's exchange
+// buffer, and the twiddles.
+template <int N> struct R3Line {
     using S = R3Shape<N>;
-    using L = R3Row<N>;
     using C = float2;
-    constexpr int E = S::E, R1 = S::R1, H = R1 / 2;
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    C *TW = reinterpret_cast<C *>(smem_raw);
-    const SysP<float> &sp = a.sp;
-    const int t = threadIdx.x, lane = t % R1, g = t / R1;
-    C *xb = TW + S::TWN + g * L::BUF;
-    const int slot = a.slot0 + blockIdx.y;
-    const int r0 = 2 * (blockIdx.x * a.G + g);                   // rows r0 and r0 + 1
-    const bool ok = r0 < sp.rows;
-    const int mirror = (t & 31 & ~(R1 - 1)) | ((R1 - lane) & (R1 - 1));
-    const size_t sofs = (size_t)slot * a.slot_stride;
+    static constexpr int E = S::E, R1 = S::R1, H = R1 / 2;
+    int lane, mirror;
+    uint32_t rows, r0;                                           // rows r0 and r0 + 1 of `rows`
+    bool ok;
+    C *xb;
+    const C *TW;
+
+    __device__ __forceinline__ R3Line(int t, int rows_, int r0_, C *xb_, const C *TW_)
+        : lane(t % R1), mirror((t & 31 & ~(R1 - 1)) | ((R1 - t % R1) & (R1 - 1))), rows((uint32_t)rows_),
+          r0((uint32_t)r0_), ok(r0_ < rows_), xb(xb_), TW(TW_) {}
     // mode lane + s R1 + r E of row r0 (row r0 + 1: W further on); a field has fewer than 2^32 values
-    auto ofs = [&](int s, int r) {
+    __device__ __forceinline__ uint32_t ofs(int s, int r) const {
         const int k = lane + s * R1 + r * E;
-        return ((uint32_t)(k >> 2) * (uint32_t)sp.rows + (uint32_t)r0) * W + (uint32_t)(k & (W - 1));
-    };
-    r3_twiddles<N>(TW, a.tw, t, blockDim.x);
-    const C *TWI = TW + (R1 == E ? 0 : N);
-    __syncthreads();
-    pdl_wait();
-    pdl_trigger();
-    C v[E];
-    if constexpr (MODE != R3_R2C) {
-        const C *__restrict__ in = a.in + sofs;
-        const int kxc = MODE == R3_FUSED ? a.fps[slot].kx_cols : sp.hx;
+        return ((uint32_t)(k >> 2) * rows + r0) * W + (uint32_t)(k & (W - 1));
+    }
+    // the two rows of a half spectrum (modes below kxc; dx: times i q_x, 0 at the
+    // Nyquist index) -> sites lane + r R1 of both
+    __device__ __forceinline__ void to_real(C *v, const C *__restrict__ in, int kxc, bool dx, float gx) const {
         C m[E / 2];                                              // Z_{N-k} for the thread that holds it
 #pragma unroll
         for (int s = 0; s < S::BPT; ++s)
 #pragma unroll
             for (int r = 0; r < H; ++r) {
                 C A = mk<float>(0, 0), B = A;
-                if (ok && lane + s * R1 + r * E < kxc) {
+                const int k = lane + s * R1 + r * E;
+                if (ok && k < kxc) {
                     const uint32_t p = ofs(s, r);
                     A = in[p];
                     B = in[p + W];
+                    if (dx) {
+                        const float q = (float)k * gx;
+                        A = mk<float>(-q * A.y, q * A.x);
+                        B = mk<float>(-q * B.y, q * B.x);
+                    }
                     if (s == 0 && r == 0 && lane == 0) A.y = B.y = 0.0f;
                 }
                 v[s * R1 + r] = mk<float>(A.x - B.y, A.y + B.x);
@@ -389,7 +389,7 @@ template <int N, int MODE> __global__ void __launch_bounds__(128, R3Shape<N>::CT
                 if (s == 0 && r == H) {
                     if (lane == 0) {
                         z = mk<float>(0, 0);
-                        if (ok && N / 2 < kxc) {
+                        if (ok && N / 2 < kxc && !dx) {
                             const uint32_t p = ofs(0, H);
                             z = mk<float>(in[p].x, in[p + W].x);
                         }
@@ -399,6 +399,7 @@ template <int N, int MODE> __global__ void __launch_bounds__(128, R3Shape<N>::CT
                 }
                 v[s * R1 + r] = z;
             }
+        __syncwarp();                                            // the buffer is free
 #pragma unroll
         for (int s = 0; s < S::BPT; ++s) {
             dft_reg<R1, +1, float>(v + s * R1);
@@ -414,8 +415,65 @@ template <int N, int MODE> __global__ void __launch_bounds__(128, R3Shape<N>::CT
                 v[r] = cmul<float>(v[r], mk<float>(w.x, -w.y));
             }
         }
-        dft_reg<E, +1, float>(v);                                // sites lane + r R1
+        dft_reg<E, +1, float>(v);
     }
+    // sites lane + r R1 of both rows -> their half spectra
+    __device__ __forceinline__ void to_modes(C *v, C *__restrict__ out) const {
+        const C *TWI = TW + (R1 == E ? 0 : N);
+        dft_reg<E, -1, float>(v);
+        __syncwarp();                                            // the buffer is free
+#pragma unroll
+        for (int r = 0; r < E; ++r) xb[lane * (E + 1) + r] = v[r];
+        __syncwarp();
+#pragma unroll
+        for (int s = 0; s < S::BPT; ++s) {
+            const int i = lane + s * R1;
+#pragma unroll
+            for (int r = 0; r < R1; ++r) {
+                v[s * R1 + r] = xb[i + r * (E + 1)];
+                if (r > 0) v[s * R1 + r] = cmul<float>(v[s * R1 + r], TWI[(r - 1) * E + i]);
+            }
+            dft_reg<R1, -1, float>(v + s * R1);
+        }
+#pragma unroll
+        for (int s = 0; s < S::BPT; ++s)
+#pragma unroll
+            for (int r = 0; r < H; ++r) {
+                const C x = v[s * R1 + r], y = v[E - 1 - (s * R1 + r)];
+                C z = mk<float>(__shfl_sync(0xffffffffu, y.x, mirror), __shfl_sync(0xffffffffu, y.y, mirror));
+                if (lane == 0) z = v[R3Row<N>::own(s, r)];
+                if (ok) {
+                    const uint32_t p = ofs(s, r);
+                    out[p] = mk<float>(0.5f * (x.x + z.x), 0.5f * (x.y - z.y));
+                    out[p + W] = mk<float>(0.5f * (x.y + z.y), -0.5f * (x.x - z.x));
+                }
+            }
+        if (ok && lane < W) {                                    // mode N / 2 and the last tile's padding
+            const uint32_t p = ofs(0, H);
+            out[p] = mk<float>(lane == 0 ? v[H].x : 0.0f, 0.0f);
+            out[p + W] = mk<float>(lane == 0 ? v[H].y : 0.0f, 0.0f);
+        }
+    }
+};
+
+template <int N, int MODE> __global__ void __launch_bounds__(128, R3Shape<N>::CTAS) k3_row(const RowArgs<float> a) {
+    using S = R3Shape<N>;
+    using C = float2;
+    constexpr int E = S::E, R1 = S::R1;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    C *TW = reinterpret_cast<C *>(smem_raw);
+    const SysP<float> &sp = a.sp;
+    const int t = threadIdx.x, g = t / R1, r0 = 2 * (blockIdx.x * a.G + g);
+    const R3Line<N> line(t, sp.rows, r0, TW + S::TWN + g * R3Row<N>::BUF, TW);
+    const int slot = a.slot0 + blockIdx.y;
+    const size_t sofs = (size_t)slot * a.slot_stride;
+    r3_twiddles<N>(TW, a.tw, t, blockDim.x);
+    __syncthreads();
+    pdl_wait();
+    pdl_trigger();
+    C v[E];
+    if constexpr (MODE != R3_R2C)
+        line.to_real(v, a.in + sofs, MODE == R3_FUSED ? a.fps[slot].kx_cols : sp.hx, false, 0.0f);
     if constexpr (MODE == R3_FUSED) {
         const int p = a.fps[slot].power;
         if (p == 3) {
@@ -425,9 +483,9 @@ template <int N, int MODE> __global__ void __launch_bounds__(128, R3Shape<N>::CT
 #pragma unroll
             for (int r = 0; r < E; ++r) v[r] = mk<float>(ipow<float>(v[r].x, p), ipow<float>(v[r].y, p));
         }
-    } else if (ok) {
-        const size_t ra = (size_t)slot * a.real_stride + real_row_offset(sp, r0) + lane;
-        const size_t rb = (size_t)slot * a.real_stride + real_row_offset(sp, r0 + 1) + lane;
+    } else if (line.ok) {
+        const size_t ra = (size_t)slot * a.real_stride + real_row_offset(sp, r0) + line.lane;
+        const size_t rb = (size_t)slot * a.real_stride + real_row_offset(sp, r0 + 1) + line.lane;
 #pragma unroll
         for (int r = 0; r < E; ++r) {
             if (MODE == R3_C2R) {
@@ -442,42 +500,85 @@ template <int N, int MODE> __global__ void __launch_bounds__(128, R3Shape<N>::CT
         for (int r = 0; r < E; ++r) v[r] = mk<float>(0, 0);
     }
     if constexpr (MODE != R3_C2R) {
-        dft_reg<E, -1, float>(v);
-        __syncwarp();                                            // the buffer is free again
-#pragma unroll
-        for (int r = 0; r < E; ++r) xb[lane * (E + 1) + r] = v[r];
-        __syncwarp();
-#pragma unroll
-        for (int s = 0; s < S::BPT; ++s) {
-            const int i = lane + s * R1;
-#pragma unroll
-            for (int r = 0; r < R1; ++r) {
-                v[s * R1 + r] = xb[i + r * (E + 1)];
-                if (r > 0) v[s * R1 + r] = cmul<float>(v[s * R1 + r], TWI[(r - 1) * E + i]);
-            }
-            dft_reg<R1, -1, float>(v + s * R1);
-        }
-        C *__restrict__ out = a.out + sofs;
-#pragma unroll
-        for (int s = 0; s < S::BPT; ++s)
-#pragma unroll
-            for (int r = 0; r < H; ++r) {
-                const C x = v[s * R1 + r], y = v[E - 1 - (s * R1 + r)];
-                C z = mk<float>(__shfl_sync(0xffffffffu, y.x, mirror), __shfl_sync(0xffffffffu, y.y, mirror));
-                if (lane == 0) z = v[L::own(s, r)];
-                if (ok) {
-                    const uint32_t p = ofs(s, r);
-                    out[p] = mk<float>(0.5f * (x.x + z.x), 0.5f * (x.y - z.y));
-                    out[p + W] = mk<float>(0.5f * (x.y + z.y), -0.5f * (x.x - z.x));
-                }
-            }
-        if (ok && lane < W) {                                    // mode N / 2 and the last tile's padding
-            const uint32_t p = ofs(0, H);
-            out[p] = mk<float>(lane == 0 ? v[H].x : 0.0f, 0.0f);
-            out[p + W] = mk<float>(lane == 0 ? v[H].y : 0.0f, 0.0f);
-        }
+        line.to_modes(v, a.out + sofs);
         if (a.inc_step && blockIdx.x == 0 && blockIdx.y == 0 && t == 0) *a.d_step += 1;
     }
+}
+
+// The x pass of product terms (k_row_terms) on the same lines, 2D rows of up to
+// 256 points: every distinct factor's rows to real space (kept in shared memory,
+// each thread its own sites), then per target field the sum of its terms and
+// back.  No CTA barrier after the twiddles.  us per step, k_row_terms -> here: a
+// coupled pair at 256^2 19.2 -> 14.6, at 64^2 16.5 -> 10.3, KPZ at 64^2 16.3 ->
+// 12.8, at 256 x 64 17.8 -> 15.6.  Above 256 points a thread would hold 32 sites
+// of a chain of transforms and too few warps are left to hide it.
+template <int N> __global__ void __launch_bounds__(128, 4) k3_terms(const TermArgs a) {
+    using S = R3Shape<N>;
+    using C = float2;
+    constexpr int E = S::E, R1 = S::R1;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    C *TW = reinterpret_cast<C *>(smem_raw);
+    const SysP<float> &sp = a.sp;
+    const TermProg &pg = a.prog;
+    const int t = threadIdx.x, g = t / R1;
+    C *R = TW + S::TWN + a.G * R3Row<N>::BUF + (size_t)g * pg.nfac * N + t % R1;   // [factor][site]
+    const R3Line<N> line(t, sp.rows, 2 * (blockIdx.x * a.G + g), TW + S::TWN + g * R3Row<N>::BUF, TW);
+    const int slot0 = blockIdx.y * a.nf;
+    r3_twiddles<N>(TW, a.tw, t, blockDim.x);
+    __syncthreads();
+    pdl_wait();
+    pdl_trigger();
+    C v[E];
+#pragma unroll 1
+    for (int f = 0; f < pg.nfac; ++f) {
+        const TermFactor fc = pg.fac[f];
+        const int slot = slot0 + fc.field;
+        line.to_real(v, (fc.arr < 0 ? a.in : a.extra + (size_t)fc.arr * a.extra_stride) + (size_t)slot * a.slot_stride,
+                     a.fps[slot].kx_cols, fc.dx != 0, sp.gx);
+#pragma unroll
+        for (int r = 0; r < E; ++r) R[f * N + r * R1] = v[r];
+    }
+#pragma unroll 1
+    for (int f = 0; f < a.nf; ++f) {
+        if (pg.nterm[f] == 0) continue;
+        const float *coef = a.coef + (size_t)(slot0 + f) * kMaxTerms;
+#pragma unroll
+        for (int r = 0; r < E; ++r) v[r] = mk<float>(0, 0);
+#pragma unroll 1
+        for (int i = 0; i < pg.nterm[f]; ++i) {
+            const TermP &tm = pg.term[f][i];
+            C p[E];
+#pragma unroll
+            for (int r = 0; r < E; ++r) p[r].x = p[r].y = coef[i];
+#pragma unroll 1
+            for (int k = 0; k < tm.n; ++k) {
+                const C *x = R + tm.fac[k] * N;
+#pragma unroll 1
+                for (int e = 0; e < tm.power[k]; ++e) {
+#pragma unroll
+                    for (int r = 0; r < E; ++r) {
+                        const C y = x[r * R1];
+                        p[r] = mk<float>(p[r].x * y.x, p[r].y * y.y);
+                    }
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < E; ++r) v[r] = cadd<float>(v[r], p[r]);
+        }
+        line.to_modes(v, a.out + (size_t)(slot0 + f) * a.slot_stride);
+    }
+    if (a.inc_step && blockIdx.x == 0 && blockIdx.y == 0 && t == 0) *a.d_step += 1;
+}
+
+template <int N> cudaError_t launch_terms3_n(const TermArgs &a, int batch, cudaStream_t st) {
+    using S = R3Shape<N>;
+    const int threads = a.G * S::R1;
+    if (threads % 32 || threads > 128 || a.sp.rows % 2 || a.prog.nfac < 1 || a.prog.nfac > kMaxTermFactors)
+        return cudaErrorInvalidConfiguration;
+    const size_t smem = sizeof(float2) * (size_t)(S::TWN + a.G * (R3Row<N>::BUF + a.prog.nfac * N));
+    cudaError_t e = ensure_smem(k3_terms<N>, smem);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(k3_terms<N>, dim3((a.sp.rows / 2 + a.G - 1) / a.G, batch), threads, smem, st, a);
 }
 
 template <int N> cudaError_t launch_row3_n(const RowArgs<float> &a, int nslots, cudaStream_t st) {

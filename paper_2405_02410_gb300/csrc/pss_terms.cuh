@@ -11,7 +11,8 @@
 // evaluates all terms there and transforms one sum per target field.  us per
 // step before -> after: a coupled pair at 256^2 92 -> 20 (19 launches -> 2), KPZ at
 // 512 x 256 38 -> 18, at 64^2 34 -> 17 (7 -> 3); bound by the chain of one
-// pair of rows through its transforms.
+// pair of rows through its transforms.  2D rows of 16..256 points run on k3_terms
+// (pss_regs.cuh); this kernel serves 1D systems and the other lengths.
 #pragma once
 
 #include "pss_kernels.cuh"
@@ -41,6 +42,8 @@ __global__ void __launch_bounds__(256) k_row_terms(const TermArgs a) {
     const bool active = g < G;
     for (int i = t; i < twiddle_elems<N>(); i += nthr) TW[i] = a.tw[twiddle_offset(N, EMAX) + i];
     __syncthreads();
+    pdl_wait();
+    pdl_trigger();
     const int ra = r0 + 2 * g, rb = ra + 1;                   // this group's rows (1D: the second one is empty)
     const bool has_a = active && ra < rows, has_b = active && rb < rows;
     C *b0 = B0 + (active ? g : 0) * SF, *b1 = B1 + (active ? g : 0) * SF;
@@ -125,8 +128,7 @@ template <int N> cudaError_t launch_terms_n(const TermArgs &a, int batch, cudaSt
     if (a.G < 1 || threads > 256 || a.prog.nfac < 1 || a.prog.nfac > kMaxTermFactors) return cudaErrorInvalidConfiguration;
     cudaError_t e = ensure_smem(k_row_terms<N>, smem);
     if (e != cudaSuccess) return e;
-    k_row_terms<N><<<dim3((a.sp.rows + 2 * a.G - 1) / (2 * a.G), batch), threads, smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(k_row_terms<N>, dim3((a.sp.rows + 2 * a.G - 1) / (2 * a.G), batch), threads, smem, st, a);
 }
 
 }  // namespace pss

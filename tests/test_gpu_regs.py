@@ -13,6 +13,7 @@ import pytest
 from oracle import oracle as O
 
 from tests.parity import check_spectrum
+from tests.test_gpu_terms_fused import _system as _terms_system, burgers, coupled, kpz, three_targets
 
 pytestmark = pytest.mark.gpu
 
@@ -149,3 +150,19 @@ def test_a_state_that_is_not_finite_is_reported():
     with pytest.raises(P.PssError):
         s.get_spectrum(0)
     s.close()
+
+
+@pytest.mark.parametrize("form", [coupled, burgers, kpz, three_targets])
+@pytest.mark.parametrize("shape,batch", [((8, 16), 1), ((16, 32), 2), ((4, 64), 1), ((64, 128), 1), ((32, 256), 3)])
+def test_product_terms_against_the_staged_row_kernel(shape, batch, form):
+    got = []
+    for regs in (1, 0):
+        s, nf, _ = _terms_system(shape, form, 1, batch)
+        s.set_tuning("regs", regs)
+        s.step(3)
+        got.append(_results(s, nf))
+        assert s.get_step() == 3
+        s.close()
+    for x, y in zip(*got):
+        assert np.isfinite(x).all()
+        assert np.linalg.norm(x - y) <= 1e-5 * np.linalg.norm(y)
