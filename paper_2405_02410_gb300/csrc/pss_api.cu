@@ -97,8 +97,6 @@ struct pss_system {
     void *GS = nullptr;                      // product terms: factor / product spectrum [slot][field_elems]
     void *term_extra = nullptr;              // fused product terms: further y-inverses [extra][slot][field_elems]
     size_t term_extra_bytes = 0;
-    float *term_coef = nullptr;              // their real-space coefficients [slot][kMaxTerms]
-    int coef_slots = 0;
     mutable std::shared_ptr<TermPlan> plan;  // made for generation plan_gen
     mutable uint64_t plan_gen = 0;
     void *real_acc = nullptr;                // product terms: sum of the products in real space (one slot)
@@ -399,14 +397,19 @@ template <typename T> FieldP<T> field_params(const pss_system *s, int inst, int 
 // refresh the device copy of the per-slot parameters (ordered on the system's stream)
 template <typename T> int upload_params_t(pss_system *s) {
     if (!s->fps_dirty) return PSS_OK;
-    std::vector<FieldP<T>> h;
-    h.reserve(s->nslots());
+    // one copy: the slots' parameters and, behind them, the coefficients of fused
+    // product terms (FP32)
+    const size_t np = s->nslots(), pb = sizeof(FieldP<T>) * np;
+    std::vector<unsigned char> h(pb + (std::is_same<T, float>::value && fused_terms(s) ? sizeof(float) * kMaxTerms * np : 0));
     for (int b = 0; b < s->batch; ++b)
-        for (int fi = 0; fi < (int)s->fields.size(); ++fi) h.push_back(field_params<T>(s, b, fi));
-    if (std::is_same<T, float>::value && fused_terms(s)) {
+        for (int fi = 0; fi < (int)s->fields.size(); ++fi) {
+            const FieldP<T> p = field_params<T>(s, b, fi);
+            std::memcpy(h.data() + sizeof p * ((size_t)b * s->fields.size() + fi), &p, sizeof p);
+        }
+    if (h.size() > pb) {
         // the coefficients of the terms' sums in real space, [slot][kMaxTerms]
         const TermPlan &pl = term_plan(s);
-        std::vector<float> c((size_t)s->nslots() * kMaxTerms, 1.0f);
+        std::vector<float> c(np * kMaxTerms, 1.0f);
         for (int b = 0; b < s->batch; ++b)
             for (int fi = 0; fi < (int)s->fields.size(); ++fi)
                 for (size_t i = 0; i < pl.coef[fi].size(); ++i)
@@ -415,19 +418,13 @@ template <typename T> int upload_params_t(pss_system *s) {
                         for (const Mono &m : pl.coef[fi][i]) v += m.scale * pval(s, b, m.param);
                         c[((size_t)b * s->fields.size() + fi) * kMaxTerms + i] = (float)v;
                     }
-        if (s->coef_slots != s->nslots()) {
-            cudaFree(s->term_coef);
-            s->term_coef = nullptr;
-            s->coef_slots = 0;
-            CK(cudaMalloc(&s->term_coef, sizeof(float) * c.size()));
-            s->coef_slots = s->nslots();
-        }
-        CK(cudaMemcpyAsync(s->term_coef, c.data(), sizeof(float) * c.size(), cudaMemcpyHostToDevice, s->stream));
+        std::memcpy(h.data() + pb, c.data(), sizeof(float) * c.size());
     }
-    if (!h.empty()) CK(cudaMemcpyAsync(s->fps, h.data(), sizeof(FieldP<T>) * h.size(), cudaMemcpyHostToDevice, s->stream));
+    if (!h.empty()) CK(cudaMemcpyAsync(s->fps, h.data(), h.size(), cudaMemcpyHostToDevice, s->stream));
     s->fps_dirty = false;
     return PSS_OK;
 }
+float *term_coef(const pss_system *s) { return (float *)((char *)s->fps + sizeof(FieldP<float>) * (size_t)s->nslots()); }
 
 int upload_params(pss_system *s) { return s->prec == PSS_F64 ? upload_params_t<double>(s) : upload_params_t<float>(s); }
 
@@ -1297,7 +1294,7 @@ template <typename T> struct Seq {
             a.extra_stride = all;
             a.out = (float2 *)B();
             a.slot_stride = s->field_elems;
-            a.coef = s->term_coef;
+            a.coef = term_coef(s);
             a.tw = (const float2 *)s->tw;
             a.d_step = s->d_step;
             a.nf = nf;
@@ -1481,9 +1478,9 @@ template <typename T> int full_prologue(pss_system *s, cudaStream_t st) {
 
 template <typename T> int run_prologue(pss_system *s) { return full_prologue<T>(s, s->stream); }
 
-int alloc_term_scratch(pss_system *s) {
+int alloc_term_scratch(pss_system *s, bool for_persist) {
     if (!any_general(s)) return PSS_OK;
-    if (fused_terms(s)) {
+    if (fused_terms(s) && !for_persist) {
         const size_t need = term_plan(s).extras.size() * csize(s) * s->field_elems * (size_t)s->nslots();
         if (s->term_extra_bytes < need) {
             cudaFree(s->term_extra);
@@ -1492,9 +1489,10 @@ int alloc_term_scratch(pss_system *s) {
             CK(cudaMalloc(&s->term_extra, need));
             s->term_extra_bytes = need;
         }
-        if (!persist2d(s)) return PSS_OK;    // (the persistent KPZ step keeps its second array in GS)
+        return PSS_OK;
     }
     if (!s->GS) CK(cudaMalloc(&s->GS, csize(s) * s->field_elems * (size_t)s->nslots()));
+    if (for_persist) return PSS_OK;          // (the persistent KPZ step keeps its second array in GS)
     if (!s->real) CK(cudaMalloc(&s->real, rsize(s) * (size_t)s->nsites));
     if (!s->real_acc) CK(cudaMalloc(&s->real_acc, rsize(s) * (size_t)s->nsites));
     if (!s->real_tp) CK(cudaMalloc(&s->real_tp, rsize(s) * (size_t)s->nsites));
@@ -1506,7 +1504,7 @@ int alloc_term_scratch(pss_system *s) {
 // that follows is a persistent launch, which computes both itself when they
 // are stale (its prologue flag): only the arrays are allocated here.
 int prologue(pss_system *s, bool for_persist = false) {
-    if (int rc = alloc_term_scratch(s)) return rc;
+    if (int rc = alloc_term_scratch(s, for_persist)) return rc;
     if (for_persist) {
         if (!s->XI) {
             const size_t bytes = csize(s) * s->field_elems * (size_t)s->nslots();
@@ -1957,7 +1955,7 @@ int grow_arrays(pss_system *s, int old_nf) {
     s->XI = nullptr;
     cudaFree(s->GS);
     s->GS = nullptr;
-    CK(cudaMalloc(&s->fps, fpsize(s) * (size_t)s->batch * nf));
+    CK(cudaMalloc(&s->fps, (fpsize(s) + sizeof(float) * kMaxTerms) * (size_t)s->batch * nf));   // (term_coef behind them)
     s->fps_dirty = true;
     return PSS_OK;
 }
@@ -2258,7 +2256,6 @@ int pss_destroy_system(pss_system *s) {
     cudaFree(s->real_acc);
     cudaFree(s->real_tp);
     cudaFree(s->term_extra);
-    cudaFree(s->term_coef);
     cudaFree(s->fps);
     cudaFree(s->tw);
     cudaFree(s->real);
