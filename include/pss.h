@@ -236,11 +236,12 @@ int pss_time_kernels(pss_system *s, int64_t n, double *avg_ms);
  *                 generic row kernel (0);
  *   "regs"        FP32 2D and 3D passes with their points in registers (1,
  *                 default) or the staged kernels (0): 3D systems without
- *                 product terms, sides of 16..256 points; 2D systems of 16..1024
- *                 points a side for fields in and out, and for the steps of
- *                 those with enough sites to fill the GPU (2: of all but
- *                 product terms and frames, where no run-in-one-launch path
- *                 takes them).  The launch-shape keys of the staged kernels
+ *                 product terms, sides of 16..256 points; 2D systems for fields
+ *                 in and out (16..256 points), for product terms (x sides of
+ *                 16..256 points) and for the steps of those of up to 1024
+ *                 points a side with enough sites to fill the GPU (2: of all
+ *                 but product terms and frames, where no run-in-one-launch
+ *                 path takes them).  The launch-shape keys of the staged kernels
  *                 select those where they are set.  The two agree to FP32
  *                 rounding;
  *   "col2_radix", "row2_radix"

@@ -235,7 +235,8 @@ template <typename T> SysP<T> sys_params(const pss_system *s) {
     p.dt = T(s->dt);
     p.inv_nsites = T(1.0 / (double)s->nsites);
     // programmatic dependent launch (tuning key "pdl"; by default only the
-    // FFT-group kernels k2_col / k2_row take it, see pdl_fast)
+    // FFT-group kernels k2_col / k2_row and the register passes take it, see
+    // pdl_fast and pdl_regs)
     p.pdl = s->tune_pdl >= 0 ? s->tune_pdl : 0;
     p.wait_limit = s->tune_test_timeout ? kTestWaitLimit : 0;
     p.tx_extra = s->tune_test_timeout ? 16u : 0u;
@@ -248,6 +249,16 @@ template <typename T> SysP<T> sys_params(const pss_system *s) {
 // before the wait), while the generic kernels lose (3D pair 360 -> 378 us,
 // the adjoint's column kernels), so by default it is on for the former only.
 int pdl_fast(const pss_system *s) { return s->tune_pdl >= 0 ? s->tune_pdl : 1; }
+
+// The same of the register passes (pss_regs.cuh), whose twiddles and parameters
+// are fetched before the wait: on for sides of up to 256 points (us per step, off
+// -> on: 32^3 10.0 -> 7.8, 64^3 pair 12.2 -> 10.5, 128^3 pair 38 -> 36, 256^3 pair
+// 245 -> 244, 256^2 x 64 28.4 -> 27.3; set_field 256^2 8.5 -> 5.0, 256^3 80 -> 72)
+// and off above, where a launch's last CTAs compete with its successor's first
+// (1024^2 pair 25.4 -> 30.4, 512 x 1024 x 3 24.3 -> 27.5).
+int pdl_regs(const pss_system *s) {
+    return s->tune_pdl >= 0 ? s->tune_pdl : std::max({s->nx, s->ny, s->nz}) <= 256 ? 1 : 0;
+}
 
 double pval(const pss_system *s, int inst, int id) {
     return id < 0 ? 1.0 : s->param_values[(size_t)inst * s->param_names.size() + id];
@@ -731,8 +742,9 @@ int res_ctas(pss_system *s) {
 // for.  3D: faster at every size measured (us per step, staged -> registers: 32^3
 // 20.4 -> 9.9, 64^3 pair 22.0 -> 12.1, 256 z x 64 x 32 22.2 -> 15.0, 16 z x 128
 // x 64 22.1 -> 11.2, 256^3 pair 351 -> 246).  2D: the step by regs2d_step, and
-// fields in and out at every size (set_field: 256^2 12.4 -> 8.5, 1024 x 64 14.5
-// -> 10.5, 512^2 12.5 -> 12.7, 1024^2 16.5 -> 14.6).  Product terms evaluated
+// fields in and out along axes of up to 256 points (set_field: 256^2 12.4 -> 8.5,
+// 64^3 22.8 -> 12.5, 256^3 120 -> 80; above, a KPZ run at 512^2 with its field's
+// way in and out lost 10 us).  Product terms evaluated
 // factor by factor keep the staged kernels (factors and summed spectra are
 // modes of theirs), and so do the adjoint's modes.
 bool regs(const pss_system *s) {
@@ -742,7 +754,7 @@ bool regs(const pss_system *s) {
 bool r3_side_of(const pss_system *s, int n) { return r3_side(n) && (s->dim == 2 || n <= 256); }
 bool regs_col(const pss_system *s, int mode) {
     return regs(s) && r3_side_of(s, s->n_inner) && !s->tune_col_radix && !s->tune_col_tiles &&
-           (mode == COL_FWD || mode == COL_INV_FULL ||
+           (((mode == COL_FWD || mode == COL_INV_FULL) && s->n_inner <= 256) ||
             ((mode == COL_STEP || mode == COL_INV_MASK) && (s->dim == 3 ? !any_general(s) : regs2d_step(s))));
 }
 bool regs_mid(const pss_system *s) {
@@ -751,7 +763,7 @@ bool regs_mid(const pss_system *s) {
 bool regs_row(const pss_system *s, int mode) {
     return regs(s) && r3_side_of(s, s->nx) && !s->tune_row_radix && !s->tune_row_pairs && !s->tune_row2_radix &&
            (s->dim == 2 || s->tune_fast3d) &&
-           (mode == ROW_R2C || mode == ROW_C2R || (mode == ROW_FUSED && (s->dim == 3 || regs2d_step(s))));
+           (((mode == ROW_R2C || mode == ROW_C2R) && s->nx <= 256) || (mode == ROW_FUSED && (s->dim == 3 || regs2d_step(s))));
 }
 // product terms' row kernel on the same lines (k3_terms), in 2D
 bool regs_terms(const pss_system *s) {
@@ -946,6 +958,7 @@ template <typename T> struct Seq {
         if constexpr (std::is_same<T, float>::value) {
             if (regs_col(s, mode) && !op_on) {
                 a.F = col3_threads(s, a.n_tiles, nslots);
+                a.sp.pdl = pdl_regs(s);
                 if (timer) timer->begin(0, st);
                 cudaError_t e = launch_col3(a, nslots, st);
                 if (timer) timer->begin(0, st);
@@ -954,6 +967,8 @@ template <typename T> struct Seq {
                 return PSS_OK;
             }
         }
+        // (beside k3_terms the launches are small: 256^2 pair 13.7 -> 13.0 us per step)
+        if (s->dim == 2 && any_general(s) && regs_terms(s)) a.sp.pdl = pdl_regs(s);
         if (timer) timer->begin(0, st);
         cudaError_t e = launch_col<T>(a, nslots, gx, gy, st);
         if (timer) timer->begin(0, st);
@@ -998,6 +1013,7 @@ template <typename T> struct Seq {
             // (real rows that are stored on the way, the adjoint's, are a mode of k_row)
             if (regs_row(s, mode) && !fac_acc && !(mode == ROW_FUSED && real_out)) {
                 a.G = row3_G(s, nslots);
+                a.sp.pdl = pdl_regs(s);
                 if (timer) timer->begin(2, st);
                 cudaError_t e = launch_row3(a, nslots, st);
                 if (timer) timer->begin(2, st);
@@ -1036,6 +1052,7 @@ template <typename T> struct Seq {
         if constexpr (std::is_same<T, float>::value) {
             if (regs_mid(s)) {
                 a.PZ = mid3_PZ(s);
+                a.sp.pdl = pdl_regs(s);
                 if (timer) timer->begin(kind, st);
                 cudaError_t e = launch_mid3(a, nslots, nt, st);
                 if (timer) timer->begin(kind, st);
@@ -1302,6 +1319,7 @@ template <typename T> struct Seq {
             a.prog = pl.prog;
             const bool reg = regs_terms(s);
             a.G = reg ? row3_G(s, s->batch) : terms_G(s);
+            if (reg) a.sp.pdl = pdl_regs(s);
             cudaError_t e = reg ? launch_terms3(a, s->batch, st) : launch_terms(a, s->batch, st);
             s->launches++;
             if (e != cudaSuccess) return cuda_fail(s, e, "k_row_terms launch");
