@@ -254,10 +254,12 @@ int pdl_fast(const pss_system *s) { return s->tune_pdl >= 0 ? s->tune_pdl : 1; }
 // are fetched before the wait: on for sides of up to 256 points (us per step, off
 // -> on: 32^3 10.0 -> 7.8, 64^3 pair 12.2 -> 10.5, 128^3 pair 38 -> 36, 256^3 pair
 // 245 -> 244, 256^2 x 64 28.4 -> 27.3; set_field 256^2 8.5 -> 5.0, 256^3 80 -> 72)
-// and off above, where a launch's last CTAs compete with its successor's first
-// (1024^2 pair 25.4 -> 30.4, 512 x 1024 x 3 24.3 -> 27.5).
+// and for few sites (1024 x 64 12.1 -> 8.8, 128 x 1024 x 4 18.5 -> 16.2); off for
+// more, where a launch's last CTAs compete with its successor's first (1024^2 pair
+// 25.4 -> 30.4, 512 x 1024 x 3 24.3 -> 27.5).
 int pdl_regs(const pss_system *s) {
-    return s->tune_pdl >= 0 ? s->tune_pdl : std::max({s->nx, s->ny, s->nz}) <= 256 ? 1 : 0;
+    if (s->tune_pdl >= 0) return s->tune_pdl;
+    return std::max({s->nx, s->ny, s->nz}) <= 256 || s->nsites * s->nslots() <= 1ll << 19 ? 1 : 0;
 }
 
 double pval(const pss_system *s, int inst, int id) {
@@ -573,10 +575,10 @@ bool fast2d_shape(const pss_system *s) {
 // -> 24.8, x 12 34.3 -> 28.2, x 32 85 -> 68; 512 x 256 x 16 23.2 -> 22.2, x 32
 // 40 -> 32; 256^2 x 32 17.8 -> 17.4, x 64 35 -> 28, x 128 70 -> 48; with a side
 // of 1024 from fewer sites on: 1024 x 512 x 2 20 -> 24, x 3 30 -> 24, 1024^2 x 2
-// 29.5 -> 25.5, x 8 107 -> 67; against the generic kernels (a side of 1024, the
-// other below 256) 1024 x 128 x 8 18.3 -> 18.2, x 16 29.4 -> 22.5, 128 x 1024 x
-// 32 54 -> 29.  One field of one instance (the adjoint's systems) stays below
-// these.
+// 29.5 -> 25.5, x 8 107 -> 67.  A side of 1024 with one below 256 always (against
+// the generic kernels; nx x ny: 1024 x 64 12.5 -> 8.8, 1024 x 128 12.7 -> 11.8, 64 x
+// 1024 15.6 -> 14.5, 128 x 1024 x 4 16.8 -> 16.2, x 16 29.4 -> 22.5, 1024 x 128 x 32
+// 54 -> 29).
 bool r3_side(int n) { return n >= 16 && n <= 1024; }
 bool regs2d_step(const pss_system *s) {
     if (!(s->tune_regs && s->prec == PSS_F32 && s->dim == 2 && r3_side(s->nx) && r3_side(s->ny) && !any_general(s) &&
@@ -585,15 +587,16 @@ bool regs2d_step(const pss_system *s) {
           !s->tune_row2_noise))
         return false;
     if (s->tune_regs > 1) return true;
+    if (!s->tune_fast2d) return false;       // the generic kernels are asked for
     const long long sites = s->nsites * s->nslots();
     if (fast2d_shape(s)) return std::max(s->nx, s->ny) == 1024 ? sites >= 3ll << 19 : sites > 1ll << 21;
-    return !(side_res(s->nx) && side_res(s->ny)) && sites >= 1ll << 20;
+    return !(side_res(s->nx) && side_res(s->ny));
 }
 bool fast2d(const pss_system *s) { return fast2d_shape(s) && !regs2d_step(s); }
-// Launch shape of the fast path, measured on GB300.  2D: radix-16 passes for
-// sides of 512 and 1024 (two warps per 1024-point transform, three passes),
+// Launch shape of the fast path, measured on GB300.  2D columns: radix-16 passes
+// for sides of 512 and 1024 (two warps per 1024-point transform, three passes),
 // radix 8 for 256 (one warp per transform: the 256^2 step is latency-bound,
-// 7.9 us against 9.7 us with radix 16), 4 row pairs per row CTA.  The 3D x
+// 7.9 us against 9.7 us with radix 16); rows: row2_radix, row2_pairs.  The 3D x
 // pass takes radix 16 at every side: at 256 points that is half a warp per
 // transform and two passes instead of three, and there the passes are bound
 // by shared-memory bandwidth (x pass of the 256^3 pair 130 -> 113 us).
@@ -803,9 +806,18 @@ int col2_radix(const pss_system *s) {
     const int r = s->tune_col2_radix ? s->tune_col2_radix : ((s->ny >= 512 || big_batch(s)) ? 16 : 8);
     return r == 32 && s->ny != 1024 ? 16 : r;   // radix-32 passes serve 1024 points only
 }
+// Row kernel: radix 8 chains its two transforms through registers and has twice
+// the threads per row pair (us per step, radix 16 -> 8: 512^2 pair 13.2 -> 11.1, 512
+// x 1024 14.1 -> 12.1, 1024 x 512 pair 15.6 -> 14.3, 512 x 256 9.8 -> 7.8).  Systems
+// of the persistent step keep its radix here, so that both give the same bits.
+// The adjoint's x pass stays with the radix it was measured with.
+int row2_adj_radix(const pss_system *s) {
+    const int r = s->tune_row2_radix ? s->tune_row2_radix : s->nx >= 512 ? 16 : 8;
+    return r == 32 && s->nx != 1024 ? 16 : r;
+}
 int row2_radix(const pss_system *s) {
     const int r = s->tune_row2_radix ? s->tune_row2_radix
-                                     : ((s->dim == 3 || (s->nx >= 512 && !big_batch(s))) ? 16 : 8);
+                                     : ((s->dim == 3 || (s->nx >= 512 && persist2d_ok(s))) ? 16 : 8);
     return r == 32 && s->nx != 1024 ? 16 : r;
 }
 // CTA size limits of the two kernels (their launch bounds leave radix-32
@@ -815,7 +827,7 @@ int row2_max_threads(int E) { return E == 32 ? 512 : 1024; }
 int col2_warps(const pss_system *s) {
     const int E = col2_radix(s);
     const int fft_warps = 4 * s->ny / E / 32;
-    const int want = s->tune_col2_warps > 0 ? s->tune_col2_warps : (big_batch(s) && s->ny == 256 ? 4 : 8);
+    const int want = s->tune_col2_warps > 0 ? s->tune_col2_warps : ((big_batch(s) && s->ny == 256) || (s->ny == 512 && !persist2d_ok(s)) ? 4 : 8);
     return std::max(1, std::min(want, col2_max_threads(E) / 32 - fft_warps));
 }
 int row2_noise_warps(const pss_system *s, int pairs) {
@@ -829,10 +841,14 @@ bool any_noisy(const pss_system *s) {
         if (f.noisy) return true;
     return false;
 }
-// row pairs per CTA: a power of two with at most 512 threads per CTA
+// row pairs per CTA: a power of two with at most 512 threads per CTA; fewer
+// where long rows are few enough for a CTA each (512 x 256 7.8 -> 6.8, 1024 x 256
+// 10.8 -> 7.9, 1024 x 512 12.9 -> 11.9 us per step; 512^2 loses with fewer, 9.3 -> 9.8)
 int row2_pairs(const pss_system *s) {
     const int tpf = s->nx / row2_radix(s);
-    const int nw = s->tune_row2_pairs > 0 ? s->tune_row2_pairs : (big_batch(s) ? 8 : 4);
+    int nw = s->tune_row2_pairs > 0 ? s->tune_row2_pairs : (big_batch(s) ? 8 : 4);
+    if (s->tune_row2_pairs <= 0 && !big_batch(s) && !persist2d_ok(s) && s->nx >= 512 && (s->ny <= 256 || s->nx == 1024))
+        while (nw > 1 && (long long)s->rows / 2 * s->nslots() / nw < 128) nw /= 2;
     int p = 1;
     while (p * tpf < 32) p *= 2;   // whole warps of transform threads
     while (p * 2 <= nw && p * 2 <= 8 && p * 2 * tpf <= 512) p *= 2;
@@ -844,8 +860,8 @@ int row2_pairs(const pss_system *s) {
 // every SM gets a CTA (at 256^2 the step's 4 pairs would leave 32 CTAs of
 // four warps on 152 SMs), with whole warps of transform threads.
 int row2_adj_pairs(const pss_system *s, int nslots) {
-    const int tpf = s->nx / row2_radix(s);
-    const int maxp = std::min(8, row2_max_threads(row2_radix(s)) / tpf);
+    const int tpf = s->nx / row2_adj_radix(s);
+    const int maxp = std::min(8, row2_max_threads(row2_adj_radix(s)) / tpf);
     int p = 1;
     while (p * tpf < 32) p *= 2;
     if (s->tune_adj_row_pairs > 0) {
@@ -1197,7 +1213,7 @@ template <typename T> struct Seq {
             a.d_step = s->d_step;
             a.d_status = s->d_status;
             a.mode = ROW_ADJ;
-            a.E = row2_radix(s);
+            a.E = row2_adj_radix(s);
             a.G = row2_adj_pairs(s, nslots);
             a.kx_cols_max = s->hx;
             if (timer) timer->begin(2, st);
