@@ -572,8 +572,8 @@ bool fast2d_shape(const pss_system *s) {
 // there are enough sites to fill the chip with them: 512 and 1024 points take
 // 32 of them per thread, so a launch lasts about 10 us however small.  us per
 // step, the FFT-group kernels (or cluster-resident run) -> here: 512^2 x 8 24.0
-// -> 24.8, x 12 34.3 -> 28.2, x 32 85 -> 68; 512 x 256 x 16 23.2 -> 22.2, x 32
-// 40 -> 32; 256^2 x 32 17.8 -> 17.4, x 64 35 -> 28, x 128 70 -> 48; with a side
+// -> 24.8, x 12 34.3 -> 28.2, x 32 85 -> 62; 512 x 256 x 16 23.2 -> 22.2, x 32
+// 40 -> 32; 256^2 x 32 17.8 -> 17.4, x 64 35 -> 26, x 128 70 -> 48; with a side
 // of 1024 from fewer sites on: 1024 x 512 x 2 20 -> 24, x 3 30 -> 24, 1024^2 x 2
 // 29.5 -> 25.5, x 8 107 -> 67.  A side of 1024 with one below 256 always (against
 // the generic kernels; nx x ny: 1024 x 64 12.5 -> 8.8, 1024 x 128 12.7 -> 11.8, 64 x
@@ -743,8 +743,8 @@ int res_ctas(pss_system *s) {
 // The register passes of FP32 2D and 3D systems (k3_col, k3_mid, k3_row) where
 // the side has their shape and no launch shape of the staged kernels is asked
 // for.  3D: faster at every size measured (us per step, staged -> registers: 32^3
-// 20.4 -> 9.9, 64^3 pair 22.0 -> 12.1, 256 z x 64 x 32 22.2 -> 15.0, 16 z x 128
-// x 64 22.1 -> 11.2, 256^3 pair 351 -> 246).  2D: the step by regs2d_step, and
+// 20.4 -> 7.8, 64^3 pair 22.0 -> 10.7, 256 x 256 x 64 54 -> 34, 16 z x 128 x 64 22.1
+// -> 8.9, 256^3 pair 351 -> 237).  2D: the step by regs2d_step, and
 // fields in and out along axes of up to 256 points (set_field: 256^2 12.4 -> 8.5,
 // 64^3 22.8 -> 12.5, 256^3 120 -> 80; above, a KPZ run at 512^2 with its field's
 // way in and out lost 10 us).  Product terms evaluated

@@ -12,14 +12,15 @@
 // one's first pass reads, so the update runs in registers between them.  The
 // noise is drawn into shared memory while the loads are in flight, a pair of
 // columns per Philox call.  us, staged -> here: 256^3, two fields: z pass 153
-// -> 111 (466 MB: 4.2 TB/s), y inverse 52 -> 37, y forward 63 -> 52 (270 MB:
-// 5.2 TB/s), x pass 104 -> 66 (225 MB: 3.4 TB/s), the step 351 -> 246; whole
-// steps of 128^3 35 -> 22, 256 x 256 x 64 54 -> 36, 64^3 (two fields) 22.0 ->
-// 12.1, 32^3 20.4 -> 9.9; 2D batches against the FFT-group kernels: 512^2 x 32
-// 85 -> 68, 1024^2 x 8 107 -> 67.  The step's column pass takes 5 CTAs per SM and
+// -> 104 (466 MB: 4.5 TB/s), y inverse 52 -> 37, y forward 63 -> 52 (270 MB:
+// 5.2 TB/s), x pass 104 -> 66 (225 MB: 3.4 TB/s), the step 351 -> 237; whole
+// steps of 128^3 (two fields) 58 -> 35, 256 x 256 x 64 54 -> 34, 64^3 (two fields)
+// 22.0 -> 10.7, 32^3 20.4 -> 7.8; 2D batches against the FFT-group kernels: 512^2 x 32
+// 85 -> 62, 1024^2 x 8 107 -> 67.  The step's column pass takes 5 CTAs per SM and
 // 96 registers, the state among them; 6 CTAs and 80 registers with the state
 // copied to shared memory asynchronously measured 118 .. 126 us at 256^3 in place
-// of 111.  512 and 1024 points put 32 points on a thread, so there the state
+// of 111; tests of planes, kept positions and the noise's power that hold for the
+// whole CTA, hoisted out of the per-mode code, took it from 111 to 104.  512 and 1024 points put 32 points on a thread, so there the state
 // goes through shared memory with the noise.
 
 #pragma once
@@ -83,7 +84,8 @@ __global__ void __launch_bounds__(128, MODE == R3_STEP && N < 512 ? 5 : R3Shape<
     const bool lone = is3 && op == opp;                          // its own partner: the second chunk is a copy
     const int first_tile = blockIdx.x * ctiles, tile = first_tile + (is3 ? ch >> 1 : ch);
     const int o = is3 && (ch & 1) ? opp : op, kx = tile * W + c;
-    const bool ok = tile < a.n_tiles, writes = ok && !((ch & 1) && lone);
+    // (one tile per CTA: the grid covers them exactly)
+    const bool ok = (is3 && 2 * S::CHUNK == 128) || tile < a.n_tiles, writes = ok && !((ch & 1) && lone);
     const size_t ofs = (size_t)slot * a.slot_stride + ((size_t)tile * sp.n_outer + o) * N * W + c;
     C *xb = XCH + ch * S::BUF + c;
     r3_twiddles<N>(TW, a.tw, t, nthr);
@@ -92,6 +94,8 @@ __global__ void __launch_bounds__(128, MODE == R3_STEP && N < 512 ? 5 : R3Shape<
     __syncthreads();
     const int oy = is3 ? signed_k(o, sp.ny) : 0;                 // ky of the pencil
     const bool full = a.mode == COL_INV_FULL;
+    // CTA-uniform: it holds kx = 0 or Nx/2 (and with Nx/2 the columns past the grid)
+    const bool planes = first_tile == 0 || (first_tile * W <= sp.nx / 2 && sp.nx / 2 < (first_tile + ctiles) * W);
     auto kept_o = [&](int k) { return !is3 || abs(signed_k(k, sp.ny)) <= fp.kmax[1]; };
     // CTA-uniform: nothing of the inverse is kept
     const bool inverse = MODE != R3_FWD && (full || (first_tile * W <= fp.kmax[0] && kept_o(op)));
@@ -100,6 +104,9 @@ __global__ void __launch_bounds__(128, MODE == R3_STEP && N < 512 ? 5 : R3Shape<
     if (MODE == R3_INV && !inverse) return;
     const bool keep = kx < sp.hx && (full || (kx <= fp.kmax[0] && kept_o(o)));
     const int kmax_pos = full ? N : is3 ? fp.kmax[2] : fp.kmax[1];
+    // whether position lane + r R1 is kept: |k| <= kmax_pos, as bounds on the lane
+    const int keep_hi = keep ? kmax_pos : -1, keep_lo = keep ? N - kmax_pos : 2 * N;
+    auto kept_pos = [&](int r) { return 2 * r < E ? lane <= keep_hi - r * R1 : lane >= keep_lo - r * R1; };
     const float gpos = is3 ? sp.gz : sp.gy;
     C v[E];                                                      // from the forward transform on: positions lane + r R1
     if constexpr (MODE != R3_INV) {
@@ -116,29 +123,37 @@ __global__ void __launch_bounds__(128, MODE == R3_STEP && N < 512 ? 5 : R3Shape<
             const float qx0s = qx0 * qx0, qx1s = qx1 * qx1, qo2 = qo * qo;
             const PhiloxKey key = philox_key(fp.seed_lo, fp.seed_hi);
             const uint32_t step = (uint32_t)(*a.d_step), fid = (uint32_t)fp.field_id;
-            const bool on_plane = kx0 == 0 || 2 * kx0 == sp.nx, has1 = kx0 + 1 < sp.hx, noisy = !S::ALIAS || fp.noisy != 0;
+            // (a test of the whole CTA: most hold neither plane)
+            const bool on_plane = planes && (kx0 == 0 || 2 * kx0 == sp.nx), has1 = kx0 + 1 < sp.hx, noisy = !S::ALIAS || fp.noisy != 0;
             const int npow = fp.noise_pow;
             const float sigma0 = fp.sigma0;
             const C *st = a.state + ofs - c + 2 * cp;
             C *xi = XI + ch * XS + 2 * cp;
             C n0 = mk<float>(0, 0), n1 = n0;
             if (S::ALIAS && ok) ld_pair<float>(st + (u >> 1) * W, n0, n1);
+            auto draw = [&](auto plane, auto odd) {
 #pragma unroll 1
-            for (int pos = u >> 1; pos < N; pos += 2 * R1) {
-                C x0 = mk<float>(0, 0), x1 = x0;
-                const C f0 = n0, f1 = n1;
-                if (S::ALIAS && ok && pos + 2 * R1 < N) ld_pair<float>(st + (pos + 2 * R1) * W, n0, n1);   // the next one's
-                if (noisy) {
-                    const float qp = (float)signed_k(pos, N) * gpos, qyz2 = qp * qp + qo2;
-                    noise_pair<float>(on_plane, kx0, is3 ? o : pos, is3 ? pos : 0, sigma0, npow, qx0s + qyz2, qx1s + qyz2, has1,
-                                      sp, fid, key, step, x0, x1);
+                for (int pos = u >> 1; pos < N; pos += 2 * R1) {
+                    C x0 = mk<float>(0, 0), x1 = x0;
+                    const C f0 = n0, f1 = n1;
+                    if (S::ALIAS && ok && pos + 2 * R1 < N) ld_pair<float>(st + (pos + 2 * R1) * W, n0, n1);   // the next one's
+                    if (noisy) {
+                        const float qp = (float)signed_k(pos, N) * gpos, qyz2 = qp * qp + qo2;
+                        noise_pair<float>(decltype(plane)::value && on_plane, kx0, is3 ? o : pos, is3 ? pos : 0, sigma0, decltype(odd)::value ? 1 : npow, qx0s + qyz2, qx1s + qyz2, has1,
+                                          sp, fid, key, step, x0, x1);
+                    }
+                    if (S::ALIAS) {
+                        x0 = mk<float>(fadd(f0.x, x0.x), fadd(f0.y, x0.y));
+                        x1 = mk<float>(fadd(f1.x, x1.x), fadd(f1.y, x1.y));
+                    }
+                    st_pair<float>(xi + pos * W, x0, x1);
                 }
-                if (S::ALIAS) {
-                    x0 = mk<float>(fadd(f0.x, x0.x), fadd(f0.y, x0.y));
-                    x1 = mk<float>(fadd(f1.x, x1.x), fadd(f1.y, x1.y));
-                }
-                st_pair<float>(xi + pos * W, x0, x1);
-            }
+            };
+            // one of the three forms for the whole CTA: no plane and conserved noise of
+            // power 1, no plane, any
+            if (planes) draw(std::true_type{}, std::false_type{});
+            else if (npow == 1) draw(std::false_type{}, std::true_type{});
+            else draw(std::false_type{}, std::false_type{});
         };
         if (MODE == R3_STEP && !S::ALIAS && fp.noisy) noise();
 #pragma unroll
@@ -202,7 +217,7 @@ __global__ void __launch_bounds__(128, MODE == R3_STEP && N < 512 ? 5 : R3Shape<
         }
         // Hermitian part on the kx = 0 and Nx/2 planes (the field is real): phi(k) <-
         // (phi(k) + conj phi(-k)) / 2, the partner at position -pos (of the partner pencil)
-        if (first_tile == 0 || (first_tile * W <= sp.nx / 2 && sp.nx / 2 < (first_tile + ctiles) * W)) {
+        if (planes) {
             const bool plane = ok && (kx == 0 || 2 * kx == sp.nx);
             __syncthreads();
             if (plane) {
@@ -222,22 +237,20 @@ __global__ void __launch_bounds__(128, MODE == R3_STEP && N < 512 ? 5 : R3Shape<
         C *out = (a.state_out ? a.state_out : a.state) + ofs;
         if (writes) {
 #pragma unroll
-            for (int r = 0; r < E; ++r) out[(lane + r * R1) * W] = kx < sp.hx ? v[r] : mk<float>(0, 0);
+            for (int r = 0; r < E; ++r) out[(lane + r * R1) * W] = !planes || kx < sp.hx ? v[r] : mk<float>(0, 0);
         }
         if (MODE == R3_FWD || !inverse) return;
         __syncthreads();                                         // the exchange buffer is free again
     } else {
 #pragma unroll
         for (int r = 0; r < E; ++r) {
-            const int k = lane + r * R1 - (2 * r >= E ? N : 0);
-            v[r] = ok && keep && abs(k) <= kmax_pos ? a.state[ofs + (lane + r * R1) * W] : mk<float>(0, 0);
+            v[r] = ok && kept_pos(r) ? a.state[ofs + (lane + r * R1) * W] : mk<float>(0, 0);
         }
     }
     // ---- the inverse of the de-aliased, 1 / N_sites-scaled field
 #pragma unroll
     for (int r = 0; r < E; ++r) {
-        const int k = lane + r * R1 - (2 * r >= E ? N : 0);
-        v[r] = keep && abs(k) <= kmax_pos ? cscale<float>(v[r], sp.inv_nsites) : mk<float>(0, 0);
+        v[r] = kept_pos(r) ? cscale<float>(v[r], sp.inv_nsites) : mk<float>(0, 0);
     }
     dft_reg<E, +1, float>(v);
 #pragma unroll
