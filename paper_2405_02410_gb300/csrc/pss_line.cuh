@@ -81,6 +81,7 @@ __global__ void __launch_bounds__(LineShape<T, N>::NT) k_line(const LineArgs<T> 
             update_factors<T>(q * q, dtO, dtM, MG[k].x, MG[k].y);
         }
     }
+    __syncthreads();   // the update reads factors of other threads, without a product before any other barrier
     const PhiloxKey key = philox_key(fp.seed_lo, fp.seed_hi);
 
     // Point k of the half-length inverse transform of a half spectrum X:

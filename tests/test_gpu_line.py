@@ -138,3 +138,29 @@ def test_nonfinite_is_reported():
     with pytest.raises(P.PssError) as ei:
         s.sync()
     assert ei.value.code == P.PSS_ENONFINITE
+
+
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+@pytest.mark.parametrize("n", [64, 512, 1024])
+def test_every_launch_of_a_linear_field_has_its_factors(n, prec):
+    # no product, no noise: a step multiplies mode k by 1 / (1 + dt O(q_k)), and the
+    # factors of a launch are read by other threads than the ones that made them; one
+    # step per launch, so that each launch's first update counts.  Bar per step, in half
+    # ulps: 16 of the denominator (q^2 carries 5, its square 10, coefficients 3, sums 3), 4
+    # of the reciprocal, 1 of the product, 11 of the reference's own
+    lhs = ((0.3, 0), (0.7, 1), (0.4, 2))
+    s = pss().System((n,), dt=0.01, seed=3, precision=prec, dx=(0.8,))
+    _field(s, "a", [], noise=None, lhs=lhs)
+    x = np.random.default_rng(n).uniform(-1.0, 1.0, n).astype(s.rdtype)
+    q2 = (2 * np.pi * np.arange(n // 2 + 1) / (n * 0.8)) ** 2
+    g = 1.0 / (1.0 + 0.01 * sum(c * q2 ** p for c, p in lhs))
+    tol = 64 * 32 * np.finfo(s.rdtype).eps / 2
+    for _ in range(8):
+        s.set_field(0, x)
+        h0 = s.get_spectrum(0).astype(np.complex128)
+        l0 = s.launch_count
+        for _ in range(64):
+            s.step(1)
+        assert s.launch_count - l0 == 64
+        h = s.get_spectrum(0)
+        assert np.all(np.abs(h - h0 * g ** 64) <= tol * np.abs(h0 * g ** 64) + 1e-30)
