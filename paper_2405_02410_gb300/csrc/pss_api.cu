@@ -2018,15 +2018,19 @@ const std::vector<double2> &host_tables() {
             for (int quarter = j / (kMaxFftN / 4); quarter > 0; --quarter) { const double x = c; c = -s; s = x; }
             h[kRootsOffset + j] = make_double2(c, -s);
         }
-        // (1/c, ln c) of the interval j of [1, 2), the upper half taken at half its
+        // (1/c, 2 ln c) of the interval j of [1, 2), the upper half taken at half its
         // value; c = 1 for the two intervals next to 1
         for (int j = 0; j < kLogEntries; ++j) {
             long double c = 1.0L + (j + 0.5L) / kLogEntries;
             if (j >= kLogEntries / 2) c /= 2;
             const double inv = (j == 0 || j == kLogEntries - 1) ? 1.0 : (double)(1.0L / c);
-            h[kLogOffset + j] = make_double2(inv, (double)-std::log((long double)inv));
+            h[kLogOffset + j] = make_double2(inv, (double)(-2 * std::log((long double)inv)));
         }
-        for (int k = 0; k < 32; ++k) h[kLn2Offset + k] = make_double2((double)(k * std::log(2.0L)), 0.0);
+        // 2 k ln 2 as a double and the remainder
+        for (int k = 0; k < 32; ++k) {
+            const long double v = 2 * k * std::log(2.0L);
+            h[kLn2Offset + k] = make_double2((double)v, (double)(v - (long double)(double)v));
+        }
         return h;
     }();
     return tables;

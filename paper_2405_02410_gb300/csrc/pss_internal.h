@@ -26,8 +26,8 @@ __host__ __device__ constexpr int twiddle_offset(int n, int emax) {
     return (emax == 2 ? 8 * kMaxFftN : emax == 4 ? 6 * kMaxFftN : emax == 32 ? 4 * kMaxFftN : emax == 16 ? 2 * kMaxFftN : 0) + n;
 }
 // behind the tables: the kMaxFftN-th roots of unity, exp(-2 pi i j / kMaxFftN),
-// and (FP64) the logarithm tables of noise_mode: kLogEntries pairs (1/c, ln c)
-// and the multiples k ln 2, k < 32 (in x)
+// and (FP64) the logarithm tables of noise_mode: kLogEntries pairs (1/c, 2 ln c)
+// and 2 k ln 2, k < 32, as (double, remainder)
 constexpr int kRootsOffset = 10 * kMaxFftN;
 constexpr int kLogOffset = 11 * kMaxFftN;
 constexpr int kLogEntries = 128;

@@ -82,3 +82,33 @@ def test_nonfinite_is_reported():
         with pytest.raises(P.PssError) as ei:
             s.sync()
         assert ei.value.code == P.PSS_ENONFINITE
+
+
+@pytest.mark.parametrize("D,dt", [(1.0, 1.0), (0.05, 0.01)])
+def test_normals_have_no_common_error(D, dt):
+    # the relative error that all draws of a run share adds up over its steps, unlike
+    # their independent roundings.  Projection of the increments' error on the increments,
+    # in units of 2^-53: the 16 000 components' roundings (about 1 each) leave 0.01, the
+    # 128 intervals' table entries (0.3 each, halved by the root) 0.02; bar 0.15
+    ld = np.longdouble
+    ny = nx = 128
+    seed = 20240502
+    s = pss().System((ny, nx), dt=dt, seed=seed, precision="f64")
+    f = s.add_field("phi")
+    s.set_noise(f, s.add_param("D", D), 0)
+    s.step(1)
+    got = s.get_spectrum(f)[:, 1:nx // 2]
+    kx, ky = np.meshgrid(np.arange(1, nx // 2), np.arange(ny))
+    hxe = nx // 2 + 2
+    ctr = np.zeros((kx.size, 4), dtype=np.uint32)
+    ctr[:, 0] = ((ky * hxe + kx) >> 1).reshape(-1)
+    w = O.philox(ctr, np.tile(np.array([seed & 0xFFFFFFFF, seed >> 32], dtype=np.uint32), (kx.size, 1)))
+    odd = (kx.reshape(-1) & 1) == 1
+    u0, u1 = ((np.where(odd, w[:, 2 + i], w[:, i]) >> 8).astype(ld) + ld(0.5) for i in (0, 1))
+    u0, u1 = u0 / 2 ** 24, u1 / 2 ** 24
+    pi = 4 * np.arctan(ld(1))
+    r = np.sqrt(-2 * np.log(u0)) * ld(np.sqrt(ny * nx * D * dt))
+    re, im = r * np.cos(2 * pi * u1), r * np.sin(2 * pi * u1)
+    er, ei = got.real.reshape(-1).astype(ld) - re, got.imag.reshape(-1).astype(ld) - im
+    common = float((er * re + ei * im).sum() / (re * re + im * im).sum() * ld(2) ** 53)
+    assert abs(common) <= 0.15, common
