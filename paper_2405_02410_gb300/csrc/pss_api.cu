@@ -468,13 +468,19 @@ int col_emax(const pss_system *s) {
     if (s->tune_col_radix) return s->tune_col_radix;
     return (s->dim == 3 || s->n_inner >= 1024) ? 16 : 8;
 }
-int row_emax(const pss_system *s) {
+// `whole`: a whole field on its way in or out.  A radix-2 or 4 transform has more
+// twiddle multiplications, and their roundings, than one of radix 8 (relative error of
+// a 128^2 transform in FP64 3.3e-16 -> 4.2e-16).  A step's product enters the state
+// times dt, where nothing of that is left (errors of runs the same to three digits);
+// a whole field takes it at full size, so it keeps radix 8 (us, radix 2 and 4 against
+// 8: set_field 128^2 15 -> 25, 64 x 32 x 128 37 -> 47, 1024^2 101 -> 98).
+int row_emax(const pss_system *s, bool whole = false) {
     return s->tune_row_radix ? s->tune_row_radix
-         : s->prec == PSS_F64 ? f64_radix(s, s->nx, (long long)(s->rows + 1) / 2 * s->nslots()) : 8;
+         : s->prec == PSS_F64 && !whole ? f64_radix(s, s->nx, (long long)(s->rows + 1) / 2 * s->nslots()) : 8;
 }
 // (a y CTA holds at least kTileW transforms and at most 256 threads)
-int mid_emax(const pss_system *s) {
-    return s->tune_mid_radix ? s->tune_mid_radix : s->prec != PSS_F64 ? 16
+int mid_emax(const pss_system *s, bool whole = false) {
+    return s->tune_mid_radix ? s->tune_mid_radix : s->prec != PSS_F64 || whole ? 16
          : s->ny < 16 ? 8 : s->ny <= 256 ? 4 : s->ny <= 512 ? 8 : 16;
 }
 // FP64 column kernel on single columns (not the adjoint's modes): at least 16
@@ -513,8 +519,8 @@ int col_tiles_per_cta(const pss_system *s) {
 
 // row pairs per CTA of the row kernel: a power of two with G * TPF <= 128
 // threads, and at least ~8 CTAs when there are few rows
-int row_G(const pss_system *s) {
-    const int tpf = fft_TPF(s->nx, row_emax(s));
+int row_G(const pss_system *s, bool whole = false) {
+    const int tpf = fft_TPF(s->nx, row_emax(s, whole));
     if (s->tune_row_pairs > 0) {
         int G = 1;
         while (G * 2 <= s->tune_row_pairs && G * 2 * tpf <= 256 && G * 2 <= std::max(1, s->rows / 2)) G *= 2;
@@ -543,8 +549,8 @@ int terms_G(const pss_system *s) {
     return G;
 }
 
-int mid_PZ(const pss_system *s) {
-    const int tpf = fft_TPF(s->ny, mid_emax(s));
+int mid_PZ(const pss_system *s, bool whole = false) {
+    const int tpf = fft_TPF(s->ny, mid_emax(s, whole));
     int pz = std::max(1, 256 / (kTileW * tpf));
     if (s->tune_mid_planes > 0) {
         int p = 1;
@@ -910,6 +916,7 @@ template <typename T> struct Seq {
     cudaStream_t st;
     int slot0, nslots;
     Timer *timer = nullptr;
+    bool whole = false;                      // whole fields in or out (row_emax)
     // a product-term factor in flight: the column inverse applies op(q), the
     // row inverse folds r^n into the term's product instead of storing r
     int op_on = 0, op_deriv = -1, op_lap = 0;
@@ -949,7 +956,12 @@ template <typename T> struct Seq {
         a.d_step = s->d_step;
         a.d_status = s->d_status;
         a.mode = mode;
-        const bool single = col_single(s, mode);
+        // (whole fields: radix-8 tiles, where they fit shared memory)
+        bool single = col_single(s, mode);
+        if (single && whole) {
+            const size_t need = col_smem_bytes<T>(s->n_inner, col_tiles_per_cta(s) * kTileW * (s->dim == 3 ? 2 : 1), col_emax(s), mode);
+            single = need == 0 || need > 227 * 1024;
+        }
         a.E = single ? col_single_radix(s) : col_emax(s);
         a.wc = single ? 1 : kTileW;
         a.tiles_per_cta = single ? col_singles_per_cta(s) : col_tiles_per_cta(s);
@@ -1014,8 +1026,8 @@ template <typename T> struct Seq {
         a.d_step = s->d_step;
         a.d_status = s->d_status;
         a.mode = mode;
-        a.E = row_emax(s);
-        a.G = row_G(s);
+        a.E = row_emax(s, whole);
+        a.G = row_G(s, whole);
         a.kx_cols_max = 0;
         for (int i = 0; i < (int)s->fields.size(); ++i) a.kx_cols_max = std::max(a.kx_cols_max, kept_cols(s, i));
         a.inc_step = inc ? 1 : 0;
@@ -1060,8 +1072,8 @@ template <typename T> struct Seq {
         a.d_step = s->d_step;
         a.d_status = s->d_status;
         a.mode = mode;
-        a.E = mid_emax(s);
-        a.PZ = mid_PZ(s);
+        a.E = mid_emax(s, whole);
+        a.PZ = mid_PZ(s, whole);
         a.inc_step = inc ? 1 : 0;
         const int nt = mode == MID_INV_MASK ? max_kept_tiles(s) : s->ntiles;
         const int kind = mode == MID_FWD ? 3 : 1;
@@ -1388,6 +1400,7 @@ template <typename T> struct Seq {
     // real field (by default the scratch) -> state of the sequence's slots
     int forward_from_real(const void *real = nullptr) {
         int rc;
+        whole = true;
         const T *r = (const T *)(real ? real : s->real);
         if (s->dim == 3) {
             if ((rc = row_ptrs(ROW_R2C, A(), A(), false, r, nullptr, 0))) return rc;   // real -> A
@@ -1401,6 +1414,7 @@ template <typename T> struct Seq {
     // state -> real field (by default the scratch)
     int inverse_to_real(void *real = nullptr) {
         int rc;
+        whole = true;
         void *r = real ? real : s->real;
         if ((rc = col(COL_INV_FULL, false, true))) return rc;                     // state -> A
         if (s->dim == 3) {

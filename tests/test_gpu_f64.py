@@ -112,3 +112,24 @@ def test_normals_have_no_common_error(D, dt):
     er, ei = got.real.reshape(-1).astype(ld) - re, got.imag.reshape(-1).astype(ld) - im
     common = float((er * re + ei * im).sum() / (re * re + im * im).sum() * ld(2) ** 53)
     assert abs(common) <= 0.15, common
+
+
+@pytest.mark.parametrize("shape", [(64,), (128, 128), (16, 512), (32, 16, 64)])
+def test_whole_fields_take_radix_8_transforms(shape):
+    # a field's way in and out is the radix-8 (y and z in 3D: 16) transform's, bit for bit,
+    # whatever radix the steps' products take; the transforms of fewer roundings
+    P = pss()
+    x = np.random.default_rng(5).uniform(-1.0, 1.0, shape)
+    out = []
+    for radix in ({}, dict(row_radix=8, col_radix=16 if len(shape) == 3 else 8, mid_radix=16)):
+        s = P.System(shape, dt=0.01, precision="f64")
+        s.add_field("phi")
+        for k, v in radix.items():
+            s.set_tuning(k, v)
+        s.set_field(0, x)
+        h = s.get_spectrum(0)
+        if out:
+            s.set_spectrum(0, out[0][0])
+        out.append((h, s.get_field(0)))
+    np.testing.assert_array_equal(out[0][0], out[1][0])
+    np.testing.assert_array_equal(out[0][1], out[1][1])
