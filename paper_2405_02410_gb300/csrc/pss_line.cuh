@@ -208,15 +208,17 @@ __global__ void __launch_bounds__(LineShape<T, N>::NT) k_line(const LineArgs<T> 
         }
         __syncthreads();
         if (fl.frame_w > 0) {
-            // the real field with its frame, and its spectrum
+            // the change that sets the frame on the real field, zero inside it, added to
+            // the spectrum: the transforms' roundings reach the state by the size of that
+            // change, not of the field
             auto full = [&](int k) {
                 C v = cscale<T>(PHI[k], sp.inv_nsites);
                 if (k == 0 || k == M) v.y = T(0);
                 return v;
             };
             const C *Z = there_and_back([&](int k) { return tangle(full(k), full(M - k), k); },
-                                        [&](int x, T v) { return x < fl.frame_w ? fl.frame_lo : x >= N - fl.frame_w ? fl.frame_hi : v; });
-            for (int k = t; k <= M; k += S::NT) PHI[k] = untangle(Z, k);
+                                        [&](int x, T v) { return x < fl.frame_w ? fl.frame_lo - v : x >= N - fl.frame_w ? fl.frame_hi - v : T(0); });
+            for (int k = t; k <= M; k += S::NT) PHI[k] = cadd<T>(PHI[k], untangle(Z, k));
             __syncthreads();
         }
         if (has_product && n + 1 < a.nsteps) P = product();
