@@ -1820,21 +1820,22 @@ int launch_resident(pss_system *s, int nsteps, cudaStream_t st) {
     return PSS_OK;
 }
 
+// (a launch that is refused leaves the host's counter at the steps issued before it)
 int run_resident(pss_system *s, int64_t n, cudaStream_t st) {
     for (int64_t done = 0; done < n;) {
         const int len = (int)std::min<int64_t>(kMaxPersistSteps, n - done);
-        if (int rc = launch_resident(s, len, st)) return rc;
+        if (int rc = launch_resident(s, len, st)) { s->step += done; return rc; }
+        s->stale = true;
         done += len;
     }
-    s->stale = true;
     return PSS_OK;
 }
 
 // pss_step_many: the resident systems' runs, side by side on their capture
 // streams after everything issued on the list's stream (the most costly
 // first; a single one with no graph beside it stays on that stream); the
-// others' graph follows on the list's stream, and join_resident makes that
-// stream wait for them.
+// others' graph follows on the list's stream, and join_resident, after a
+// failure too, makes that stream wait for them.
 int run_resident_beside(pss_system *s0, std::vector<pss_system *> &res, bool beside, int64_t steps) {
     if (res.empty()) return PSS_OK;
     std::stable_sort(res.begin(), res.end(), [](const pss_system *a, const pss_system *b) {
@@ -1849,8 +1850,10 @@ int run_resident_beside(pss_system *s0, std::vector<pss_system *> &res, bool bes
         cudaEventDestroy(ev);
         if (e != cudaSuccess) return cuda_fail(s0, e, "forking the resident runs");
     }
-    for (pss_system *s : res)
-        if (int rc = run_resident(s, steps, ev ? s->cap_stream : s0->stream)) return fail(s0, rc, "%s", s->err.c_str());
+    for (pss_system *s : res) {
+        if (int rc = run_resident(s, steps, ev ? s->cap_stream : s0->stream)) return s == s0 ? rc : fail(s0, rc, "%s", s->err.c_str());
+        s->step += steps;
+    }
     return PSS_OK;
 }
 
@@ -2619,9 +2622,6 @@ int pss_step_many(pss_system **systems, int n, int64_t steps) {
     for (int i = 0; i < n; ++i)
         for (int j = 0; j < i; ++j) twice |= systems[i] == systems[j];
     for (int i = 0; i < n; ++i) (!twice && resident(systems[i]) ? res : rest).push_back(systems[i]);
-    if (int rc = run_resident_beside(s0, res, !rest.empty(), steps)) return rc;
-    pss_system **all = systems;
-    const int n_all = n;
     systems = rest.data();
     n = (int)rest.size();
     const int chunk = s0->tune_graph_steps > 0 ? s0->tune_graph_steps : kDefaultGraphSteps;
@@ -2657,22 +2657,32 @@ int pss_step_many(pss_system **systems, int n, int64_t steps) {
         *out = ge;
         return PSS_OK;
     };
+    // every graph first: a capture that fails leaves all systems as they were.  After
+    // that a failure keeps what was issued: joined, and counted in each system's steps
+    for (const int64_t len : {std::min<int64_t>(chunk, steps), steps % chunk}) {
+        cudaGraphExec_t ge = nullptr;
+        if (n > 0 && len > 0)
+            if (int rc = graph_of((int)len, &ge)) return rc;
+    }
+    int rc = run_resident_beside(s0, res, n > 0, steps);
     int64_t done = 0;
-    while (n > 0 && done < steps) {
+    while (rc == PSS_OK && n > 0 && done < steps) {
         const int len = (int)std::min<int64_t>(chunk, steps - done);
         cudaGraphExec_t ge = nullptr;
-        if (int rc = graph_of(len, &ge)) return rc;
+        if ((rc = graph_of(len, &ge))) break;
         cudaError_t e = cudaGraphLaunch(ge, s0->stream);
-        if (e != cudaSuccess) return cuda_fail(s0, e, "cudaGraphLaunch");
+        if (e != cudaSuccess) { rc = cuda_fail(s0, e, "cudaGraphLaunch"); break; }
         for (int i = 0; i < n; ++i) systems[i]->launches += (int64_t)len * systems[i]->graph_launches;
         done += len;
     }
-    if (int rc = join_resident(s0, res)) return rc;
-    for (int i = 0; i < n_all; ++i) {
-        all[i]->step += steps;
-        if (resident(all[i])) all[i]->stale = true;
+    for (int i = 0; i < n; ++i) {
+        systems[i]->step += done;
+        if (done > 0 && resident(systems[i])) systems[i]->stale = true;
     }
-    return PSS_OK;
+    const std::string first = s0->err;
+    const int jrc = join_resident(s0, res);
+    if (rc) s0->err = first;
+    return rc ? rc : jrc;
 }
 
 int pss_adjoint_forward(pss_system *s, int64_t n) {

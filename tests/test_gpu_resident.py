@@ -152,3 +152,32 @@ def test_nonfinite_state_is_reported():
     with pytest.raises(P.PssError) as ei:
         s.sync()
     assert ei.value.code == P.PSS_ENONFINITE
+
+
+@pytest.mark.parametrize("first", [0, 1])
+def test_step_many_leaves_every_system_as_it_was_when_a_capture_fails(first):
+    # a system of the list whose launch the host refuses (its radix-8 columns of 1024 points
+    # take too many threads), found while its graph is captured: nothing of the list runs
+    P = pss()
+    res = P.model_b((64, 64), dt=0.01, a=-1, b=1, K=1, D=0.05, seed=4, precision="f32")
+    bad = P.model_b((1024, 4, 4), dt=0.001, a=-1, b=1, K=1, D=0.05, seed=4, precision="f64")
+    systems = [res, bad] if first == 0 else [bad, res]
+    for s in systems:
+        s.init_uniform(0, -0.1, 0.1)
+    P.step_many(systems, 2)
+    before = [s.get_spectrum(0) for s in systems]
+    bad.set_tuning("col_radix", 8)
+    for _ in range(2):
+        with pytest.raises(P.PssError):
+            P.step_many(systems, 20)
+        for s, x in zip(systems, before):
+            assert s.get_step() == 2
+            np.testing.assert_array_equal(s.get_spectrum(0), x)
+    bad.set_tuning("col_radix", 0)
+    P.step_many(systems, 20)
+    for s in systems:
+        assert s.get_step() == 22
+    twin = P.model_b((64, 64), dt=0.01, a=-1, b=1, K=1, D=0.05, seed=4, precision="f32")
+    twin.init_uniform(0, -0.1, 0.1)
+    twin.step(22)
+    np.testing.assert_array_equal(res.get_spectrum(0), twin.get_spectrum(0))
