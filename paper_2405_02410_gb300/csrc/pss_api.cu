@@ -195,6 +195,7 @@ int fail(pss_system *s, int code, const char *fmt, ...) {
 }
 
 int cuda_fail(pss_system *s, cudaError_t e, const char *what) {
+    cudaGetLastError();   // reported here: not again by the next launch's check
     return fail(s, e == cudaErrorMemoryAllocation ? PSS_ENOMEM : PSS_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
@@ -2693,9 +2694,9 @@ int pss_adjoint_forward(pss_system *s, int64_t n) {
     if (any_general(s)) return fail(s, PSS_EUNSUPPORTED, "the adjoint covers power products only");
     int64_t K = (int64_t)std::ceil(std::sqrt((double)n));
     const int64_t nck = (n + K - 1) / K;
+    s->adj_ready = false;                    // (arrays of an earlier run may go before an allocation fails)
     int rc = adj_alloc(s, nck, K);
     if (rc) return rc;
-    s->adj_ready = false;
     s->adj_n = n;
     s->adj_step0 = s->step;
     s->adj_K = K;

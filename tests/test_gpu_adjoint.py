@@ -427,3 +427,29 @@ def test_adjoint_workload_at_its_own_size():
         fd = (4.0 * central(name, h / 2) - central(name, h)) / 3.0
         assert abs(grads["f64"][i] - fd) <= 1e-6 * abs(fd), (name, grads["f64"][i], fd)
     assert np.max(np.abs(grads["f32"] - grads["f64"]) / np.abs(grads["f64"])) < 1e-3, (grads["f32"], grads["f64"])
+
+
+def test_a_forward_run_that_does_not_fit_leaves_no_run_to_go_back():
+    # 10^18 steps: the checkpoints (terabytes) are refused by the allocator.  The run before
+    # is gone with its arrays, and backward says so instead of reading them
+    P = pss()
+    shape = (32, 32)
+    s = _gpu_system(shape, "f32", 0.02, 3)
+    lam = np.ones(s.half_shape, dtype=s.cdtype)
+    s.adjoint_forward(10)
+    with pytest.raises(P.PssError) as ei:
+        s.adjoint_forward(10 ** 18)
+    assert ei.value.code == P.PSS_ENOMEM
+    with pytest.raises(P.PssError) as ei:
+        s.adjoint_backward(lam, 4)
+    assert ei.value.code == P.PSS_EINVAL
+    s.set_step(0)
+    s.init_uniform(0, -0.3, 0.3)
+    s.adjoint_forward(10)
+    g, l0 = s.adjoint_backward(lam, 4)
+    t = _gpu_system(shape, "f32", 0.02, 3)
+    t.adjoint_forward(10)
+    gt, lt = t.adjoint_backward(lam, 4)
+    # (FP64 sums of the gradients by atomics: their order may differ)
+    np.testing.assert_allclose(g, gt, rtol=1e-9)
+    np.testing.assert_array_equal(l0, lt)
