@@ -2456,7 +2456,7 @@ int pss_add_term(pss_system *s, int field_id, int implicit, int n_mono, const in
     }
     s->stale = true;
     s->fps_dirty = true;
-    if (any_general(s)) invalidate(s);   // the fused terms are launch arguments
+    if (!implicit || any_general(s)) invalidate(s);   // the explicit terms of 1D runs and the fused ones are launch arguments
     return PSS_OK;
 }
 

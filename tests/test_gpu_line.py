@@ -193,3 +193,24 @@ def test_frame_adds_no_error_of_whole_transforms(n):
         got = np.fft.irfft(s.get_spectrum(f).astype(np.clongdouble), n)
         err += float(((got - r) ** 2).sum() / (r * r).sum()) / 16
     assert err <= 1e-15 ** 2, err ** 0.5
+
+
+def test_an_explicit_term_added_after_a_captured_run():
+    # a list with a system twice is captured, with the 1D run's explicit term among its
+    # launch arguments: a term that is added later has to reach the next call
+    P = pss()
+
+    def make():
+        s = P.System((64,), dt=0.01, seed=9, precision="f64")
+        f = s.add_field("a")
+        s.add_term(f, True, [(-1, 0.5, 1)], [(f, 1)])
+        s.init_uniform(f, -0.5, 0.5)
+        return s
+    a, b = make(), make()
+    P.step_many([a, a], 2)
+    b.step(4)
+    for s in (a, b):
+        s.add_term(0, False, [(-1, -1.0, 0)], [(0, 3)])
+    P.step_many([a, a], 2)
+    b.step(4)
+    np.testing.assert_array_equal(a.get_spectrum(0), b.get_spectrum(0))
