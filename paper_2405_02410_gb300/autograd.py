@@ -42,8 +42,9 @@ class PSSRun(torch.autograd.Function):
             raise ValueError("h0 must be a CUDA tensor (the half spectrum stays on the device)")
         sys_ = system
         sys_.set_stream(torch.cuda.current_stream(h0.device))
-        for pid, value in zip(param_ids, params.detach().tolist()):   # one copy to the host
-            sys_.set_param(pid, value)
+        values = params.detach().cpu()   # one copy to the host
+        for i, pid in enumerate(param_ids):
+            sys_.set_param(pid, float(values[i]))
         sys_.set_step(step0)
         sys_.set_spectrum(0, h0.detach().to(_cdtype(sys_)).contiguous())
         sys_.adjoint_forward(int(nsteps))

@@ -453,3 +453,16 @@ def test_a_forward_run_that_does_not_fit_leaves_no_run_to_go_back():
     # (FP64 sums of the gradients by atomics: their order may differ)
     np.testing.assert_allclose(g, gt, rtol=1e-9)
     np.testing.assert_array_equal(l0, lt)
+
+
+def test_torch_autograd_function_wants_a_value_for_every_parameter():
+    import torch
+    from paper_2405_02410_gb300 import autograd as A
+    s = pss().model_b((32, 32), dt=0.02, seed=9, precision="f64", **PARAMS)
+    h0 = torch.zeros(s.half_shape, dtype=torch.complex128, device="cuda")
+    with pytest.raises(IndexError):
+        A.run(h0, torch.tensor([-1.0, 1.0], dtype=torch.float64, device="cuda"), s, [0, 1, 2], 4)
+    # a column of values counts as one value per row; values beyond the parameters are not used
+    with torch.no_grad():
+        A.run(h0, torch.tensor([[-0.5], [0.75], [9.0]], dtype=torch.float64, device="cuda"), s, [0, 1], 4)
+    assert [s.get_param(i) for i in range(4)] == [-0.5, 0.75, PARAMS["K"], PARAMS["D"]]
