@@ -80,8 +80,8 @@ def binned_structure_factor(h: torch.Tensor, shape, nbins: int = 64, dx: float =
     the bin of a mode is ceil(|q| nbins dx / pi) - 1.  Returns (S[nbins], counts[nbins])."""
     shape = tuple(shape)
     n = int(np.prod(shape))
-    # the bins on h's device, in FP64 (the same operations as on the host, each
-    # correctly rounded)
+    # the bins on h's device, in FP64, by correctly rounded operations (a division by a
+    # Python number would go through its reciprocal there: m is a tensor)
     s2, w = 0.0, None
     for axis, m in enumerate(shape):
         last = axis == len(shape) - 1
@@ -89,7 +89,7 @@ def binned_structure_factor(h: torch.Tensor, shape, nbins: int = 64, dx: float =
         k = (i if last else torch.where(i < (m + 1) // 2, i, i - m)).to(torch.float64)
         view = [1] * len(shape)
         view[axis] = -1
-        s2 = s2 + ((2.0 * nbins * k / m) ** 2).view(view)
+        s2 = s2 + ((2.0 * nbins * k / torch.full_like(k, m)) ** 2).view(view)
         if last:
             w = torch.where((i == 0) | ((2 * i == m) if m % 2 == 0 else (i < 0)), 1.0, 2.0).to(torch.float64).view(view)
     s = torch.sqrt(s2)

@@ -36,3 +36,23 @@ def test_matches_oracle(shape, dx, nbins, prec):
     # sums of at most 2^19 positive terms, each a few roundings
     np.testing.assert_allclose(S, S0, rtol=1e-11, atol=0)
     assert abs(L - L0) <= 1e-11 * max(abs(L0), 1e-300)
+
+
+@pytest.mark.parametrize("shape,nbins", [((640, 480), 64), ((640, 480), 16), ((100, 100), 49), ((63, 77), 49),
+                                         ((128, 64), 64), ((45,), 16), ((12, 20, 28), 32)])
+def test_torch_bins_of_any_shape(shape, nbins):
+    # a mode on a bin's edge belongs to the bin below: ceil(|q| nbins dx / pi) - 1 with every
+    # operation correctly rounded, as numpy's are; bin counts and sums of |phi|^2 = 1
+    import torch
+    from paper_2405_02410_gb300 import autograd as A
+    h = torch.ones(shape[:-1] + (shape[-1] // 2 + 1,), dtype=torch.complex128, device="cuda")
+    S, cnt = A.binned_structure_factor(h, shape, nbins)
+    ks = [np.rint(np.fft.fftfreq(m) * m) for m in shape[:-1]] + [np.arange(shape[-1] // 2 + 1)]
+    g = np.meshgrid(*ks, indexing="ij")
+    s2 = sum((2.0 * nbins * k / m) ** 2 for k, m in zip(g, shape))
+    s = np.sqrt(s2)
+    valid = (s2 > 0) & (s <= nbins)
+    w = np.where((g[-1] == 0) | (2 * g[-1] == shape[-1]), 1.0, 2.0) * valid
+    want = np.bincount(np.where(valid, np.ceil(s) - 1, 0).astype(int).reshape(-1), w.reshape(-1), minlength=nbins)
+    np.testing.assert_array_equal(cnt.cpu().numpy(), want)
+    np.testing.assert_allclose(S.cpu().numpy(), np.where(want > 0, 1.0 / np.prod(shape), 0.0), rtol=1e-12)
