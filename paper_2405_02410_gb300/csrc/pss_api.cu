@@ -2873,7 +2873,10 @@ int pss_set_tuning(pss_system *s, const char *key, int value) {
 // held at their best so far, and keeps the value whose timed run of steps is
 // fastest (by more than 1 %, so that timing noise does not move it).  The
 // lists hold only values the launch-shape tests run (the helpers above clamp
-// them to the kernels' thread limits).
+// them to the kernels' thread limits).  Knobs that do not act on the run are
+// reported as they stand and not tried: timing noise would set one now and
+// then, and a launch shape that is set turns the register passes off for
+// fields in and out.
 // ---------------------------------------------------------------------------
 namespace {
 
@@ -2908,6 +2911,14 @@ std::vector<TuneKnob> tune_space(const pss_system *s) {
     k.push_back({"pdl", &pss_system::tune_pdl, {0, 1}});
     k.push_back({"graph_steps", &pss_system::tune_graph_steps, {8, 16, 32}});
     return k;
+}
+
+// whether a knob acts on runs of steps with the settings of now: on the runs in
+// one launch on chip none does, on the persistent step its radix and the choice of
+// the path
+bool knob_acts(const pss_system *s, int pss_system::*field) {
+    if (persist2d(s)) return field == &pss_system::tune_persist || field == &pss_system::tune_col2_radix;
+    return !resident(s);
 }
 
 // Milliseconds per step: the fastest of `reps` timed runs of at least `n`
@@ -2946,6 +2957,7 @@ int autotune_search(pss_system *s, int64_t n, const std::vector<TuneKnob> &space
     if ((rc = tune_trial(s, n, reps, e0, e1, &best)) == PSS_OK) {
         ++*trials;
         for (const TuneKnob &k : space) {
+            if (!knob_acts(s, k.field)) continue;
             const int keep = s->*k.field;
             int arg = keep;
             for (int v : k.values) {

@@ -155,3 +155,20 @@ def test_autotune_rejects_bad_arguments():
     P.add_model_b_field(s, a=-1.0, b=1.0, K=1.0, D=0.01)
     with pytest.raises(P.PssError):
         s.autotune(steps_per_trial=0)
+
+
+@pytest.mark.parametrize("shape,prec,free", [((64, 64), "f32", set()), ((128, 512), "f32", set()), ((256,), "f32", set()),
+                                             ((1024,), "f64", set()), ((512, 512), "f32", {"persist", "col2_radix"})])
+def test_knobs_that_do_not_act_on_the_run_stay(shape, prec, free):
+    # runs in one launch (on chip; persistent) take none of the per-step kernels' launch
+    # shapes: none is tried (the start and the two final comparisons of two are timed; beside
+    # them persist 0 and col2_radix 8 and 16 of the persistent step), and
+    # none is left set, which would take fields in and out off their own kernels
+    s = pss().model_b(shape, dt=0.01, a=-1.0, b=1.0, K=1.0, D=0.01, seed=7, precision=prec)
+    s.init_uniform(0, -0.1, 0.1)
+    rep = s.autotune(steps_per_trial=16)
+    assert rep["path"] != 1                  # (the persistent step wins at 512^2: 6 us against 10)
+    assert rep["trials"] == 5 + (3 if free else 0)
+    for k, v in rep.items():
+        if k not in {"path", "trials", "skipped", "initial_ms", "tuned_ms", "persist"} | free:
+            assert v == (-1 if k == "pdl" else 0), k
