@@ -2134,22 +2134,24 @@ int forward_field(pss_system *s, int field_id, const void *real = nullptr) {
 }
 
 // The checkpoints and a segment's arrays, kept from one adjoint run to the next
-// and grown when a run needs more (cudaMalloc and cudaFree of all of them, and
+// where it needs at most what there is and at least a quarter of it, so that a short
+// run gives back what a long one took (cudaMalloc and cudaFree of all of them, and
 // capturing the segment again, were 0.5 ms of every run).  The segment's graph
 // holds the run's first step and segment length, and these buffers.
 int adj_alloc(pss_system *s, int64_t nck, int64_t K) {
     const size_t slot_bytes = csize(s) * s->field_elems;
     const bool noise = persist2d_ok(s);
-    const bool grow_seg = K > s->seg_cap || (noise && !s->seg_noise);
-    if (nck > s->ck_cap || grow_seg || s->adj_K != K || s->adj_step0 != s->step) s->adj_graph_valid = false;
-    if (nck > s->ck_cap) {
+    const bool new_ck = nck > s->ck_cap || nck < s->ck_cap / 4;
+    const bool new_seg = K > s->seg_cap || K < s->seg_cap / 4 || (noise && !s->seg_noise);
+    if (new_ck || new_seg || s->adj_K != K || s->adj_step0 != s->step) s->adj_graph_valid = false;
+    if (new_ck) {
         cudaFree(s->ck);
         s->ck = nullptr;
         s->ck_cap = 0;
         CK(cudaMalloc(&s->ck, slot_bytes * (size_t)(nck + 1)));
         s->ck_cap = nck;
     }
-    if (grow_seg) {
+    if (new_seg) {
         for (void **p : {&s->seg, &s->seg_prod, &s->seg_real, &s->seg_noise}) {
             cudaFree(*p);
             *p = nullptr;

@@ -466,3 +466,61 @@ def test_torch_autograd_function_wants_a_value_for_every_parameter():
     with torch.no_grad():
         A.run(h0, torch.tensor([[-0.5], [0.75], [9.0]], dtype=torch.float64, device="cuda"), s, [0, 1], 4)
     assert [s.get_param(i) for i in range(4)] == [-0.5, 0.75, PARAMS["K"], PARAMS["D"]]
+
+
+@pytest.mark.parametrize("shape,prec", [((32, 32), "f32"), ((256, 256), "f32"), ((32, 16), "f64"), ((8, 16, 8), "f32")])
+def test_runs_of_one_system_after_one_another(shape, prec):
+    # the checkpoints, a segment's arrays and its captured graph stay with the system: runs
+    # of other lengths, from other steps, after a change of tuning or of a parameter, and the
+    # same run again, each against a system of its own.  The operations are the same: dJ/dphi_0
+    # bit for bit, the parameter sums (FP64 atomics) to their order
+    s = _gpu_system(shape, prec, 0.02, 3)
+    h0 = s.get_spectrum(0)
+    lam = h0 / np.prod(shape)
+    last = None
+    for n, step0, knob, a in [(30, 0, None, -1.0), (30, 0, None, -1.0), (9, 0, None, -1.0), (30, 4, None, -1.0),
+                              (500, 0, None, -0.9), (30, 0, "persist_adj", -1.0), (30, 7, "fuse_adjoint", -0.8), (5, 1, None, -1.0)]:
+        t = _gpu_system(shape, prec, 0.02, 3)
+        if last and last != knob:
+            s.set_tuning(last, 1)
+        for q in (s, t):
+            if knob and (q is t or knob != last):
+                q.set_tuning(knob, 0)
+            q.set_param(0, a)
+            q.set_spectrum(0, h0)
+            q.set_step(step0)
+            q.adjoint_forward(n)
+        (gs, ls), (gt, lt) = s.adjoint_backward(lam, 4), t.adjoint_backward(lam, 4)
+        np.testing.assert_array_equal(ls, lt)
+        np.testing.assert_allclose(gs, gt, rtol=1e-9, err_msg=str((n, step0, knob, a)))
+        t.close()
+        last = knob
+
+
+def test_a_short_run_gives_back_what_a_long_one_took():
+    # 4000 steps at 256^2: 64 checkpoints and 64 steps of a segment, 85 MB; 16 steps: 5 MB
+    import torch
+    s = _gpu_system((256, 256), "f32", 0.02, 3)
+    s.adjoint_forward(4000)
+    s.sync()
+    before = torch.cuda.mem_get_info()[0]
+    s.adjoint_forward(16)
+    s.sync()
+    assert torch.cuda.mem_get_info()[0] - before >= 50e6
+
+
+@pytest.mark.parametrize("shape", [(1024, 64), (32, 1024)])
+def test_adjoint_beside_the_register_passes(shape):
+    # FP32 sides of 1024 with one below 256 step by k3_col and k3_row; the recomputed
+    # segments take k3_col with a state of its own to write.  Against the staged kernels:
+    # FP32 rounding of two transform orders through 20 steps and back, as for the other
+    # adjoint paths (1e-3)
+    out = []
+    for regs in (1, 0):
+        s = _gpu_system(shape, "f32", 0.02, 3)
+        s.set_tuning("regs", regs)
+        lam = s.get_spectrum(0) / np.prod(shape)
+        s.adjoint_forward(20)
+        out.append(s.adjoint_backward(lam, 4))
+    np.testing.assert_allclose(out[0][0], out[1][0], rtol=1e-3)
+    assert rel(out[0][1], out[1][1]) < 1e-3
