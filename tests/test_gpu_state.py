@@ -129,3 +129,42 @@ def test_load_rejects_another_system_and_leaves_it_unchanged():
     c = _model_b((64, 64), prec="f64")
     with pytest.raises(pss.PssError):
         c.load_state(blob)                                      # other precision
+
+
+@pytest.mark.parametrize("shape,prec", [((64, 64), "f32"), ((8, 512), "f32"), ((16, 8, 32), "f32"), ((64,), "f32"),
+                                        ((32, 64), "f64"), ((4,), "f32"), ((4, 8, 4), "f64")])
+@pytest.mark.parametrize("offset", [0, 1, 3])
+def test_device_buffers_at_any_address(shape, prec, offset):
+    # fields and spectra go in and out where they are in device memory: from an address of any
+    # alignment (an element, not a vector) the same bits as through host memory, and not a
+    # value beside the buffer is touched
+    import torch
+    pss = P()
+    n = int(np.prod(shape))
+    rng = np.random.default_rng(n + offset)
+    x = rng.uniform(-1.0, 1.0, shape)
+    host, dev = (pss.model_b(shape, dt=0.01, seed=2, precision=prec) for _ in range(2))
+    x = x.astype(host.rdtype)
+    host.set_field(0, x)
+    buf = torch.full((n + 8,), 7.0, dtype=torch.float64 if prec == "f64" else torch.float32, device="cuda")
+    buf[offset:offset + n] = torch.from_numpy(x.reshape(-1)).cuda()
+    torch.cuda.synchronize()
+    dev.set_field(0, buf[offset:offset + n].view(shape))
+    want = host.get_spectrum(0)
+    np.testing.assert_array_equal(dev.get_spectrum(0), want)
+    out = torch.full_like(buf, 5.0)
+    torch.cuda.synchronize()
+    dev.get_field(0, out=out[offset:offset + n].view(shape))
+    o = out.cpu().numpy()
+    np.testing.assert_array_equal(o[offset:offset + n].reshape(shape), host.get_field(0))
+    assert (o[:offset] == 5.0).all() and (o[offset + n:] == 5.0).all()
+    m = want.size
+    hb = torch.full((m + 8,), 3.0, dtype=torch.complex128 if prec == "f64" else torch.complex64, device="cuda")
+    torch.cuda.synchronize()
+    dev.get_spectrum(0, out=hb[offset:offset + m].view(want.shape))
+    h = hb.cpu().numpy()
+    np.testing.assert_array_equal(h[offset:offset + m].reshape(want.shape), want)
+    assert (h[:offset] == 3.0).all() and (h[offset + m:] == 3.0).all()
+    other = pss.model_b(shape, dt=0.01, seed=2, precision=prec)
+    other.set_spectrum(0, hb[offset:offset + m].view(want.shape))
+    np.testing.assert_array_equal(other.get_spectrum(0), want)
