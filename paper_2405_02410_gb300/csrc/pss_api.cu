@@ -1953,6 +1953,18 @@ int ensure_half(pss_system *s) {
     return PSS_OK;
 }
 
+// Whether kernels may use the caller's buffer where it is: memory of the system's
+// device (or managed), `align` bytes aligned.  Everything else that a copy takes, of
+// another device or of the host, goes through the scratch by a copy that looks at
+// both addresses (user_copy).
+bool in_place(const pss_system *s, const void *p, int where, size_t align) {
+    if (where == PSS_HOST || (uintptr_t)p % align != 0) return false;
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) { cudaGetLastError(); return false; }
+    return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == s->device);
+}
+cudaMemcpyKind user_copy(int where, cudaMemcpyKind host) { return where == PSS_HOST ? host : cudaMemcpyDefault; }
+
 int report_status(pss_system *s, int st);
 
 int device_errors(pss_system *s) {
@@ -2562,11 +2574,10 @@ int pss_set_field(pss_system *s, int field_id, const void *real, int where) {
     if (!real) return fail(s, PSS_EINVAL, "real is NULL");
     // the row kernel reads a device field where it is (its bulk copies want 16-byte
     // alignment); host fields and others go through the scratch
-    if (where != PSS_HOST && (uintptr_t)real % 16 == 0) return forward_field(s, field_id, real);
+    if (in_place(s, real, where, 16)) return forward_field(s, field_id, real);
     if ((rc = ensure_real(s))) return rc;
     const size_t bytes = rsize(s) * (size_t)s->nsites;
-    CK(cudaMemcpyAsync(s->real, real, bytes, where == PSS_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice,
-                       s->stream));
+    CK(cudaMemcpyAsync(s->real, real, bytes, user_copy(where, cudaMemcpyHostToDevice), s->stream));
     return forward_field(s, field_id);
 }
 
@@ -3088,7 +3099,7 @@ int pss_get_field(pss_system *s, int field_id, void *real_out, int where) {
     if (rc) return rc;
     if (!real_out) return fail(s, PSS_EINVAL, "real_out is NULL");
     // the row kernel writes a device field where it is wanted
-    const bool direct = where != PSS_HOST && (uintptr_t)real_out % rsize(s) == 0;
+    const bool direct = in_place(s, real_out, where, rsize(s));
     if (!direct && (rc = ensure_real(s))) return rc;
     if ((rc = upload_params(s))) return rc;
     const int slot = cur_slot(s, field_id);
@@ -3098,8 +3109,7 @@ int pss_get_field(pss_system *s, int field_id, void *real_out, int where) {
     if (s->dim == 3) s->stale = true;   // the y pass reused B
     const size_t bytes = rsize(s) * (size_t)s->nsites;
     if (!direct)
-        CK(cudaMemcpyAsync(real_out, s->real, bytes, where == PSS_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice,
-                           s->stream));
+        CK(cudaMemcpyAsync(real_out, s->real, bytes, user_copy(where, cudaMemcpyDeviceToHost), s->stream));
     return device_errors(s);
 }
 
@@ -3107,7 +3117,7 @@ int pss_get_spectrum(pss_system *s, int field_id, void *half_out, int where) {
     int rc = check_field(s, field_id);
     if (rc) return rc;
     if (!half_out) return fail(s, PSS_EINVAL, "half_out is NULL");
-    const bool direct = where != PSS_HOST && (uintptr_t)half_out % csize(s) == 0;
+    const bool direct = in_place(s, half_out, where, csize(s));
     if (!direct && (rc = ensure_half(s))) return rc;
     void *dst = direct ? half_out : s->half;
     const size_t ofs = csize(s) * s->field_elems * (size_t)cur_slot(s, field_id);
@@ -3120,8 +3130,7 @@ int pss_get_spectrum(pss_system *s, int field_id, void *half_out, int where) {
     if (e != cudaSuccess) return cuda_fail(s, e, "layout kernel");
     const size_t bytes = csize(s) * (size_t)s->hx * s->ny * s->nz;
     if (!direct)
-        CK(cudaMemcpyAsync(half_out, s->half, bytes, where == PSS_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice,
-                           s->stream));
+        CK(cudaMemcpyAsync(half_out, s->half, bytes, user_copy(where, cudaMemcpyDeviceToHost), s->stream));
     return device_errors(s);
 }
 
@@ -3131,10 +3140,9 @@ int pss_set_spectrum(pss_system *s, int field_id, const void *half_in, int where
     if (!half_in) return fail(s, PSS_EINVAL, "half_in is NULL");
     const size_t bytes = csize(s) * (size_t)s->hx * s->ny * s->nz;
     const void *src = half_in;
-    if (where == PSS_HOST || (uintptr_t)half_in % csize(s) != 0) {
+    if (!in_place(s, half_in, where, csize(s))) {
         if ((rc = ensure_half(s))) return rc;
-        CK(cudaMemcpyAsync(s->half, half_in, bytes, where == PSS_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice,
-                           s->stream));
+        CK(cudaMemcpyAsync(s->half, half_in, bytes, user_copy(where, cudaMemcpyHostToDevice), s->stream));
         src = s->half;
     }
     const size_t ofs = csize(s) * s->field_elems * (size_t)cur_slot(s, field_id);

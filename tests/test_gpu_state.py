@@ -168,3 +168,29 @@ def test_device_buffers_at_any_address(shape, prec, offset):
     other = pss.model_b(shape, dt=0.01, seed=2, precision=prec)
     other.set_spectrum(0, hb[offset:offset + m].view(want.shape))
     np.testing.assert_array_equal(other.get_spectrum(0), want)
+
+
+@pytest.mark.parametrize("shape,prec", [((64, 64), "f32"), ((16, 8, 32), "f64"), ((64,), "f32")])
+def test_buffers_that_are_not_the_devices_own_are_copied(shape, prec):
+    # a pointer passed as device memory that is pinned memory of the host: no kernel works on
+    # it, the copies find its place
+    import ctypes
+    import torch
+    pss = P()
+    x = np.random.default_rng(3).uniform(-1.0, 1.0, shape)
+    host, dev = (pss.model_b(shape, dt=0.01, seed=2, precision=prec) for _ in range(2))
+    x = x.astype(host.rdtype)
+    host.set_field(0, x)
+    pin = torch.from_numpy(x.copy()).pin_memory()
+    out = torch.zeros_like(pin).pin_memory()
+    h = torch.zeros(host.half_shape, dtype=torch.complex128 if prec == "f64" else torch.complex64).pin_memory()
+    ptr = lambda t: ctypes.c_void_p(t.data_ptr())
+    assert pss.lib.pss_set_field(dev._h, 0, ptr(pin), pss.PSS_DEVICE) == pss.PSS_OK
+    np.testing.assert_array_equal(dev.get_spectrum(0), host.get_spectrum(0))
+    assert pss.lib.pss_get_field(dev._h, 0, ptr(out), pss.PSS_DEVICE) == pss.PSS_OK
+    np.testing.assert_array_equal(out.numpy(), host.get_field(0))
+    assert pss.lib.pss_get_spectrum(dev._h, 0, ptr(h), pss.PSS_DEVICE) == pss.PSS_OK
+    np.testing.assert_array_equal(h.numpy(), host.get_spectrum(0))
+    other = pss.model_b(shape, dt=0.01, seed=2, precision=prec)
+    assert pss.lib.pss_set_spectrum(other._h, 0, ptr(h), pss.PSS_DEVICE) == pss.PSS_OK
+    np.testing.assert_array_equal(other.get_spectrum(0), host.get_spectrum(0))
