@@ -140,9 +140,9 @@ struct pss_system {
     int tune_fast3d = 1;                     // FP32 3D x pass with one FFT group per row pair (0 = generic k_row)
     int tune_test_timeout = 0;               // check of the bounded waits: one CTA's wait runs out (tests)
     int tune_persist = 1;                    // square FP32 2D systems: a run of steps as one persistent launch
-    int tune_adj_col2 = 1;
+    int tune_adj_col2 = 1;                   // FP32 2D adjoint: column parts on FFT groups (0: generic kernel)
     int tune_adj_radix = 0;                  // FFT radix of that backward pass (8 or 16; 0: the forward's)
-    int tune_persist_adj = 1;                // FP32 2D adjoint on the persistent path: a segment's backward pass in one launch                   // FP32 2D adjoint: column parts on FFT groups (0: generic kernel)
+    int tune_persist_adj = 1;                // FP32 2D adjoint on the persistent path: a segment's backward pass in one launch
     int tune_fuse_terms = 1;                 // FP32 1D/2D product terms in one row kernel (0: factor by factor)
     int tune_regs = 1;                       // FP32 2D and 3D: passes with their points in registers (0: staged kernels; 2: all 2D systems they take)
     int tune_resident = 1;                   // FP32 2D sides of 32..512: a run of steps with every slot in one cluster
@@ -580,7 +580,7 @@ bool fast2d_shape(const pss_system *s) {
 // 32 of them per thread, so a launch lasts about 10 us however small.  us per
 // step, the FFT-group kernels (or cluster-resident run) -> here: 512^2 x 8 24.0
 // -> 24.8, x 12 34.3 -> 28.2, x 32 85 -> 62; 512 x 256 x 16 23.2 -> 22.2, x 32
-// 40 -> 32; 256^2 x 32 17.8 -> 17.4, x 64 35 -> 26, x 128 70 -> 48; with a side
+// 40 -> 32; 256^2 x 32 17.6 -> 18.4, x 64 35 -> 26, x 128 70 -> 48; with a side
 // of 1024 from fewer sites on: 1024 x 512 x 2 20 -> 24, x 3 30 -> 24, 1024^2 x 2
 // 29.5 -> 25.5, x 8 107 -> 67.  A side of 1024 with one below 256 always (against
 // the generic kernels; nx x ny: 1024 x 64 12.5 -> 8.8, 1024 x 128 12.7 -> 11.8, 64 x
@@ -674,15 +674,20 @@ int res_active(const pss_system *s, int C) {
     if (launch_res2(a, s->nslots(), nullptr, &active) != cudaSuccess) { cudaGetLastError(); active = 0; }
     return active;
 }
-// Where it is the faster path, measured on GB300 (us per step, other path ->
-// cluster-resident; batch x shape): with a side below 256 always (generic
-// kernels: 32^2 9.6 -> 2.7, 64^2 10.4 -> 3.2, 128^2 11.6 -> 4.2, 64^2 x 128
-// 13.7 -> 4.7, 128^2 x 128 27.3 -> 13.1, 128 x 512 12.4 -> 7.3, two fields of
-// 512 x 128 12.6 -> 8.4).  With both sides of 256 or more the two-kernel step
-// spreads one slot over the whole chip: 256^2 x 8 8.8 -> 10.1, x 32 20.7 ->
-// 17.6, x 128 73 -> 68, 512 x 256 8.2 -> 12.2, 512^2 x 32 85 -> 100; only
-// 256^2 gains, when its clusters of four fill most of the chip (36 at a time) and
-// there are too few sites for the register passes.
+// Where it is taken, measured on GB300 (us per step, other path ->
+// cluster-resident): with a side below 256, against the generic kernels (ny x nx:
+// 32^2 9.6 -> 2.7, 64^2 10.4 -> 3.2, 128^2 11.6 -> 4.2, 64^2 x 128 instances 13.7 ->
+// 4.7, 128^2 x 128 27.3 -> 13.1, 128 x 512 12.4 -> 7.3, two fields of 512 x 128 12.6 ->
+// 8.4; 128 x 512 x 64 51 -> 32, 512 x 128 x 128 112 -> 70, 128 x 256 x 128 48 -> 29).
+// Large batches of rectangles would be faster still on the register passes
+// (tuning key "regs" 2 and "resident" 0: those three 27, 55 and 26; 64 x 512 x 128 29
+// -> 26), smaller ones and squares not (128 x 512 x 32 16.3 against 17.7, 64 x 512 x 64
+// 14.7 against 17.4, 128^2 x 256 25.9 against 26.9).  With both sides of 256 or more
+// the two-kernel step spreads one slot over the whole chip: 256^2 x 8 8.8 -> 10.1,
+// x 128 73 -> 68, 512 x 256 8.2 -> 12.2, 512^2 x 32 85 -> 100; only 256^2 gains, when
+// its clusters of four fill most of the chip (36 at a time) and there are no more
+// sites than regs2d_step leaves: x 29 20.1 -> 17.6, x 32 20.7 -> 17.6 (the register
+// passes 18.4).
 constexpr int kRes256Fill = 29;   // slots per wave of 256^2 clusters from which it gains
 bool resident2d(const pss_system *s) {
     if (!(s->tune_resident && s->tune_fast2d && s->prec == PSS_F32 && s->dim == 2 && side_res(s->nx) &&

@@ -98,15 +98,14 @@ template <typename T> __device__ __forceinline__ T uniform24(uint32_t x) {
     return (T(x >> 8) + T(0.5)) * T(5.9604644775390625e-08);
 }
 
-// square root and reciprocal: FP32 through the hardware approximations
-// (about 2 ulp), FP64 correctly rounded
-__device__ __forceinline__ float fast_sqrt(float x) { return x > 0.0f ? x * rsqrtf(x) : 0.0f; }
-__device__ __forceinline__ double fast_sqrt(double x) { return sqrt(x); }
+// reciprocal: FP32 through the hardware approximation (about 2 ulp), FP64 correctly
+// rounded
 __device__ __forceinline__ float fast_rcp(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ double fast_rcp(double x) { return 1.0 / x; }
 
-// sqrt as x rsqrt(x) by the hardware approximation (about 2 ulp; 0 stays 0,
-// subnormals count as 0), without a branch or a select
+// sqrt of x >= 0 as x rsqrt(x) by the hardware approximation (about 2 ulp), without a
+// branch or a select: the root's argument is at least 2^-126, so 0 stays 0 and a
+// subnormal x gives x times 2^63, below its root
 __device__ __forceinline__ float root_approx(float x) {
     float r;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fmaxf(x, 1.17549435e-38f)));

@@ -281,9 +281,6 @@ struct P2AdjArgs {
 cudaError_t launch_p2_adj(const P2AdjArgs &a, int n, int E, int nblocks, cudaStream_t st);
 // The cluster-resident FP32 2D step (k_res2d: sides of 32..512 points): one
 // cluster of C CTAs per slot runs nsteps steps.
-#ifndef PSS_RES_E8
-#define PSS_RES_E8 128
-#endif
 constexpr int kResMaxThreads = 576;    // transform threads of a CTA
 constexpr int kResNoiseWarps = 4;      // and the warps that draw the noise
 struct Res2Args {
@@ -351,7 +348,9 @@ template <typename T> cudaError_t launch_line(const LineArgs<T> &a, int nslots, 
 
 // Values per thread of k_res2d's transforms of n points, the points of shared
 // memory one takes, and a CTA's dynamic shared memory (C CTAs per cluster)
-__host__ __device__ constexpr int res_e(int n) { return n <= PSS_RES_E8 ? 8 : 16; }
+// (8 values up to 128 points: more threads shorten a phase's chain, 128^2 7.0 -> 4.8 us
+// per step; at 256 the second pass would then be 32 points, four lanes' work)
+__host__ __device__ constexpr int res_e(int n) { return n <= 128 ? 8 : 16; }
 __host__ __device__ constexpr int res_xld(int n) { return n + res_e(n) + 2; }
 __host__ __device__ constexpr size_t res2_smem_bytes(int nx, int ny, int C) {
     const size_t cols = 2 * (size_t)(((nx / 2 + 2) / 2 + C - 1) / C), pairs = (size_t)(ny / 2 / C);

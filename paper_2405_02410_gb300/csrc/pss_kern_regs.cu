@@ -1,4 +1,4 @@
-// pss_kern_regs3d.cu -- the register passes of FP32 2D and 3D systems.
+// pss_kern_regs.cu -- the register passes of FP32 2D and 3D systems.
 #include <type_traits>
 
 #include "pss_regs.cuh"
