@@ -91,15 +91,16 @@ __global__ void __launch_bounds__(LineShape<T, N>::NT) k_line(const LineArgs<T> 
         // i (w.x - i w.y) d = (w.y + i w.x) d
         return mk<T>(s.x + (w.y * d.x - w.x * d.y), s.y + (w.y * d.y + w.x * d.x));
     };
-    // Mode k of the half spectrum from the half-length forward transform Z:
-    // ((Z_k + conj Z_{M-k}) - i exp(-2 pi i k / N) (Z_k - conj Z_{M-k})) / 2
-    auto untangle = [&](const C *Z, int k) {
+    // Twice mode k of the half spectrum from the half-length forward transform Z:
+    // (Z_k + conj Z_{M-k}) - i exp(-2 pi i k / N) (Z_k - conj Z_{M-k})
+    auto untangle2 = [&](const C *Z, int k) {
         const int p = k & (M - 1), r = (M - k) & (M - 1);
         const C x = Z[S::WIDE ? p : spad(p)], y = Z[S::WIDE ? r : spad(r)], w = WN[k];
         const C s = mk<T>(x.x + y.x, x.y - y.y), d = mk<T>(x.x - y.x, x.y + y.y);
         // -i (w.x + i w.y) d = (w.y - i w.x) d
-        return mk<T>(T(0.5) * (s.x + (w.y * d.x + w.x * d.y)), T(0.5) * (s.y + (w.y * d.y - w.x * d.x)));
+        return mk<T>(s.x + (w.y * d.x + w.x * d.y), s.y + (w.y * d.y - w.x * d.x));
     };
+    auto untangle = [&](const C *Z, int k) { return cscale<T>(untangle2(Z, k), T(0.5)); };
     // the real rows of the inverse transform, two sites per complex value, go
     // through `site(n, x)` and forward again; returns the buffer of the result
     auto there_and_back = [&](auto src, auto site) {
@@ -217,8 +218,15 @@ __global__ void __launch_bounds__(LineShape<T, N>::NT) k_line(const LineArgs<T> 
                 return v;
             };
             const C *Z = there_and_back([&](int k) { return tangle(full(k), full(M - k), k); },
-                                        [&](int x, T v) { return x < fl.frame_w ? fl.frame_lo - v : x >= N - fl.frame_w ? fl.frame_hi - v : T(0); });
-            for (int k = t; k <= M; k += S::NT) PHI[k] = cadd<T>(PHI[k], untangle(Z, k));
+                                        [&](int x, T v) {
+                                            const bool lo = x < fl.frame_w;
+                                            const T b = lo ? fl.frame_lo : fl.frame_hi;
+                                            return lo || x >= N - fl.frame_w ? b - v : T(0);
+                                        });
+            for (int k = t; k <= M; k += S::NT) {
+                const C d = untangle2(Z, k), h = PHI[k];
+                PHI[k] = mk<T>(ffma(T(0.5), d.x, h.x), ffma(T(0.5), d.y, h.y));
+            }
             __syncthreads();
         }
         if (has_product && n + 1 < a.nsteps) P = product();
