@@ -756,7 +756,7 @@ int res_ctas(pss_system *s) {
 // the side has their shape and no launch shape of the staged kernels is asked
 // for.  3D: faster at every size measured (us per step, staged -> registers: 32^3
 // 20.4 -> 7.8, 64^3 pair 22.0 -> 10.7, 256 x 256 x 64 54 -> 34, 16 z x 128 x 64 22.1
-// -> 8.9, 256^3 pair 351 -> 237).  2D: the step by regs2d_step, and
+// -> 8.9, 256^3 pair 351 -> 238).  2D: the step by regs2d_step, and
 // fields in and out along axes of up to 256 points (set_field: 256^2 12.4 -> 8.5,
 // 64^3 22.8 -> 12.5, 256^3 120 -> 80; above, a KPZ run at 512^2 with its field's
 // way in and out lost 10 us).  Product terms evaluated

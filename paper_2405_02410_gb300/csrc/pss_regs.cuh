@@ -13,7 +13,7 @@
 // noise is drawn into shared memory while the loads are in flight, a pair of
 // columns per Philox call.  us, staged -> here: 256^3, two fields: z pass 153
 // -> 104 (466 MB: 4.5 TB/s), y inverse 52 -> 37, y forward 63 -> 52 (270 MB:
-// 5.2 TB/s), x pass 104 -> 66 (225 MB: 3.4 TB/s), the step 351 -> 237; whole
+// 5.2 TB/s), x pass 104 -> 66 (225 MB: 3.4 TB/s), the step 351 -> 238; whole
 // steps of 128^3 (two fields) 58 -> 35, 256 x 256 x 64 54 -> 34, 64^3 (two fields)
 // 22.0 -> 10.7, 32^3 20.4 -> 7.8; 2D batches against the FFT-group kernels: 512^2 x 32
 // 85 -> 62, 1024^2 x 8 107 -> 67.  The step's column pass takes 5 CTAs per SM and
